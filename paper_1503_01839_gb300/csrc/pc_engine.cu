@@ -163,6 +163,7 @@ static int read_slots(pc_ctx* ctx, int n, i128* out)
     ctx->stats.easy_runs += c[1];
     ctx->stats.easy_run_leaves += c[2];
     ctx->stats.p2_clears += c[3];
+    ctx->stats.hard_leaves += c[4];   // those read from the pi table
     float ms = 0;
     if (ctx->easy_timed && cudaEventElapsedTime(&ms, ctx->ev[2], ctx->ev[3]) == cudaSuccess) ctx->stats.ms_easy_kernel += ms;
     if (ctx->p2_timed && cudaEventElapsedTime(&ms, ctx->ev[4], ctx->ev[5]) == cudaSuccess) ctx->stats.ms_p2_kernel += ms;
@@ -232,7 +233,9 @@ static u32 choose_seg(const pc_ctx* ctx, u64 x)
 
 // Leaf decomposition of phi(x, a) and P2(x, a); a == 0 selects pi(y).
 // parts: S1, trivial, easy, hard, P2 (P2 only when want_p2).
-static int leaf_parts(pc_ctx* ctx, u64 x, u64 y, u32 c, u64 a, bool want_p2, i128 parts[5], u64* a_out)
+// total_only: the caller wants the sum of the leaves, not how it splits into easy and hard.
+static int leaf_parts(pc_ctx* ctx, u64 x, u64 y, u32 c, u64 a, bool want_p2, bool total_only, i128 parts[5],
+                      u64* a_out)
 {
     if (y < 1 || y > pc_isqrt(x) || c > 7) {
         pc_set_error(ctx, "leaf sums need 1 <= y <= isqrt(x) and c <= 7");
@@ -242,8 +245,8 @@ static int leaf_parts(pc_ctx* ctx, u64 x, u64 y, u32 c, u64 a, bool want_p2, i12
     const u64 z = x / y;
     const u64 r = pc_isqrt(x);
     PC_TRY(tables_ensure(ctx, r > y ? r : y, pc_max(y, pc_isqrt(z)), y, c));
-    u64 vals[2] = {y, pc_isqrt(z)}, pv[2];
-    PC_TRY(tables_pi_values(ctx, vals, pv, 2));
+    u64 vals[3] = {y, pc_isqrt(z), pc_isqrt(r)}, pv[3];
+    PC_TRY(tables_pi_values(ctx, vals, pv, 3));
     const u64 piy = pv[0], B = pv[1];
     if (a == 0) a = piy;
     if (a > piy || c > a) {
@@ -252,7 +255,8 @@ static int leaf_parts(pc_ctx* ctx, u64 x, u64 y, u32 c, u64 a, bool want_p2, i12
         return PC_EINVAL;
     }
     PC_TRY(sync_timed(ctx, &ctx->stats.ms_tables, t));
-    LeafProblem P{x, y, z, c, a, a < piy, piy, B};
+    LeafProblem P{x, y, z, c, a, a < piy, piy, B, pv[2]};
+    P.table_in_easy = total_only;
     ctx->stats.y = y;
     ctx->stats.z = z;
     ctx->stats.a = a;
@@ -288,7 +292,7 @@ extern "C" int pc_leaf_sums(pc_ctx* ctx, uint64_t x, uint64_t y, uint32_t c, uin
     stats_begin(ctx, x);
     Timer t;
     i128 parts[5];
-    PC_TRY(leaf_parts(ctx, x, y, c, a, true, parts, nullptr));
+    PC_TRY(leaf_parts(ctx, x, y, c, a, true, false, parts, nullptr));
     for (int i = 0; i < 5; i++) out[i] = to_pc(parts[i]);
     ctx->stats.ms_total = t.ms();
     return PC_OK;
@@ -322,15 +326,15 @@ static int s2_hard_impl(pc_ctx* ctx, uint64_t x, uint64_t y, uint32_t c, u32 sha
     const u64 z = x / y;
     const u64 r = pc_isqrt(x);
     PC_TRY(tables_ensure(ctx, r > y ? r : y, pc_max(y, pc_isqrt(z)), y, c));
-    u64 vals[2] = {y, pc_isqrt(z)}, pv[2];
-    PC_TRY(tables_pi_values(ctx, vals, pv, 2));
+    u64 vals[3] = {y, pc_isqrt(z), pc_isqrt(r)}, pv[3];
+    PC_TRY(tables_pi_values(ctx, vals, pv, 3));
     const u64 piy = pv[0], B = pv[1];
     if (c > piy) {
         pc_set_error(ctx, "c=%u exceeds pi(y)=%llu", c, (unsigned long long)piy);
         return PC_EINVAL;
     }
     PC_TRY(sync_timed(ctx, &ctx->stats.ms_tables, ph));
-    LeafProblem P{x, y, z, c, piy, false, piy, B};
+    LeafProblem P{x, y, z, c, piy, false, piy, B, pv[2]};
     P.shard_k = shard_k;
     P.shard_n = shard_n;
     ctx->stats.y = y;
@@ -408,7 +412,7 @@ int pi_count_impl(pc_ctx* ctx, u64 x, u32 alpha, u64* out)
     }
     i128 parts[5];
     u64 a = 0;
-    const int rc = leaf_parts(ctx, x, y, c, 0, true, parts, &a);
+    const int rc = leaf_parts(ctx, x, y, c, 0, true, true, parts, &a);
     ctx->seg_call = 0;
     ctx->ctas_call = 0;
     if (rc != PC_OK) return rc;
@@ -466,7 +470,7 @@ int phi_impl(pc_ctx* ctx, u64 x, u64 a, u64* out_phi)
     if (y > r) y = r;
     u32 c = a < 5 ? (u32)a : 5;
     i128 parts[5];
-    PC_TRY(leaf_parts(ctx, x, y, c, a, false, parts, nullptr));
+    PC_TRY(leaf_parts(ctx, x, y, c, a, false, true, parts, nullptr));
     i128 phi = parts[0] + parts[1] + parts[2] + parts[3];
     if (phi < 0 || (phi >> 64) != 0) return PC_EOVERFLOW;
     *out_phi = (u64)phi;

@@ -25,7 +25,12 @@
 // blocks in Section 3 becomes one scan.
 //
 // A hard leaf (b, m) has u < x / p_b^2, so a segment starting at L only
-// needs the primes p_b <= isqrt(x / L): B_s = pi(isqrt(x/L)).
+// needs the primes p_b <= isqrt(x / L).  The hard leaves with u < p_b^2 are read
+// from the pi table (easy_range in pc_leaves.cu), so it needs only those with
+// p_b^2 <= L + span - 1 as well: B_s = pi(min(isqrt(x/L), isqrt(L + span - 1))),
+// at most pi(x^(1/4)).  The segments with B_s >= b are thus consecutive,
+// s >= p_b^2 / span; there the carry of b starts from phi(v, b-1) =
+// pi(v) - b + 2, v = L - 1 < p_b^2, again from the pi table.
 //
 // Load balance: hard leaves crowd near u = y (their density falls like
 // 1/u^2), so one segment can hold a large share of them.  A pre-pass counts
@@ -90,10 +95,10 @@ struct HardArgs {
     u32 nsl;
     const u32* primes;
     const u64* primes_rcp;
-    u64 rcp_y;          // floor((2^64 - 1) / y)
     const u32* segB;
     const u64* rcp_seg;   // per segment: reciprocals of L_s and L_s + span (0 for L = 0)
     const u64* off;
+    const u32* rlo;     // first segment of row b (index b - k0): entry s of the row is off + s - rlo
     const u64* start;   // phi(L_{s0} - 1, b) for b = k0 .. bmax (index b - k0), or null for s0 = 0
     u32* counts;
     i32* tallies;
@@ -117,19 +122,18 @@ struct __align__(16) StepInfo {
                    // bit 5: p >= GROUP_P and p^3 > the last integer of the segment (see group_cross),
                    // bit 6: bit 5 and p >= the sub-range's bytes >> RUN_SHIFT (see sparse_runs)
     u32 pself;     // segment bit of p_b itself, or ~0
-    u32 row;       // off[b - k0]: start of the count / tally rows of b
+    u32 row;       // off - rlo of b, mod 2^32: the count / tally rows' entry of segment s is row + s
     u32 runcap;    // bit 6: bound of the step's log entries, 8 ceil(sub_bytes / p) + 1
     u32 pad[2];
 };
 
-// leaf range of prime b in the segment [L, L + span): m in (mlo, mhi].
+// leaf range of prime b in the segment [L, L + span): m in (mlo, mhi], u >= p_b^2.
 // vp, vL, vLs: reciprocals of p, L (0 when L = 0) and L + span.
 __device__ __forceinline__ bool leaf_window(const HardArgs& A, u64 p, u64 vp, u64 xp, u64 L, u64 vL, u64 vLs,
                                             u64& mlo, u64& mhi)
 {
-    // hard: u >= min(p^2, y); xp / p^2 = floor(floor(xp / p) / p)
-    const u64 xT = p * p <= A.y ? div_rcp(div_rcp(xp, p, vp), p, vp) : div_rcp(xp, A.y, A.rcp_y);
-    mhi = pc_min(A.y, xT);
+    // u >= p^2; xp / p^2 = floor(floor(xp / p) / p)
+    mhi = pc_min(A.y, div_rcp(div_rcp(xp, p, vp), p, vp));
     if (L) mhi = pc_min(mhi, div_rcp(xp, L, vL));                        // u >= L
     mlo = pc_max(div_rcp(A.y, p, vp), div_rcp(xp, L + A.span, vLs));     // u < L + span, m > y / p
     return mhi > mlo;
@@ -331,7 +335,7 @@ __global__ void __launch_bounds__(MAXT, MINB) hard_sieve_kernel(HardArgs A0, Mul
                 si.xp = div_rcp(A.x, p, vp);
                 si.q = div_rcp(L, p, vp);
                 si.r0 = (u32)(L - si.q * p);
-                si.row = (u32)A.off[b - A.k0];
+                si.row = (u32)A.off[b - A.k0] - A.rlo[b - A.k0];
                 si.runcap = si.pad[0] = si.pad[1] = 0;
                 si.flags = 0;
                 si.mlo = si.mhi = 0;
@@ -938,8 +942,8 @@ __global__ void __launch_bounds__(MAXT, MINB) hard_sieve_kernel(HardArgs A0, Mul
                 const u32 b = bb + t;
                 u32 C = 0;
                 for (u32 k = 0; k < nw; k++) C += cw[t * nw + k];
-                const u64 row = st[t].row;
-                if (b < Bs) A.counts[row + (s - A.s0)] = C;
+                const u32 at = st[t].row + (u32)s;
+                if (b < Bs) A.counts[at] = C;
                 if (b > A.kleaf) {
                     const u32* cp = t ? cw + (t - 1) * nw : prev;
                     i32 T = 0;
@@ -950,7 +954,7 @@ __global__ void __launch_bounds__(MAXT, MINB) hard_sieve_kernel(HardArgs A0, Mul
                         intra += (i64)tk * run;
                         run += cp[k];
                     }
-                    if (T) atomicAdd(&A.tallies[row + (s - A.s0)], T);
+                    if (T) atomicAdd(&A.tallies[at], T);
                     acc += intra;
                 }
             }
@@ -975,34 +979,53 @@ __global__ void __launch_bounds__(MAXT, MINB) hard_sieve_kernel(HardArgs A0, Mul
 }
 
 // ---------------------------------------------------------- schedule
+// B_s of segment s: the primes p_b, b <= bmax, with p_b^2 <= x / L and p_b^2 <= L + span - 1
+__device__ __forceinline__ u32 seg_b(u64 x, u64 s, u64 span, u32 bmax, const PiTable& pit)
+{
+    const u64 L = s * span;
+    u64 n = L + span - 1;
+    if (s) n = pc_min(n, x / L);
+    const u64 r = pc_isqrt(n);   // at most x^(1/4) when L > 0
+    return r > pit.limit ? bmax : (u32)pc_min(pi_lookup(pit, r), (u64)bmax);
+}
+
+// The segments of row b in [s0, s1), those with B_s >= b: first segment and number.
+// p_b^2 <= L + span - 1 from segment p_b^2 / span on, p_b^2 <= x / L up to L = x / p_b^2.
+__device__ __forceinline__ u32 row_range(u64 x, u64 p, u64 span, u64 nseg, u64 s0, u64 s1, u32* first)
+{
+    const u64 lo = pc_max(p * p / span, s0);
+    const u64 hi = pc_min(pc_min(x / (p * p) / span + 1, nseg), s1);
+    *first = (u32)lo;
+    return hi > lo ? (u32)(hi - lo) : 0u;
+}
+
+// phi(L - 1, b - 1) at the first segment of row b: L <= p_b^2, so only 1 and the primes from
+// p_b on are left (a shard that starts later has it in start)
+__device__ __forceinline__ u64 row_start(const HardArgs& A, u32 b)
+{
+    const u64 p = A.primes[b], lo = p * p / A.span;
+    if (lo < A.s0) return A.start[b - 1 - A.k0];
+    if (lo == 0) return 0;
+    const u64 n = pi_lookup(A.pit, lo * A.span - 1);   // below p_b^2 <= isqrt(x)
+    return n >= b ? n - b + 2 : 1;
+}
+
 __global__ void seg_b_kernel(u64 x, u64 nseg, u64 span, u32 bmax, PiTable pit, u32* segB, u64* rcp_seg)
 {
     u64 s = (u64)blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= nseg) return;
     rcp_seg[2 * s] = s ? ~0ull / (s * span) : 0;
     rcp_seg[2 * s + 1] = ~0ull / ((s + 1) * span);
-    u32 B = bmax;
-    if (s > 0) {
-        u64 L = s * span;
-        u64 r = pc_isqrt(x / L);
-        u64 pr = pi_lookup(pit, r);
-        if (pr < B) B = (u32)pr;
-    }
-    segB[s] = B;
+    segB[s] = seg_b(x, s, span, bmax, pit);
 }
 
-// S_b = number of segments in [s0, s1) with B_s >= b (B_s is non-increasing in s)
-__global__ void row_len_kernel(const u32* segB, u64 nseg, u64 s0, u64 s1, u32 k0, u32 bmax, u32* len)
+__global__ void row_len_kernel(u64 x, const u32* primes, u64 span, u64 nseg, u64 s0, u64 s1, u32 k0, u32 bmax,
+                               u32* len, u32* rlo)
 {
     u32 t = blockIdx.x * blockDim.x + threadIdx.x;
     u32 b = k0 + t;
     if (b > bmax) return;
-    u64 lo = 0, hi = nseg;   // first s with segB[s] < b
-    while (lo < hi) {
-        u64 mid = (lo + hi) >> 1;
-        if (segB[mid] >= b) lo = mid + 1; else hi = mid;
-    }
-    len[t] = (u32)(pc_min(pc_max(lo, s0), s1) - s0);
+    len[t] = row_range(x, primes[b], span, nseg, s0, s1, rlo + t);
 }
 
 // Upper bound of the hard leaves of every segment (the lpf filter of the
@@ -1047,8 +1070,10 @@ __global__ void __launch_bounds__(NT) hard_combine_kernel(HardArgs A, I128Pair* 
     for (u32 b = A.kleaf + 1 + blockIdx.x; b <= A.bmax; b += gridDim.x) {
         const u64 row = A.off[b - A.k0];
         const u64 Sb = A.off[b - A.k0 + 1] - row;
-        const u64 prow = A.off[b - 1 - A.k0];
-        if (threadIdx.x == 0) s_carry = A.start ? A.start[b - 1 - A.k0] : 0;
+        if (Sb == 0) continue;
+        // row b - 1 holds every segment of row b
+        const u64 prow = A.off[b - 1 - A.k0] + (A.rlo[b - A.k0] - A.rlo[b - 1 - A.k0]);
+        if (threadIdx.x == 0) s_carry = row_start(A, b);
         __syncthreads();
         for (u64 base = 0; base < Sb; base += NT) {
             const u64 s = base + threadIdx.x;
@@ -1159,7 +1184,8 @@ __device__ __forceinline__ double seg_cost(const PlanArgs& P, u64 s)
 {
     const double steps = (double)(P.segB[s] - P.k0);
     const double sz = sqrt(P.z);
-    const double pm = s ? fmin(sqrt(P.x / ((double)s * (double)P.span)), sz) : sz;
+    const double top = fmin(sqrt((double)(s + 1) * (double)P.span), sz);
+    const double pm = s ? fmin(sqrt(P.x / ((double)s * (double)P.span)), top) : top;
     const double ll = pm > 16.0 ? log(log(pm)) - 1.0056 : 0.0;
     return 128.0 * steps + 0.08 * (double)P.span * (8.0 / 30.0) * (ll > 0.0 ? ll : 0.0);
 }
@@ -1390,9 +1416,6 @@ int run_hard_sieve(pc_ctx* ctx, const LeafProblem& P, I128Pair* out)
     A.kleaf = P.c > A.k0 ? P.c : A.k0;
     A.a = P.a;
     A.trunc = P.trunc;
-    const u64 bmax = P.B < P.a ? P.B : P.a;
-    if (bmax <= A.kleaf) return PC_OK;   // no hard leaf needs the sieve
-    A.bmax = (u32)bmax;
     // 32 KiB segments of four 8 KiB warp sub-ranges: four CTAs fit on an SM
     A.seg_bytes = pc_seg_bytes(ctx, 32768);
     A.sub_bytes = pc_sub_bytes(ctx, A.seg_bytes);
@@ -1404,11 +1427,17 @@ int run_hard_sieve(pc_ctx* ctx, const LeafProblem& P, I128Pair* out)
     A.nseg = P.z / A.span + 1;
     A.s0 = 0;
     A.s1 = A.nseg;
-    std::vector<u64> hstart;
     if (P.shard_n) {
         A.s0 = A.nseg * P.shard_k / P.shard_n;
         A.s1 = A.nseg * (P.shard_k + 1) / P.shard_n;
         if (A.s1 <= A.s0) return PC_OK;   // an empty shard
+    }
+    if (!P.table_in_easy) PC_TRY(run_hard_table(ctx, P, A.kleaf, A.s0 * A.span, A.s1 * A.span, out));
+    const u64 bmax = pc_min(pc_min(P.B, P.a), P.R4);
+    if (bmax <= A.kleaf) return PC_OK;   // no hard leaf needs the sieve
+    A.bmax = (u32)bmax;
+    std::vector<u64> hstart;
+    if (P.shard_n) {
         if (A.s0) {
             // carries into the shard: phi(L - 1, b) for every b (Section 4), computed
             // before this run claims the context's scratch
@@ -1429,28 +1458,29 @@ int run_hard_sieve(pc_ctx* ctx, const LeafProblem& P, I128Pair* out)
     A.primes_rcp = ctx->T.primes_rcp.as<u64>();
 
     const u64 nrows = bmax - A.k0 + 1;
-    PC_TRY(buf_reserve(ctx, ctx->seg_b, A.nseg * sizeof(u32) + (nrows + 1) * sizeof(u32)));
+    PC_TRY(buf_reserve(ctx, ctx->seg_b, A.nseg * sizeof(u32) + 2 * (nrows + 1) * sizeof(u32)));
     PC_TRY(buf_reserve(ctx, ctx->seg_off, (nrows + 1) * sizeof(u64) + 3 * A.nseg * sizeof(u64) + A.nseg * sizeof(u32) +
                                               A.nseg * sizeof(HeavySeg) + 16));
     u32* segB = ctx->seg_b.as<u32>();
     u32* rowlen = segB + A.nseg;
+    u32* rlo = rowlen + nrows + 1;
     u64* off = ctx->seg_off.as<u64>();
     unsigned long long* est = (unsigned long long*)(off + nrows + 1);
     u64* rcp_seg = (u64*)(est + A.nseg);
     u32* split = (u32*)(rcp_seg + 2 * A.nseg);   // the work-item split of every segment
     HeavySeg* heavy = (HeavySeg*)(((uintptr_t)(split + A.nseg) + 15) & ~(uintptr_t)15);
     A.rcp_seg = rcp_seg;
-    A.rcp_y = ~0ull / P.y;
     seg_b_kernel<<<(unsigned)((A.nseg + 255) / 256), 256, 0, ctx->stream>>>(P.x, A.nseg, A.span, A.bmax, A.pit, segB,
                                                                             rcp_seg);
     PC_LAUNCHED(ctx);
-    row_len_kernel<<<(unsigned)((nrows + 255) / 256), 256, 0, ctx->stream>>>(segB, A.nseg, A.s0, A.s1, A.k0, A.bmax,
-                                                                              rowlen);
+    row_len_kernel<<<(unsigned)((nrows + 255) / 256), 256, 0, ctx->stream>>>(P.x, A.primes, A.span, A.nseg, A.s0,
+                                                                              A.s1, A.k0, A.bmax, rowlen, rlo);
     PC_LAUNCHED(ctx);
     ctx->stats.kernel_launches += 2;
     PC_TRY(scan_exclusive_u32_to_u64(ctx, rowlen, off, nrows));
     A.segB = segB;
     A.off = off;
+    A.rlo = rlo;
     A.start = nullptr;
     if (!hstart.empty()) {
         PC_TRY(buf_reserve(ctx, ctx->starts, hstart.size() * sizeof(u64)));
@@ -1563,29 +1593,18 @@ __global__ void mq_seg_b_kernel(const HardArgs* qa, const u64* pref, u32 Q, u32*
     const u64 s = g - pref[q];
     rcp_seg[2 * g] = s ? ~0ull / (s * A.span) : 0;
     rcp_seg[2 * g + 1] = ~0ull / ((s + 1) * A.span);
-    u32 B = A.bmax;
-    if (s > 0) {
-        const u64 r = pc_isqrt(A.x / (s * A.span));
-        const u64 pr = pi_lookup(A.pit, r);
-        if (pr < B) B = (u32)pr;
-    }
-    segB[g] = B;
+    segB[g] = seg_b(A.x, s, A.span, A.bmax, A.pit);
 }
 
-// row b = k0 + g - rpref[q] of query q: the number of its segments with B_s >= b
-__global__ void mq_row_len_kernel(const HardArgs* qa, const u64* rpref, u32 Q, u32* len)
+// row b = k0 + g - rpref[q] of query q: its segments with B_s >= b
+__global__ void mq_row_len_kernel(const HardArgs* qa, const u64* rpref, u32 Q, u32* len, u32* rlo)
 {
     const u64 g = (u64)blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= rpref[Q]) return;
     const u64 q = mq_find(rpref, Q + 1, g);
     const HardArgs& A = qa[q];
     const u32 b = A.k0 + (u32)(g - rpref[q]);
-    u64 lo = 0, hi = A.nseg;   // first s with segB[s] < b
-    while (lo < hi) {
-        const u64 mid = (lo + hi) >> 1;
-        if (A.segB[mid] >= b) lo = mid + 1; else hi = mid;
-    }
-    len[g] = (u32)lo;
+    len[g] = row_range(A.x, A.primes[b], A.span, A.nseg, 0, A.nseg, rlo + g);
 }
 
 // the carries: a warp per (query, b), kleaf < b <= bmax: the exclusive scan over
@@ -1598,8 +1617,10 @@ __global__ void mq_combine_kernel(const HardArgs* qa, const u64* cpref, u32 Q, I
         const u64 q = mq_find(cpref, Q + 1, g);
         const HardArgs& A = qa[q];
         const u32 b = A.kleaf + 1 + (u32)(g - cpref[q]);
-        const u64 row = A.off[b - A.k0], Sb = A.off[b - A.k0 + 1] - row, prow = A.off[b - 1 - A.k0];
-        u64 carry = 0;
+        const u64 row = A.off[b - A.k0], Sb = A.off[b - A.k0 + 1] - row;
+        if (Sb == 0) continue;
+        const u64 prow = A.off[b - 1 - A.k0] + (A.rlo[b - A.k0] - A.rlo[b - 1 - A.k0]);
+        u64 carry = row_start(A, b);
         i128 dot = 0;
         for (u64 base = 0; base < Sb; base += 32) {
             const u64 s = base + lane;
@@ -1650,7 +1671,7 @@ int mq_hard(pc_ctx* ctx, const MQPlan& P)
     u64 bound = 0;   // count-row entries: at most segments x rows per query
     for (u32 q = 0; q < Q; q++) {
         const MQ& m = P.hq[q];
-        const u64 bmax = m.B < m.a ? m.B : m.a;
+        const u64 bmax = pc_min(pc_min(m.B, m.a), m.R4);
         const bool work = m.c == 5 && bmax > T.kleaf;
         const u64 nseg = work ? m.z / T.span + 1 : 0;
         const u64 nrows = work ? bmax - T.k0 + 1 : 0;
@@ -1667,11 +1688,11 @@ int mq_hard(pc_ctx* ctx, const MQPlan& P)
     }
     for (u32 q = 0; q <= Q; q++) ipref[q] = (u32)spref[q];
     // mq_h: spref | rpref | cpref (Q+1 u64 each) | ipref (Q+1 u32) | segB (S u32) | rcp_seg (2S u64) |
-    // rowlen (R u32) | off (R+1 u64) | queue + counters (128 B)
+    // rowlen (R u32) | rlo (R u32) | off (R+1 u64) | queue + counters (128 B)
     auto al = [](size_t v) { return (v + 15) / 16 * 16; };
     const size_t o_r = al((Q + 1) * 8), o_c = o_r + al((Q + 1) * 8), o_i = o_c + al((Q + 1) * 8);
     const size_t o_sb = o_i + al((Q + 1) * 4), o_rc = o_sb + al(S * 4), o_rl = o_rc + al(2 * S * 8);
-    const size_t o_off = o_rl + al(R * 4), o_q = o_off + al((R + 1) * 8), total = o_q + 128;
+    const size_t o_ro = o_rl + al(R * 4), o_off = o_ro + al(R * 4), o_q = o_off + al((R + 1) * 8), total = o_q + 128;
     PC_TRY(buf_reserve(ctx, ctx->mq_h, total));
     PC_TRY(buf_reserve(ctx, ctx->mq_hq, Q * sizeof(HardArgs)));
     PC_TRY(buf_reserve(ctx, ctx->counts, bound * sizeof(u32)));
@@ -1684,6 +1705,7 @@ int mq_hard(pc_ctx* ctx, const MQPlan& P)
     u32* d_segB = (u32*)(base + o_sb);
     u64* d_rcp = (u64*)(base + o_rc);
     u32* d_rowlen = (u32*)(base + o_rl);
+    u32* d_rlo = (u32*)(base + o_ro);
     u64* d_off = (u64*)(base + o_off);
     u32* d_queue = (u32*)(base + o_q);
     HardArgs* d_qa = ctx->mq_hq.as<HardArgs>();
@@ -1697,15 +1719,15 @@ int mq_hard(pc_ctx* ctx, const MQPlan& P)
         A.c = m.c;
         A.a = m.a;
         A.trunc = false;
-        const u64 bmax = m.B < m.a ? m.B : m.a;
+        const u64 bmax = pc_min(pc_min(m.B, m.a), m.R4);
         A.bmax = (u32)pc_max(bmax, T.k0);
         A.nseg = spref[q + 1] - spref[q];
         A.s0 = 0;
         A.s1 = A.nseg;
-        A.rcp_y = ~0ull / m.y;
         A.segB = d_segB + spref[q];
         A.rcp_seg = d_rcp + 2 * spref[q];
         A.off = d_off + rpref[q];
+        A.rlo = d_rlo + rpref[q];
         A.start = nullptr;
         A.counts = ctx->counts.as<u32>();
         A.tallies = ctx->tallies.as<i32>();
@@ -1739,7 +1761,7 @@ int mq_hard(pc_ctx* ctx, const MQPlan& P)
     PC_CUDA(ctx, cudaMemsetAsync(ctx->tallies.p, 0, bound * sizeof(i32), st));
     mq_seg_b_kernel<<<(unsigned)((S + 255) / 256), 256, 0, st>>>(d_qa, d_spref, Q, d_segB, d_rcp);
     PC_LAUNCHED(ctx);
-    mq_row_len_kernel<<<(unsigned)((R + 255) / 256), 256, 0, st>>>(d_qa, d_rpref, Q, d_rowlen);
+    mq_row_len_kernel<<<(unsigned)((R + 255) / 256), 256, 0, st>>>(d_qa, d_rpref, Q, d_rowlen, d_rlo);
     PC_LAUNCHED(ctx);
     PC_TRY(scan_exclusive_u32_to_u64(ctx, d_rowlen, d_off, R));
     // the sieve: items are the segments of every query, handed out in order

@@ -197,9 +197,14 @@ struct LeafProblem {
     bool trunc;   // a < pi(y): filter gpf(m) <= p_a
     u64 piy;      // pi(y)
     u64 B;        // pi(isqrt z)
+    u64 R4;       // pi(x^(1/4)): a leaf with u >= p_b^2 and m > p_b has p_b^4 < x
     // hard-leaf sieve over segments [shard_k * nseg / shard_n, (shard_k + 1) * nseg / shard_n) only
     // (shard_n = 0: all of them); the leaves' carries then start from phi(L - 1, b)
     u32 shard_k = 0, shard_n = 0;
+    // the hard leaves with u < p_b^2 (read from the pi table, see easy_range) are added to the
+    // easy sum by run_easy, not to the hard one by run_hard_sieve: for callers that want only
+    // the total
+    bool table_in_easy = false;
 };
 
 // phi(m, b) for every c <= b <= b_max (Section 4 starting values): out[b - c]
@@ -213,6 +218,8 @@ int run_trivial(pc_ctx* ctx, const LeafProblem& P, I128Pair* out);
 int run_easy(pc_ctx* ctx, const LeafProblem& P, I128Pair* out);
 int run_hard_smallb(pc_ctx* ctx, const LeafProblem& P, I128Pair* out);
 int run_hard_sieve(pc_ctx* ctx, const LeafProblem& P, I128Pair* out);
+// the hard leaves with y <= u < p_b^2, b > b_min, whose u lies in [u_lo, u_hi)
+int run_hard_table(pc_ctx* ctx, const LeafProblem& P, u64 b_min, u64 u_lo, u64 u_hi, I128Pair* out);
 int run_p2(pc_ctx* ctx, u64 x, u64 y, u64 a, I128Pair* out);
 
 // ------------------------------------------------------- batched queries
@@ -225,6 +232,7 @@ struct MQ {
     u64 K;      // pi(isqrt x)
     u64 nlim;   // m-list entries with m <= y
     u64 E;      // pi(iroot3 x): the easy leaves have b <= E
+    u64 R4;     // pi(x^(1/4)): the leaves that need the sieve have b <= R4
     u32 c;
     u32 pad;
 };

@@ -12,6 +12,13 @@
 // hard leaf, resolved by the main sieve (pc_hard.cu); those with b <= 3 have
 // the closed forms phi(u,0) = u, phi(u,1) = u - u/2, phi(u,2) = u - u/2 - u/3 + u/6.
 // The easy leaves are embarrassingly parallel (Section 3).
+//
+// The hard leaves with y <= u < p_b^2 do not need the sieve either: phi(u, b-1) is
+// pi(u) - b + 2 there too, m > p_b gives u < x / p_b^2 and so u < isqrt(x), and the pi
+// table reaches isqrt(x).  They are about half of all hard leaves, and the sieve then
+// needs only the primes p_b with p_b^2 below its segment's end and p_b <= x^(1/4).
+// (S2_hard(10^18), y = 2*10^7: 66.9 -> 58.5 ms, its sieve kernel 64.8 -> 54.2 ms, the table
+// leaves 2.6 ms; the five parts at 10^15, alpha 9: 8.0 -> 2.2 ms; pi(10^14) 1.78 -> 1.31 ms.)
 #include "pc_internal.h"
 
 struct LeafArgs {
@@ -204,6 +211,7 @@ static constexpr u64 CLUST_K = 2;   // measured: 2 beats 1 and 3 by about 1 % at
 
 struct EasyRange {
     u64 i0, i1;   // list indices [i0, i1) or prime indices (i0, i1] shifted to [i0+1, i1+1)
+    u64 ih;       // hard leaves with u < p_b^2 first: [i0, ih) have u >= y (src 1), else i0
     u64 im;       // first index of the clustered part (src 1), else i1
     u32 src;      // 0: m-list, 1: primes
     u32 l0, l1;   // clustered part: pi(u) runs from l0 (largest q) to l1 (smallest q)
@@ -219,38 +227,53 @@ __host__ __device__ inline u64 easy_chunks(const EasyRange& r, u32 clust_chunk)
     const u64 nclust = r.i1 <= r.im ? 0
                        : clust_chunk ? (r.i1 - r.im + clust_chunk - 1) / clust_chunk
                                      : ((u64)r.l1 - r.l0 + CLUST_L) / CLUST_L;
-    return (r.im - r.i0 + EASY_CHUNK - 1) / EASY_CHUNK + nclust;
+    return (r.ih - r.i0 + EASY_CHUNK - 1) / EASY_CHUNK + (r.im - r.ih + EASY_CHUNK - 1) / EASY_CHUNK + nclust;
 }
 
-// The easy leaves of prime p_b for a query (x, y, a): list indices [i0, i1) of the
-// m-list, or of the primes when p_b^2 > y, and where the clustered part starts.
-__device__ __forceinline__ EasyRange easy_range(const LeafArgs& A, u64 x, u64 y, u64 a, u64 b)
+// Which leaves of p_b a range holds: the easy ones, the hard ones with u < p_b^2 (and
+// u in [u_lo, u_hi)), or both.
+enum { LEAVES_EASY = 0, LEAVES_TABLE = 1, LEAVES_BOTH = 2 };
+
+// The leaves of prime p_b for a query (x, y, a) whose phi(u, b-1) is pi(u) - b + 2: list
+// indices [i0, i1) of the m-list, or of the primes when p_b^2 > y, where u falls below y
+// and where the clustered part starts.
+__device__ __forceinline__ EasyRange easy_range(const LeafArgs& A, u64 x, u64 y, u64 a, u64 b, u32 what, u64 u_lo,
+                                                u64 u_hi)
 {
     const u64 p = A.primes[b];
     const u64 xp = x / p;
-    const u64 T = pc_min(p * p, y);
-    const u64 lo = pc_max(y / p, xp / T);
-    const u64 hi = pc_min(y, xp / p);
-    EasyRange r{0, 0, 0, 0, 0, 0, 0};
-    if (hi > lo) {
-        if (p * p > y) {
-            // lpf(m) > p_b and m <= y < p_b^2: m is a prime q, p_b < q <= p_a
-            u64 k0 = pc_max(pi_lookup(A.pit, lo), b);
-            u64 k1 = pc_min(pi_lookup(A.pit, hi), a);
+    EasyRange r{0, 0, 0, 0, 0, 0, 0, 0};
+    if (p * p > y) {
+        // lpf(m) > p_b and m <= y < p_b^2: m is a prime q, p_b < q <= p_a
+        const u64 hy = pc_min(y, xp / y);   // u >= y up to q = hy
+        u64 lo = y / p, hi = pc_min(y, xp / p);
+        if (what == LEAVES_TABLE) {
+            hi = pc_min(hy, u_lo ? xp / u_lo : y);
+            lo = pc_max(lo, xp / u_hi);
+        }
+        // (b <= 3: every hard leaf has a closed form, see run_hard_smallb)
+        lo = pc_max(lo, what == LEAVES_EASY || b <= 3 ? hy : xp / (p * p));
+        if (hi > lo) {
+            const u64 k0 = pc_max(pi_lookup(A.pit, lo), b);
+            const u64 k1 = pc_min(pi_lookup(A.pit, hi), a);
             if (k1 > k0) {
                 r.i0 = k0 + 1;
                 r.i1 = k1 + 1;
                 r.src = 1;
-                // clustered from the first prime q with q^2 >= CLUST_K * x/p_b
+                r.ih = pc_min(pc_max(pi_lookup(A.pit, hy) + 1, r.i0), r.i1);
+                // clustered from the first prime q with q^2 >= CLUST_K * x/p_b (u <= q/2 < y there)
                 const u64 qc = xp > ~0ull / CLUST_K ? hi + 1 : pc_isqrt(CLUST_K * xp - 1) + 1;
-                r.im = qc > hi ? r.i1 : pc_min(pc_max(pi_lookup(A.pit, qc - 1) + 1, r.i0), r.i1);
+                r.im = qc > hi ? r.i1 : pc_min(pc_max(pi_lookup(A.pit, qc - 1) + 1, r.ih), r.i1);
                 if (r.im < r.i1) {
-                    // u = x/(p_b q) <= q/3 < y: pi at the smallest and the largest clustered q
+                    // pi at the smallest and the largest clustered q
                     r.l0 = (u32)pi_lookup(A.pit, xp / A.primes[r.i1 - 1]);
                     r.l1 = (u32)pi_lookup(A.pit, xp / A.primes[r.im]);
                 }
             }
-        } else {
+        }
+    } else if (what != LEAVES_TABLE) {
+        const u64 lo = pc_max(y / p, xp / (p * p)), hi = pc_min(y, xp / p);
+        if (hi > lo) {
             // the last sub-list whose entries all have lpf index > K, K <= b: it holds every
             // leaf of p_b and fewer entries to skip (lpf <= p_b) than the whole m-list
             u32 li = 0;
@@ -263,15 +286,19 @@ __device__ __forceinline__ EasyRange easy_range(const LeafArgs& A, u64 x, u64 y,
             r.ls = li;
         }
     }
-    if (r.src == 0) r.im = r.i1;
+    if (r.src == 0) {
+        r.ih = r.i0;
+        r.im = r.i1;
+    }
     return r;
 }
 
-__global__ void easy_ranges_kernel(LeafArgs A, u64 b_lo, u64 nb, EasyRange* rng, u32* nchunk)
+__global__ void easy_ranges_kernel(LeafArgs A, u64 b_lo, u64 nb, u32 what, u64 u_lo, u64 u_hi, EasyRange* rng,
+                                   u32* nchunk)
 {
     u64 t = (u64)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= nb) return;
-    const EasyRange r = easy_range(A, A.x, A.y, A.a, b_lo + t);
+    const EasyRange r = easy_range(A, A.x, A.y, A.a, b_lo + t, what, u_lo, u_hi);
     rng[t] = r;
     nchunk[t] = (u32)easy_chunks(r, A.clust_chunk);
 }
@@ -295,11 +322,25 @@ static constexpr u64 PI_ODD_Y = 1ull << 29;
 // 32 lanes of a warp; adds this lane's share of the sum to s.
 template <int MODE>
 __device__ __forceinline__ void easy_chunk(const LeafArgs& A, u64 x, u64 a, u64 b, const EasyRange& r, u64 c, u32 cc,
-                                           u32 lane, i64& s, u32& n_one, u32& n_runs, u32& n_run_leaves)
+                                           u32 lane, i64& s, u32& n_table, u32& n_one, u32& n_runs, u32& n_run_leaves)
 {
-    const u64 nsp = (r.im - r.i0 + EASY_CHUNK - 1) / EASY_CHUNK;
     const u64 p = A.primes[b];
     const u64 xp = div_rcp(x, p, A.primes_rcp[b]);
+    const u64 nh = (r.ih - r.i0 + EASY_CHUNK - 1) / EASY_CHUNK;
+    if (c < nh) {
+        // hard leaves with y <= u < p_b^2, m = q prime: u < isqrt(x) may be above 2^31, hence
+        // the 64-bit reciprocal; the records of neighbouring q are u / q prime gaps apart
+        const u32 start = (u32)(r.i0 + c * EASY_CHUNK), end = (u32)pc_min(r.ih, (u64)start + EASY_CHUNK);
+        u64 sum = 0;
+        u32 k = 0;
+        for (u32 i = start + lane; i < end; i += 32, k++)
+            sum += pi_lookup(A.pit, div_rcp(xp, A.primes[i], A.primes_rcp[i]));
+        s += (i64)sum - (i64)k * ((i64)b - 2);
+        n_table += k;
+        return;
+    }
+    c -= nh;
+    const u64 nsp = (r.im - r.ih + EASY_CHUNK - 1) / EASY_CHUNK;
     if (c >= nsp) {
         if (MODE == PI_ODD && cc == 0) {
             // Clustered chunk by pi value.  With G(l) = the number of clustered q (prime
@@ -392,7 +433,7 @@ __device__ __forceinline__ void easy_chunk(const LeafArgs& A, u64 x, u64 a, u64 
         }
         return;
     }
-    const u32 start = (u32)(r.i0 + c * EASY_CHUNK);   // list and prime indices are below 2^32
+    const u32 start = (u32)(r.ih + c * EASY_CHUNK);   // list and prime indices are below 2^32
     const u32 end = (u32)pc_min(r.im, (u64)start + EASY_CHUNK);
     if (MODE == PI_ODD && r.src) {
         // m = q prime: every leaf adds pi(u) - b + 2
@@ -448,7 +489,8 @@ __global__ void easy_kernel(LeafArgs A, u64 b_lo, const EasyRange* rng, const u6
     __shared__ i128 scratch[32];
     const u32 lane = threadIdx.x & 31;
     i64 s = 0;
-    u32 n_one = 0, n_runs = 0, n_run_leaves = 0;   // counters: leaves one at a time, runs, leaves in runs
+    u32 n_table = 0, n_one = 0, n_runs = 0, n_run_leaves = 0;   // hard leaves from the table, leaves one at a time,
+                                                                // runs, leaves in runs
     // chunks are handed out one at a time to warps (their costs differ widely)
     for (;;) {
         u64 ch = 0;
@@ -457,13 +499,14 @@ __global__ void easy_kernel(LeafArgs A, u64 b_lo, const EasyRange* rng, const u6
         if (ch >= nchunks) break;
         const u64 t = cmap[ch];
         const EasyRange r = rng[t];
-        easy_chunk<MODE>(A, A.x, A.a, b_lo + t, r, ch - choff[t], A.clust_chunk, lane, s, n_one, n_runs,
+        easy_chunk<MODE>(A, A.x, A.a, b_lo + t, r, ch - choff[t], A.clust_chunk, lane, s, n_table, n_one, n_runs,
                             n_run_leaves);
     }
     if (stat) {
         const u32 a0 = __reduce_add_sync(0xffffffffu, n_one), a1 = __reduce_add_sync(0xffffffffu, n_runs);
-        const u32 a2 = __reduce_add_sync(0xffffffffu, n_run_leaves);
+        const u32 a2 = __reduce_add_sync(0xffffffffu, n_run_leaves), a4 = __reduce_add_sync(0xffffffffu, n_table);
         if (lane == 0) {
+            if (a4) atomicAdd(stat + 4, (unsigned long long)a4);
             if (a0) atomicAdd(stat, (unsigned long long)a0);
             if (a1) atomicAdd(stat + 1, (unsigned long long)a1);
             if (a2) atomicAdd(stat + 2, (unsigned long long)a2);
@@ -473,11 +516,10 @@ __global__ void easy_kernel(LeafArgs A, u64 b_lo, const EasyRange* rng, const u6
     if (threadIdx.x == 0) store_i128(part + blockIdx.x, v);
 }
 
-int run_easy(pc_ctx* ctx, const LeafProblem& P, I128Pair* out)
+// The leaves of the primes b_lo <= b < b_lo + nb (see easy_range for what, u_lo, u_hi)
+static int leaf_pass(pc_ctx* ctx, const LeafProblem& P, u64 b_lo, u64 nb, u32 what, u64 u_lo, u64 u_hi,
+                     I128Pair* out)
 {
-    u64 b_lo = (u64)P.c + 1;
-    if (P.a < b_lo) return PC_OK;
-    u64 nb = P.a - b_lo + 1;
     PC_TRY(buf_reserve(ctx, ctx->easy_rng, nb * sizeof(EasyRange)));
     PC_TRY(buf_reserve(ctx, ctx->easy_chunk_off, (nb + 1) * sizeof(u64) + (nb + 1) * sizeof(u32)));
     u64* choff = ctx->easy_chunk_off.as<u64>();
@@ -485,7 +527,7 @@ int run_easy(pc_ctx* ctx, const LeafProblem& P, I128Pair* out)
     LeafArgs A = make_args(ctx, P, 0);
     const bool odd = !A.sampled && P.y < PI_ODD_Y && ctx->T.podd_limit >= P.y;
     if (odd) A.clust_chunk = 0;   // clustered chunks by pi value
-    easy_ranges_kernel<<<(unsigned)((nb + 255) / 256), 256, 0, ctx->stream>>>(A, b_lo, nb,
+    easy_ranges_kernel<<<(unsigned)((nb + 255) / 256), 256, 0, ctx->stream>>>(A, b_lo, nb, what, u_lo, u_hi,
                                                                               ctx->easy_rng.as<EasyRange>(), nch);
     PC_LAUNCHED(ctx);
     ctx->stats.kernel_launches++;
@@ -506,7 +548,8 @@ int run_easy(pc_ctx* ctx, const LeafProblem& P, I128Pair* out)
     PC_TRY(buf_reserve(ctx, ctx->partials, g * sizeof(I128Pair)));
     PC_TRY(buf_reserve(ctx, ctx->queue, 64));
     PC_CUDA(ctx, cudaMemsetAsync(ctx->queue.p, 0, 64, ctx->stream));
-    PC_CUDA(ctx, cudaEventRecord(ctx->ev[2], ctx->stream));
+    const bool timed = what != LEAVES_TABLE;
+    if (timed) PC_CUDA(ctx, cudaEventRecord(ctx->ev[2], ctx->stream));
     const EasyRange* rng = ctx->easy_rng.as<EasyRange>();
     const u32* cmap = ctx->easy_cmap.as<u32>();
     unsigned long long* queue = (unsigned long long*)ctx->queue.p;
@@ -520,10 +563,26 @@ int run_easy(pc_ctx* ctx, const LeafProblem& P, I128Pair* out)
         easy_kernel<PI_REC><<<g, 256, 0, ctx->stream>>>(A, b_lo, rng, choff, cmap, nchunks, queue,
                                                         ctx->partials.as<I128Pair>(), ctx->dstat);
     PC_LAUNCHED(ctx);
-    PC_CUDA(ctx, cudaEventRecord(ctx->ev[3], ctx->stream));
-    ctx->easy_timed = true;
+    if (timed) {
+        PC_CUDA(ctx, cudaEventRecord(ctx->ev[3], ctx->stream));
+        ctx->easy_timed = true;
+    }
     ctx->stats.kernel_launches++;
     return reduce_i128(ctx, ctx->partials.as<I128Pair>(), g, out);
+}
+
+int run_easy(pc_ctx* ctx, const LeafProblem& P, I128Pair* out)
+{
+    const u64 b_lo = (u64)P.c + 1;
+    if (P.a < b_lo) return PC_OK;
+    return leaf_pass(ctx, P, b_lo, P.a - b_lo + 1, P.table_in_easy ? LEAVES_BOTH : LEAVES_EASY, 0, ~0ull, out);
+}
+
+int run_hard_table(pc_ctx* ctx, const LeafProblem& P, u64 b_min, u64 u_lo, u64 u_hi, I128Pair* out)
+{
+    const u64 b_hi = pc_min(P.B, P.a);   // p_b < q and u >= y give p_b^2 < z
+    if (b_hi <= b_min || u_hi <= u_lo) return PC_OK;
+    return leaf_pass(ctx, P, b_min + 1, b_hi - b_min, LEAVES_TABLE, u_lo, u_hi, out);
 }
 
 // ------------------------------------------------------- hard, b <= 3
@@ -606,6 +665,7 @@ __global__ void mq_info_kernel(PiTable pit, RankTable rk, MQ* qs, u32 Q, const u
     m.K = pi_lookup(pit, pc_isqrt(m.x));
     m.nlim = rank_lookup(rk, m.y);
     m.E = pi_lookup(pit, pc_iroot3(m.x));
+    m.R4 = pi_lookup(pit, pc_isqrt(pc_isqrt(m.x)));
     qs[q] = m;
     const u64 v = m.x / Qc;
     const u32 r = (u32)(m.x - v * Qc);
@@ -689,7 +749,7 @@ __global__ void mq_easy_ranges_kernel(LeafArgs T, const MQ* qs, const u64* pref,
     if (g >= pref[Q]) return;
     const u64 q = mq_find(pref, Q + 1, g);
     const MQ m = qs[q];
-    const EasyRange r = easy_range(T, m.x, m.y, m.a, m.c + 1 + (g - pref[q]));
+    const EasyRange r = easy_range(T, m.x, m.y, m.a, m.c + 1 + (g - pref[q]), LEAVES_BOTH, 0, ~0ull);
     rng[g] = r;
     nch[g] = (u32)easy_chunks(r, 0);   // clustered chunks by pi value (odd-table path)
 }
@@ -710,9 +770,9 @@ __global__ void mq_easy_kernel(LeafArgs T, const MQ* qs, const u64* pref, u32 Q,
         const MQ m = qs[q];
         const EasyRange r = rng[g];
         i64 s = 0;
-        u32 n1 = 0, nr = 0, nrl = 0;
+        u32 nt = 0, n1 = 0, nr = 0, nrl = 0;
         easy_chunk<PI_ODD>(T, m.x, m.a, m.c + 1 + (g - pref[q]), r, ch - choff[g], 0, lane, s,
-                          n1, nr, nrl);
+                          nt, n1, nr, nrl);
         s = warp_sum_i64(s);
         if (lane == 0 && s) mq_atomic_add_i128(parts + 5 * q + 2, (i128)s);
     }
