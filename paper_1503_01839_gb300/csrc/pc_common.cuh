@@ -101,6 +101,35 @@ __device__ __forceinline__ u32 div_dv(u64 n, u64 dv)
     if (n - (u64)q * d >= d) q++;
     return q;
 }
+// The same quotient for many divisors of one dividend n: with k = max(0, bits of n - 32)
+// and T = floor(n / 2^k) < 2^32, the estimate floor(T v / 2^(32+s-k)) falls short of n/d by
+// less than n / 2^(32+s) + 2^k / d (from v) + 0 or 2^k / d (from T, exact when k = 0).
+// With d < 2^(s+1) and n >= 2^(31+k) if k > 0, both terms are below (n/d) / 2^31: the estimate
+// is the quotient or one less whenever the quotient is below 2^30 (and s >= k there, since
+// n/d >= 2^(31+k) / 2^(s+1)).  The remainder is below 2 d, so with d < 2^31 its low 32 bits
+// decide.  One high product, one low product and a comparison, where div_dv takes two wide
+// products and a 64-bit remainder.  The easy-leaf kernel is bound by its instructions and its
+// gathers: with this, pi_odd1's masks and the runs summed by parts, 30.1 -> 21.1 ms at
+// pi(10^18), alpha 56, 1.63 -> 1.06 ms at pi(10^16).
+struct QuotOf {
+    u32 top, lo;
+    u32 k;
+    __device__ __forceinline__ explicit QuotOf(u64 n)
+    {
+        const int kk = 32 - __clzll((long long)n);
+        k = kk > 0 ? (u32)kk : 0u;
+        top = (u32)(n >> k);
+        lo = (u32)n;
+    }
+    // dv = d, floor((2^(32+s) - 1) / d); sh = s - k
+    __device__ __forceinline__ u32 by(uint2 dv, u32 sh) const
+    {
+        const u32 q = __umulhi(top, dv.y) >> sh;
+        return q + (lo - q * dv.x >= dv.x ? 1u : 0u);
+    }
+    __device__ __forceinline__ u32 shift(u32 d) const { return (31u - (u32)__clz((int)d)) - k; }
+};
+
 PC_HD u64 pc_dv(u32 d)
 {
     if (d == 0) return 0;
@@ -147,15 +176,19 @@ __device__ __forceinline__ u64 pi_lookup(const PiTable& t, u64 v)
 
 // Odd-number pi table: record w covers [64w, 64w + 64); .x holds one bit per
 // odd number 64w + 2j + 1 (j = 0..31) that is prime, with bit 0 of record 0
-// (the number 1) standing for the prime 2, and .y = pi(64w - 1).  pi(u) for
-// 2 <= u <= limit is .y plus the bits of the odd numbers <= u: a shift, an
-// 8-byte load and one 32-bit popcount, with no division and no wheel residue.
-__device__ __forceinline__ u32 pi_odd(const uint2* t, u32 u)
+// (the number 1) standing for the prime 2, and .y = pi(64w - 1).  With
+// h = floor((u + 1) / 2) the odd numbers <= u, pi(u) for 2 <= u <= limit is
+// record h / 32's .y plus its low h mod 32 bits (u = 64w - 1 reads record w): two
+// shifts, an 8-byte load, a mask and one 32-bit popcount, no division, no wheel residue.
+__device__ __forceinline__ u32 pi_odd1(const uint2* t, u32 u1)   // u1 = u + 1
 {
-    const uint2 r = __ldg(t + (u >> 6));
-    const u32 e = ((u & 63u) + 1u) >> 1;   // odd numbers <= u in the record, 0..32
-    return r.y + __popc(__funnelshift_lc(0u, r.x, 32u - e));   // r.x << (32 - e), 0 when e = 0
+    const u32 h = u1 >> 1;
+    const uint2 r = __ldg(t + (h >> 5));
+    u32 low;   // h mod 32 low bits set
+    asm("bmsk.wrap.b32 %0, 0, %1;" : "=r"(low) : "r"(h));
+    return r.y + __popc(r.x & low);
 }
+__device__ __forceinline__ u32 pi_odd(const uint2* t, u32 u) { return pi_odd1(t, u + 1); }
 
 // rank structure over a plain bitset of [0, limit]: rank(v) = #set bits <= v.
 struct RankTable {

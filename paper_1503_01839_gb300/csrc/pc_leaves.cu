@@ -200,9 +200,9 @@ int run_trivial(pc_ctx* ctx, const LeafProblem& P, I128Pair* out)
 // grows, and stays >= p_l), so the whole run counts (run length) * (l - b + 2).
 // Those leaves (q^2 >= CLUST_K * x/p_b, i.e. u <= q / CLUST_K) are taken run by
 // run; the rest one leaf per thread.  With the odd-number pi table the runs are
-// taken by their value l, 31 consecutive l per warp pass: the run of l holds the
+// taken by their value l, 32 consecutive l per warp pass: the run of l holds the
 // clustered q with (x/p_b)/p_(l+1) < q <= (x/p_b)/p_l, so its length is a
-// difference of two pi lookups that neighbouring lanes share, and p_l's record is
+// difference of two pi lookups (summed by parts, see easy_chunk), and p_l's record is
 // read with its neighbours'.  Otherwise each thread walks the runs of a contiguous
 // slice of q, one pi lookup and two quotients per run.  Chunks go to warps one at
 // a time.
@@ -220,7 +220,7 @@ struct EasyRange {
 
 // Clustered chunks taken by pi value (clust_chunk = 0, the odd-table path): the
 // clustered leaves of p_b with pi(u) = l, for every l in [l0, l1], CLUST_L values a chunk.
-static constexpr u32 CLUST_L = 31 * 128;
+static constexpr u32 CLUST_L = 32 * 124;
 
 __host__ __device__ inline u64 easy_chunks(const EasyRange& r, u32 clust_chunk)
 {
@@ -313,8 +313,8 @@ __global__ void easy_chunk_map_kernel(u64 nb, const u64* choff, u32* cmap)
 
 // How an easy leaf reads pi(u): from the popcount pi table (PI_REC), from the
 // sampled table of Section 2.1 (PI_SAMPLED), or from the odd-number table with
-// the 32-bit reciprocal divisions of div_dv (PI_ODD, for y < 2^29: every
-// quotient taken, u < y and the run bound (x/p_b)/p_l < 2.3 y, stays below 2^31).
+// the 32-bit reciprocal divisions of QuotOf (PI_ODD, for y < 2^29: every u < y stays
+// below 2^30, and where a run bound (x/p_b)/p_l does not it is clamped to the last q).
 enum { PI_REC = 0, PI_SAMPLED = 1, PI_ODD = 2 };
 static constexpr u64 PI_ODD_Y = 1ull << 29;
 
@@ -328,13 +328,22 @@ __device__ __forceinline__ void easy_chunk(const LeafArgs& A, u64 x, u64 a, u64 
     const u64 xp = div_rcp(x, p, A.primes_rcp[b]);
     const u64 nh = (r.ih - r.i0 + EASY_CHUNK - 1) / EASY_CHUNK;
     if (c < nh) {
-        // hard leaves with y <= u < p_b^2, m = q prime: u < isqrt(x) may be above 2^31, hence
-        // the 64-bit reciprocal; the records of neighbouring q are u / q prime gaps apart
+        // hard leaves with y <= u < p_b^2, m = q prime; u < isqrt(x) may be 2^30 or more, then
+        // the 64-bit reciprocal.  The records of neighbouring q are u / q prime gaps apart.
         const u32 start = (u32)(r.i0 + c * EASY_CHUNK), end = (u32)pc_min(r.ih, (u64)start + EASY_CHUNK);
         u64 sum = 0;
         u32 k = 0;
-        for (u32 i = start + lane; i < end; i += 32, k++)
-            sum += pi_lookup(A.pit, div_rcp(xp, A.primes[i], A.primes_rcp[i]));
+        if ((xp >> 30) < A.primes[start]) {
+            const QuotOf of(xp);
+            const uint2* dv = (const uint2*)A.primes_dv;
+            for (u32 i = start + lane; i < end; i += 32, k++) {
+                const uint2 d = __ldg(dv + i);
+                sum += pi_lookup(A.pit, of.by(d, of.shift(d.x)));
+            }
+        } else {
+            for (u32 i = start + lane; i < end; i += 32, k++)
+                sum += pi_lookup(A.pit, div_rcp(xp, A.primes[i], A.primes_rcp[i]));
+        }
         s += (i64)sum - (i64)k * ((i64)b - 2);
         n_table += k;
         return;
@@ -345,43 +354,53 @@ __device__ __forceinline__ void easy_chunk(const LeafArgs& A, u64 x, u64 a, u64 
         if (MODE == PI_ODD && cc == 0) {
             // Clustered chunk by pi value.  With G(l) = the number of clustered q (prime
             // indices [im, i1)) with q <= (x/p_b)/p_l, exactly G(l) - G(l + 1) of them have
-            // pi(x/(p_b q)) = l, each adding l - b + 2.  Lane k takes l = base + k; lanes 0..30
-            // take their G(l + 1) from the next lane, so a pass covers 31 values of l, and
-            // each G costs one division (p_l's record, read coalesced) and one pi lookup.
+            // pi(x/(p_b q)) = l, each adding l - b + 2.  Summed by parts over the chunk's
+            // l = lbase .. lend, that is
+            //   sum_{l = lbase}^{lend + 1} G(l) + (lbase - b + 1) G(lbase) - (lend - b + 3) G(lend + 1),
+            // so a lane only adds up its own G's, and each G costs one division (p_l's record,
+            // read coalesced) and one pi lookup.
             const u32 lbase = r.l0 + (u32)(c - nsp) * CLUST_L;
             const u32 lend = (u32)pc_min((u64)r.l1, (u64)lbase + CLUST_L - 1);   // inclusive
-            const u32 im = (u32)r.im, nq = (u32)(r.i1 - r.im);
-            const u64 qlast = A.primes[r.i1 - 1];
-            // sum over the lane's l of n_l * l; the - (b - 2) n_l part is added per chunk, from
-            // sum n_l = G(lbase) - G(lend + 1) (the differences telescope)
-            u64 nl = 0;
-            u32 g_first = 0, g_last = 0;
-            for (u32 l0 = lbase; l0 <= lend; l0 += 31) {
-                const u32 l = l0 + lane;
-                u32 G = 0;
-                if (l <= lend + 1) {   // p_l's record exists: l <= l1 + 1 <= pi(y) + 1
-                    // (x/p_b)/p_l < 2.3 y < 2^31; below qlast <= y it is inside the pi table
-                    const u32 v = div_dv(xp, A.primes_dv[l]);
-                    if (v >= qlast) {
-                        G = nq;
-                    } else {
-                        const i32 k = (i32)pi_odd(A.podd, v) - (i32)im + 1;   // v >= q_im / 2 >= 2
-                        G = k <= 0 ? 0u : ((u32)k > nq ? nq : (u32)k);
+            const u32 qlast1 = A.primes[r.i1 - 1] + 1;
+            // The lookup is clamped to the last q, where G is the number of all clustered q.
+            // v = (x/p_b)/p_l is at least the first q up to l = l1, and below it at l1 + 1 (G = 0).
+            // An estimate short by more than one needs v >= 2^30 > qlast: the clamp again.
+            const QuotOf of(xp);
+            const uint2* dv = (const uint2*)A.primes_dv;   // p_l's record exists: l <= l1 + 1 <= pi(y) + 1
+            const i32 g0 = 1 - (i32)r.im;
+            auto G_of = [&](u32 l, u32 sh, uint2 d) -> u32 {
+                const u32 v1 = of.by(d, sh) + 1;
+                return (u32)max((i32)pi_odd1(A.podd, v1 < qlast1 ? v1 : qlast1) + g0, 0);
+            };
+            u32 sum = 0;   // up to CLUST_L / 32 + 1 values below pi(2^29) < 2^24.8: no overflow
+            if (lend - lbase >= 32) {   // whole passes; inside one, no end of the chunk but lane 0's
+                const u32 sh0 = of.shift((u32)A.primes[lbase]), sh1 = of.shift((u32)A.primes[lend]);
+                if (sh0 == sh1) {
+#pragma unroll 4
+                    for (u32 l = lbase + 1 + lane; l <= lend; l += 32) sum += G_of(l, sh0, __ldg(dv + l));
+                } else {
+                    for (u32 l = lbase + 1 + lane; l <= lend; l += 32) {
+                        const uint2 d = __ldg(dv + l);
+                        sum += G_of(l, of.shift(d.x), d);
                     }
                 }
-                const u32 Gn = __shfl_down_sync(0xffffffffu, G, 1);
-                if (lane < 31 && l <= lend) nl += (u64)(G - Gn) * l;
-                if (l0 == lbase && lane == 0) g_first = G;
-                if (l == lend + 1) g_last = G;
+            } else if (lbase + 1 + lane <= lend) {
+                const uint2 d = __ldg(dv + lbase + 1 + lane);
+                sum = G_of(lbase + 1 + lane, of.shift(d.x), d);
             }
-            // G(lbase) sits in lane 0, G(lend + 1) in the lane that computed it
-            const u32 gsum = __reduce_add_sync(0xffffffffu, g_last);
-            const u32 leaves = __shfl_sync(0xffffffffu, g_first, 0) - gsum;
-            s += (i64)nl;
-            if (lane == 0) {
-                s -= (i64)leaves * ((i64)b - 2);
-                n_runs += lend - lbase + 1;   // pi values taken
-                n_run_leaves += leaves;
+            s += sum;
+            if (lane < 2) {   // the two ends, which the passes above leave out
+                const u32 l = lane ? lend + 1 : lbase;
+                const uint2 d = __ldg(dv + l);
+                const u32 G = G_of(l, of.shift(d.x), d);
+                if (lane == 0) {
+                    s += ((i64)lbase - (i64)b + 2) * (i64)G;
+                    n_runs += lend - lbase + 1;   // pi values taken
+                    n_run_leaves += G;
+                } else {
+                    s -= ((i64)lend - (i64)b + 2) * (i64)G;
+                    n_run_leaves -= G;   // the lanes' counters are added up mod 2^32
+                }
             }
             return;
         }
@@ -437,9 +456,20 @@ __device__ __forceinline__ void easy_chunk(const LeafArgs& A, u64 x, u64 a, u64 
     const u32 end = (u32)pc_min(r.im, (u64)start + EASY_CHUNK);
     if (MODE == PI_ODD && r.src) {
         // m = q prime: every leaf adds pi(u) - b + 2
-        u64 sum = 0;
-        u32 k = 0;
-        for (u32 i = start + lane; i < end; i += 32, k++) sum += pi_odd(A.podd, div_dv(xp, A.primes_dv[i]));
+        const QuotOf of(xp);
+        const uint2* dv = (const uint2*)A.primes_dv;
+        const u32 sh0 = of.shift((u32)A.primes[start]), sh1 = of.shift((u32)A.primes[end - 1]);
+        u32 sum = 0;   // EASY_CHUNK / 32 values below pi(2^29) < 2^24.8: no overflow
+        if (sh0 == sh1) {
+#pragma unroll 4
+            for (u32 i = start + lane; i < end; i += 32) sum += pi_odd1(A.podd, of.by(__ldg(dv + i), sh0) + 1);
+        } else {   // a chunk across a power of two
+            for (u32 i = start + lane; i < end; i += 32) {
+                const uint2 d = __ldg(dv + i);
+                sum += pi_odd1(A.podd, of.by(d, of.shift(d.x)) + 1);
+            }
+        }
+        const u32 k = start + lane < end ? (end - start - lane + 31) / 32 : 0;   // this lane's leaves
         s += (i64)sum - (i64)k * ((i64)b - 2);
         n_one += k;
         return;

@@ -257,7 +257,8 @@ __global__ void dv_kernel(const u32* d, u64 n, u64* dv)
     if (i < n) dv[i] = pc_dv(d[i]);
 }
 
-// odd-number pi table (pi_odd) over [0, 64 n): a thread per odd number 2t + 1,
+// odd-number pi table (pi_odd), n records (the last may lie past the pi table: only its
+// count, pi of the table's limit, is read then): a thread per odd number 2t + 1,
 // a warp per record (blocks of 256 threads keep a record in one warp)
 __global__ void pi_odd_kernel(PiTable pit, u64 n, uint2* out)
 {
@@ -274,13 +275,13 @@ __global__ void pi_odd_kernel(PiTable pit, u64 n, uint2* out)
         }
     }
     const u32 bits = __ballot_sync(0xffffffffu, prime);
-    if ((threadIdx.x & 31) == 0 && w < n) out[w] = make_uint2(bits, w ? (u32)pi_lookup(pit, 64 * w - 1) : 0u);
+    if ((threadIdx.x & 31) == 0 && w < n) out[w] = make_uint2(bits, w ? (u32)pi_lookup(pit, pc_min(64 * w - 1, pit.limit)) : 0u);
 }
 
 static int build_pi_odd(pc_ctx* ctx, u64 limit)
 {
     Tables& T = ctx->T;
-    const u64 n = limit / 64 + 1;
+    const u64 n = (limit + 1) / 64 + 1;   // u = 64 w - 1 reads record w
     PC_TRY(buf_reserve(ctx, T.pi_odd, n * sizeof(uint2)));
     pi_odd_kernel<<<(unsigned)((32 * n + 255) / 256), 256, 0, ctx->stream>>>(T.pi(), n, T.pi_odd.as<uint2>());
     PC_LAUNCHED(ctx);

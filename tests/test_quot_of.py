@@ -1,0 +1,50 @@
+"""The arithmetic of the one-product quotient of the easy leaves, on CPU.
+
+This restates in Python the formula of QuotOf (pc_common.cuh), not the kernel: the kernels'
+results are checked on the GPU by the pi(x) and leaf-sum parity tests.  For a dividend n with
+k = max(0, bits - 32), T = floor(n / 2^k), and a divisor d with s = floor(log2 d),
+v = floor((2^(32+s) - 1) / d), the estimate floor(floor(T v / 2^32) / 2^(s-k)) is the quotient
+or one less below 2^30, s >= k there, and the remainder's low 32 bits settle it.  From 2^30 up
+to 2^31 (a clustered run's bound, clamped to q < 2^29) it may fall short by two."""
+import random
+
+import pytest
+
+
+def estimate(n, d):
+    k = max(0, n.bit_length() - 32)
+    s = d.bit_length() - 1
+    v = ((1 << (32 + s)) - 1) // d
+    assert s >= k, (n, d)
+    return (((n >> k) * v) >> 32) >> (s - k)
+
+
+def quot(n, d):
+    q = estimate(n, d)
+    r = ((n & 0xFFFFFFFF) - q * d) & 0xFFFFFFFF
+    return q + (r >= d)
+
+
+def check(n, d):
+    want = n // d
+    if want < 1 << 30:
+        assert estimate(n, d) in (want - 1, want), (n, d)
+        assert quot(n, d) == want, (n, d)
+    else:
+        assert want - 2 <= estimate(n, d) <= want, (n, d)
+        assert quot(n, d) >= 1 << 29
+
+
+@pytest.mark.parametrize("dbits", [2, 3, 13, 22, 29, 30])
+def test_quotients(dbits):
+    rng = random.Random(dbits)
+    ds = [(1 << dbits) - 1, 1 << (dbits - 1), (1 << (dbits - 1)) + 1]
+    ds += [rng.randrange(1 << (dbits - 1), 1 << dbits) for _ in range(400)]
+    for d in ds:
+        qs = [0, 1, 2, (1 << 30) - 1, 1 << 30, (1 << 30) + 1, (1 << 31) - 3]
+        qs += [rng.randrange(1, 1 << rng.randrange(1, 31)) for _ in range(60)]
+        qs += [((1 << e) // d) + o for e in range(31, 61) for o in (-1, 0, 1)]   # n around a power of two
+        for q in qs:
+            for r in (0, 1, d // 2, d - 1):
+                if 0 <= q < (1 << 31) - 2 and 0 < q * d + r < 1 << 63:
+                    check(q * d + r, d)
