@@ -130,6 +130,19 @@ struct QuotOf {
     __device__ __forceinline__ u32 shift(u32 d) const { return (31u - (u32)__clz((int)d)) - k; }
 };
 
+// floor(n / d) for n < 2^18 d and any 32-bit d, v = floor((2^(32+s) - 1) / d), s = floor(log2 d):
+// with k = max(0, s - 13), T = floor(n / 2^k) < 2^32 and floor(T v / 2^(32+s-k)) falls short of
+// n/d by less than n / 2^(32+s) + 2^k / d < 2^-13 + 2^-13: it is the quotient or one less.
+// (The offset of a leaf's u inside a warp's sub-range of 30 * 8192 integers.)
+__device__ __forceinline__ u32 div_near(u64 n, u32 d, u32 v, bool d31)   // d31: d < 2^31
+{
+    const int s = 31 - __clz((int)d);
+    const int k = s > 13 ? s - 13 : 0;
+    const u32 q = __umulhi((u32)(n >> k), v) >> (s - k);
+    if (d31) return q + ((u32)n - q * d >= d ? 1u : 0u);   // the remainder is below 2^32
+    return q + (n - (u64)q * d >= d ? 1u : 0u);
+}
+
 PC_HD u64 pc_dv(u32 d)
 {
     if (d == 0) return 0;
@@ -212,6 +225,7 @@ struct MList {
     const u32* info;
     const u32* gpf;   // prime index of the greatest prime factor
     const u64* rcp;   // floor((2^64 - 1) / m)
+    const uint4* rec; // m, its 32-bit reciprocal (pc_dv), info, gpf: one load per entry
     u64 n;
     u64 limit;        // every squarefree m <= limit with lpf(m) > p_cmin is listed
     u32 cmin;

@@ -87,11 +87,11 @@ extern "C" void pc_destroy(pc_ctx* ctx)
     if (!ctx->borrowed) {
         Tables& T = ctx->T;
         DevBuf* tabs[] = {&T.small_primes, &T.pi_rec, &T.primes, &T.primes_rcp, &T.ml_m, &T.ml_info,
-                          &T.ml_gpf, &T.ml_rcp, &T.rank_bits, &T.rank_cnt, &T.samp, &T.primes_dv, &T.pi_odd, &T.wheel19};
+                          &T.ml_gpf, &T.ml_rcp, &T.ml_rec, &T.rank_bits, &T.rank_cnt, &T.samp, &T.primes_dv, &T.pi_odd, &T.wheel19, &T.pat16};
         for (DevBuf* b : tabs) buf_free(*b);
         for (int c = 0; c < 8; c++) buf_free(T.phiT[c]);
         for (int k = 0; k < Tables::NSUB; k++) {
-            DevBuf* sb[] = {&T.sl_m[k], &T.sl_info[k], &T.sl_gpf[k], &T.sl_rcp[k], &T.sl_bits[k], &T.sl_cnt[k]};
+            DevBuf* sb[] = {&T.sl_rec[k], &T.sl_rcp[k], &T.sl_bits[k], &T.sl_cnt[k]};
             for (DevBuf* b : sb) buf_free(*b);
         }
     }

@@ -47,12 +47,13 @@
 #include "pc_sieve.cuh"
 
 static constexpr u32 BATCH = 64;
-// below this a warp crosses off whole wheel rounds per lane and recounts its blocks after;
-// from here on lanes take (class, round) pairs and decrement the block counters (64 against
-// 128: S2_hard(1e18) kernel 66.3 -> 65.0 ms)
-static constexpr u32 RECOUNT_P = 64;
-static constexpr u32 GROUP_P = 128;     // smallest prime crossed off in groups of leaf-free steps
-static_assert(GROUP_P >= RECOUNT_P, "grouped steps keep their block counters up to date");
+// below this (PATTERN_P) a warp ANDs its sub-range with the prime's periodic pattern, 16 bytes a
+// lane, and counts its blocks in the same pass; from here on lanes cross off (class, round) pairs
+static_assert(PATTERN_P <= 64, "pattern primes are below 64");
+// Block counters serve the leaves only.  A warp whose batch has few leaf steps lets them go
+// stale and counts its blocks again at each leaf step (RECOUNT_COST: measured against the decrements),
+// rather than decrement them at every crossing (about 5 instructions a pass of 32).
+static constexpr u32 RECOUNT_COST = 160;
 static constexpr u32 MAX_NW = 16;       // warps (sub-ranges) per segment
 static constexpr u32 MAX_SUB = 8192;    // bytes per sub-range: up to 256 blocks of 256 bits
 static constexpr u32 MAX_SEG = 131072;  // bytes per segment
@@ -95,6 +96,8 @@ struct HardArgs {
     u32 nsl;
     const u32* primes;
     const u64* primes_rcp;
+    const uint2* primes_dv;   // p_k and its 32-bit reciprocal (pc_dv)
+    const uint4* pat;     // patterns of the primes 7 .. 61 (Tables::pat16)
     const u32* segB;
     const u64* rcp_seg;   // per segment: reciprocals of L_s and L_s + span (0 for L = 0)
     const u64* off;
@@ -116,15 +119,13 @@ struct __align__(16) StepInfo {
     u64 vp;        // floor((2^64 - 1) / p_b)
     u32 p;
     u32 r0;        // L mod p_b
-    u32 coff[8];   // floor(p * R8[j] / 30): byte offset of class j inside a wheel round
     u8 cbit[8];    // bit of class j inside its byte
     u32 flags;     // bit 0: leaves are primes, bit 1: step has leaves, bits 2-4: m-list (0 = all, k = sub-list k-1),
-                   // bit 5: p >= GROUP_P and p^3 > the last integer of the segment (see group_cross),
-                   // bit 6: bit 5 and p >= the sub-range's bytes >> RUN_SHIFT (see sparse_runs)
+                   // bit 6: p^3 > the last integer of the segment and p >= the sub-range's bytes >> RUN_SHIFT
+                   // (see sparse_runs)
     u32 pself;     // segment bit of p_b itself, or ~0
     u32 row;       // off - rlo of b, mod 2^32: the count / tally rows' entry of segment s is row + s
     u32 runcap;    // bit 6: bound of the step's log entries, 8 ceil(sub_bytes / p) + 1
-    u32 pad[2];
 };
 
 // leaf range of prime b in the segment [L, L + span): m in (mlo, mhi], u >= p_b^2.
@@ -140,14 +141,14 @@ __device__ __forceinline__ bool leaf_window(const HardArgs& A, u64 p, u64 vp, u6
 }
 
 // A warp owns its sub-range, so crossing off one prime needs no atomics on
-// the bitset.  For p < RECOUNT_P (64) the lanes take whole wheel rounds (30 p
-// integers, p bytes), even rounds first, then odd ones, so lanes of one pass
-// touch words at least 2p bytes apart; for larger p a lane takes one residue
-// class in every fourth round, and two of its crossings by different lanes are
-// at least 4 bytes apart (classes of one round are >= floor(2p/30) bytes apart,
-// neighbouring rounds >= p - floor(29p/30) + floor(p/30); both are >= 4 for p >= 60).  Runs of steps crossed off together (group_cross) mix
-// primes in one pass and use atomics on the words.  Block counters take
-// shared-memory atomics, since lanes of one pass may share a block.
+// the bitset.  For p < PATTERN_P the lanes AND 16 bytes each with the prime's
+// pattern; for larger p a lane takes one residue class in every fourth wheel
+// round (30 p integers, p bytes) and reads and writes single bytes: two
+// multiples of p with cofactors coprime to 30 differ by at least 2p > 30, so no
+// two crossings share a byte.  Block counters take shared-memory atomics, since
+// lanes of one pass may share a block.  (S2_hard(10^18), y = 2*10^7: this kernel 54.2 -> 45.9 ms
+// against whole rounds per lane below 64, word accesses, counters decremented at every
+// crossing and grouped steps of four primes; issue-bound, 59 % of cycles, 16 warps per SM.)
 // Instantiated for several (threads, resident CTAs) launch bounds: fewer
 // registers per thread buy more resident warps to hide shared-memory latency.
 // A launch over the segments of many queries (the batched form): item g is segment
@@ -176,9 +177,8 @@ __global__ void __launch_bounds__(MAXT, MINB) hard_sieve_kernel(HardArgs A0, Mul
     u32* I = (u32*)(pre + nw * nbw);               // BATCH * (nw + 1)
     u32* cw = I + BATCH * (nw + 1);                // BATCH * nw
     i32* tw = (i32*)(cw + BATCH * nw);             // BATCH * nw
-    i32* basew = tw + BATCH * nw;                  // BATCH * nw
-    u8* kmodw = (u8*)(basew + BATCH * nw);         // BATCH * nw
-    u16* hitlog = (u16*)(kmodw + BATCH * nw);      // nw * LOG_CAP
+    u16* first = (u16*)(tw + BATCH * nw);          // BATCH * nw * 8: first byte of class j, or >= sub_bytes
+    u16* hitlog = first + BATCH * nw * 8;          // nw * LOG_CAP
 
     __shared__ u32 patw[80];
     __shared__ u32 prev[MAX_NW];
@@ -186,23 +186,18 @@ __global__ void __launch_bounds__(MAXT, MINB) hard_sieve_kernel(HardArgs A0, Mul
     __shared__ u32 s_item;
     __shared__ i128 red[32];
     // the m-lists a step may read its leaves from: index 0 the whole list, k the sub-list k-1
-    __shared__ const u32* lst_info[1 + Tables::NSUB];
-    __shared__ const u32* lst_m[1 + Tables::NSUB];
-    __shared__ const u32* lst_gpf[1 + Tables::NSUB];
-    __shared__ const u64* lst_rcp[1 + Tables::NSUB];
+    __shared__ const uint4* lst_rec[1 + Tables::NSUB];
     __shared__ RankTable lst_rank[1 + Tables::NSUB];
 
     const u32 tid = threadIdx.x, lane = tid & 31, w = tid >> 5, NT = blockDim.x;
     make_pattern_words(patw, A0.k0);
     if (tid <= Tables::NSUB) {
         const MList& l = tid == 0 ? A0.ml : A0.sl[tid - 1];
-        lst_info[tid] = l.info;
-        lst_m[tid] = l.m;
-        lst_gpf[tid] = l.gpf;
-        lst_rcp[tid] = l.rcp;
+        lst_rec[tid] = l.rec;
         lst_rank[tid] = tid == 0 ? A0.rk : A0.srk[tid - 1];
     }
     u32* my = bits + w * sub_words;
+    u8* myb = (u8*)my;
     const u64* my64 = (const u64*)my;
     u16* myblk = blk + w * nbw;
     u32* myblk32 = (u32*)myblk;
@@ -225,7 +220,8 @@ __global__ void __launch_bounds__(MAXT, MINB) hard_sieve_kernel(HardArgs A0, Mul
         return tot;
     };
     i64 acc = 0;
-    unsigned long long nleaves = 0, nclears = 0, nbusy = 0, nleafy = 0;
+    unsigned long long nbusy = 0, nleafy = 0;
+    u32 nleaves = 0, nclears = 0;   // a lane's share of a launch stays far below 2^32
 
     __shared__ __align__(16) unsigned char sA_raw[MULTI ? sizeof(HardArgs) : 16];
     __shared__ u32 s_q;
@@ -314,6 +310,7 @@ __global__ void __launch_bounds__(MAXT, MINB) hard_sieve_kernel(HardArgs A0, Mul
         __syncthreads();
         u32 cnt = __reduce_add_sync(0xffffffffu, count_blocks());
         if (lane == 0) prev[w] = cnt;
+        bool stale = false;   // the warp's block counters lag behind its bitset
         __syncthreads();
         if (tid == 0 && b_first == A.k0 + 1) {
             u32 t = 0;
@@ -336,7 +333,7 @@ __global__ void __launch_bounds__(MAXT, MINB) hard_sieve_kernel(HardArgs A0, Mul
                 si.q = div_rcp(L, p, vp);
                 si.r0 = (u32)(L - si.q * p);
                 si.row = (u32)A.off[b - A.k0] - A.rlo[b - A.k0];
-                si.runcap = si.pad[0] = si.pad[1] = 0;
+                si.runcap = 0;
                 si.flags = 0;
                 si.mlo = si.mhi = 0;
                 si.pself = (p >= L && p < L + A.span) ? seg_pos(p, L) : ~0u;
@@ -347,22 +344,16 @@ __global__ void __launch_bounds__(MAXT, MINB) hard_sieve_kernel(HardArgs A0, Mul
                         if (A.slK[k] <= b) li = k + 1;
                     si.flags = 2u | (p * p > A.y ? 1u : 0u) | (li << 2);
                 }
-                if (p >= GROUP_P && p * p > div_rcp(L + A.span - 1, p, vp)) {
-                    si.flags |= 32u;
-                    if (p >= (A.sub_bytes >> RUN_SHIFT)) {
-                        si.flags |= 64u;
-                        si.runcap = 8 * ((A.sub_bytes + (u32)p - 1) / (u32)p) + 1;
-                    }
+                if (p >= (A.sub_bytes >> RUN_SHIFT) && p * p > div_rcp(L + A.span - 1, p, vp)) {
+                    si.flags |= 64u;
+                    si.runcap = 8 * ((A.sub_bytes + (u32)p - 1) / (u32)p) + 1;
                 }
-                for (int j = 0; j < 8; j++) {
-                    const u32 pr = (u32)p * r8(j);
-                    si.coff[j] = pr / 30;
-                    si.cbit[j] = (u8)idx30(pr % 30);
-                }
+                const u32 p30 = (u32)p % 30;
+                for (int j = 0; j < 8; j++) si.cbit[j] = (u8)idx30(p30 * r8(j) % 30);
                 st[t] = si;
             }
             __syncthreads();
-            // B: leaf index boundaries of every sub-range, and first wheel rounds
+            // B: leaf index boundaries of every sub-range, and the first multiples in it
             for (u32 idx = tid; idx < nb * (nw + 1); idx += NT) {
                 const u32 t = idx / (nw + 1), k = idx - t * (nw + 1);
                 const StepInfo& si = st[t];
@@ -384,50 +375,51 @@ __global__ void __launch_bounds__(MAXT, MINB) hard_sieve_kernel(HardArgs A0, Mul
             for (u32 idx = tid; idx < nb * nw; idx += NT) {
                 const u32 t = idx / nw, k = idx - t * nw;
                 const StepInfo& si = st[t];
-                if (bb + t >= Bs) continue;
+                if (bb + t >= Bs || si.p < PATTERN_P) continue;
                 const u64 p = si.p;
                 u64 klo = si.q + div_rcp((u64)si.r0 + k * A.dspan + p - 1, p, si.vp);   // ceil(L_k / p)
                 if (klo < p) klo = p;
                 const u64 qa = klo / 30;
                 const u32 kmod = (u32)(klo - 30 * qa);
-                i64 base = (i64)(p * qa) - (i64)(L / 30 + (u64)k * sub_bytes);
-                if (p >= 128 && base < (i64)sub_bytes) {
-                    // a large prime often has no multiple in the sub-range although a
-                    // wheel round overlaps it: look at the first multiple of every class
-                    i64 first = (i64)sub_bytes;
+                // the wheel round of klo starts at byte base of the sub-range (negative when it
+                // began before it); every class's first multiple k p >= klo p is at or after 0
+                const i64 base64 = (i64)(p * qa) - (i64)(L / 30 + (u64)k * sub_bytes);
+                const i32 base = base64 > (i64)sub_bytes ? (i32)sub_bytes : (i32)base64;
+                u32 f[8];
 #pragma unroll
-                    for (u32 j = 0; j < 8; j++) {
-                        const i64 fj = base + (i64)si.coff[j] + (r8(j) < kmod ? (i64)p : 0);
-                        first = fj < first ? fj : first;
-                    }
-                    if (first >= (i64)sub_bytes) base = sub_bytes;
+                for (u32 j = 0; j < 8; j++) {
+                    const i32 fj = base + (i32)((u32)p * r8(j) / 30) + (r8(j) < kmod ? (i32)p : 0);
+                    f[j] = (u32)min(fj, (i32)sub_bytes);
                 }
-                basew[idx] = base > (i64)sub_bytes ? (i32)sub_bytes : (i32)base;
-                kmodw[idx] = (u8)kmod;
+                *(uint4*)(first + 8 * idx) = make_uint4(f[0] | f[1] << 16, f[2] | f[3] << 16, f[4] | f[5] << 16,
+                                                        f[6] | f[7] << 16);
             }
             __syncthreads();
-            // C: every warp runs the batch over its own sub-range.  Steps that touch
-            // neither its leaves nor its integers are skipped: the warp marks its
-            // busy steps (and those with leaves, and those it may cross off in a
-            // group) with ballots and fills the skipped counts afterwards.
+            // C: every warp runs the batch over its own sub-range.  It marks its steps with
+            // leaves (and, for the counters, those with work at all) with ballots.
             auto leaf_range = [&](u32 t, u32& j0, u32& j1) {
                 j0 = I[t * (nw + 1) + w + 1];
                 j1 = I[t * (nw + 1) + w];
             };
-            u64 busy = 0, leafy = 0, grp = 0, sparse = 0;
+            u64 busy = 0, leafy = 0, sparse = 0;
             u32 lj0[BATCH / 32], lj1[BATCH / 32];   // leaf range of step h*32 + lane
 #pragma unroll
             for (u32 h = 0; h < BATCH / 32; h++) {
                 const u32 t = h * 32 + lane;
-                bool on = false, g = false, sq = false;
+                bool on = false, sq = false;
                 lj0[h] = lj1[h] = 0;
                 if (t < nb) {
                     const u32 b = bb + t, fl = st[t].flags, ps = st[t].pself;
                     sq = (fl & 64u) != 0;
                     if (b < Bs) {
-                        if (basew[t * nw + w] < (i32)sub_bytes) on = true;
+                        if (st[t].p < PATTERN_P) {
+                            on = true;
+                        } else {
+                            const uint4 f = *(const uint4*)(first + 8 * (t * nw + w));
+                            const u32 m = __vminu2(__vminu2(f.x, f.y), __vminu2(f.z, f.w));
+                            on = (m & 0xFFFFu) < sub_bytes || (m >> 16) < sub_bytes;
+                        }
                         if (ps != ~0u && (ps >> A.sub_shift) == w) on = true;
-                        g = (fl & 32u) != 0;
                     }
                     if (b > A.kleaf && (fl & 2u)) {
                         leaf_range(t, lj0[h], lj1[h]);
@@ -437,19 +429,26 @@ __global__ void __launch_bounds__(MAXT, MINB) hard_sieve_kernel(HardArgs A0, Mul
                 }
                 busy |= (u64)__ballot_sync(0xffffffffu, on) << (h * 32);
                 leafy |= (u64)__ballot_sync(0xffffffffu, lj1[h] > lj0[h]) << (h * 32);
-                grp |= (u64)__ballot_sync(0xffffffffu, g) << (h * 32);
                 sparse |= (u64)__ballot_sync(0xffffffffu, sq) << (h * 32);
             }
             // the sparse steps are a suffix of the batch (both of their conditions grow with p):
-            // steps below t_sp go one by one or in groups, the rest in runs
+            // steps below t_sp go one by one, the rest in runs
             const u32 t_sp = sparse ? (u32)__ffsll((long long)sparse) - 1 : nb;
             const u64 lomask = t_sp >= 64 ? ~0ull : (1ull << t_sp) - 1;
-            grp &= busy & ~leafy & lomask;
             // Leaf data (m, its reciprocal, lpf index and mu) does not depend on the
             // sieve, so the first 32 leaves of the next leaf step are loaded ahead,
             // while the warp is still crossing off earlier primes.
-            u32 pf_info = 0, pf_m = 0, pf_gpf = 0;
-            u64 pf_v = 0;
+            // A leaf's data is a record: m, its 32-bit reciprocal, lpf index << 1 | [mu = -1], gpf;
+            // entry i of the list of a step with these flags (a prime m: lpf = itself, mu = -1)
+            auto leaf_rec = [&](u32 fl, u32 i) -> uint4 {
+                if (fl & 1u) {
+                    const uint2 d = __ldg(A.primes_dv + i);
+                    return make_uint4(d.x, d.y, ~0u, 0u);
+                }
+                return __ldg(lst_rec[(fl >> 2) & 7u] + i);
+            };
+            const uint4 no_leaf = make_uint4(1u, 0u, 0u, 0u);   // lpf index 0: no leaf of any b
+            uint4 pf = no_leaf;
             auto leaf_bounds = [&](u32 t, u32& j0, u32& j1) {
                 const u32 h = t >> 5;
                 j0 = __shfl_sync(0xffffffffu, h ? lj0[1] : lj0[0], t & 31);
@@ -459,21 +458,17 @@ __global__ void __launch_bounds__(MAXT, MINB) hard_sieve_kernel(HardArgs A0, Mul
                 u32 j0, j1;
                 leaf_bounds(t, j0, j1);
                 const u32 i = j0 + lane;
-                pf_m = 0;
-                if (i < j1) {
-                    if (st[t].flags & 1u) {
-                        pf_info = ~0u;   // a prime: lpf = itself, mu = -1
-                        pf_m = A.primes[i];
-                        pf_v = A.primes_rcp[i];
-                        pf_gpf = 0;
-                    } else {
-                        const u32 li = (st[t].flags >> 2) & 7u;
-                        pf_info = lst_info[li][i];
-                        pf_m = lst_m[li][i];
-                        pf_v = lst_rcp[li][i];
-                        pf_gpf = A.trunc ? lst_gpf[li][i] : 0;
-                    }
-                }
+                pf = i < j1 ? leaf_rec(st[t].flags, i) : no_leaf;
+            };
+            // the count end of the leaf with record r of a step with x / p_b = xp: the bits of the
+            // sub-range up to u = xp / m.  u - Lw = floor((xp - m Lw) / m) is below the sub-range's
+            // length.  A lane without a leaf gets a small end (no_leaf: rel <= 1).
+            const u64 negL = 0 - Lw;
+            const bool m31 = !(A.y >> 31);
+            auto leaf_end = [&](u64 xp, const uint4& r) -> u32 {
+                const u32 rel = div_near(xp + r.x * negL, r.x, r.y, m31);
+                const u32 q30 = rel / 30;
+                return q30 * 8 + cntle30(rel - 30 * q30);
             };
             // prefix counts of the 256-bit blocks of the sub-range (from the block counters)
             auto block_prefix = [&]() {
@@ -516,81 +511,38 @@ __global__ void __launch_bounds__(MAXT, MINB) hard_sieve_kernel(HardArgs A0, Mul
             auto count_to = [&](u32 e) -> u32 {
                 u32 bi = e >> 8;
                 if (bi >= nbw) bi = nbw - 1;
-                // set bits of block bi below the end (0..256 of them): both halves
-                // of the block at once, no data-dependent loop.  Word i keeps its
-                // bits below rem - 64 i by a left shift of 64 (i + 1) - rem, taken
-                // as at least 0; PTX clamps a 64-bit shift above 64 to 64 (result 0).
-                const u32 rem = e - (bi << 8);
+                // set bits of block bi below the end (0..256 of them), no data-dependent loop:
+                // the whole words before the end's word, and that word's bits below the end
+                const u32 rem = e - (bi << 8), wi = rem >> 6 < 3 ? rem >> 6 : 3;
                 const ulonglong2 h0 = ((const ulonglong2*)my64)[2 * bi];
-                const ulonglong2 h1 = ((const ulonglong2*)my64)[2 * bi + 1];
-                auto part = [&](u64 wv, u32 i) -> u32 {
-                    i32 sh = (i32)(64 * i + 64) - (i32)rem;
-                    sh = sh < 0 ? 0 : (sh > 64 ? 64 : sh);
-                    u64 r;
-                    asm("shl.b64 %0, %1, %2;" : "=l"(r) : "l"(wv), "r"(sh));
-                    return __popcll(r);
-                };
-                return mypre[bi] + part(h0.x, 0) + part(h0.y, 1) + part(h1.x, 2) + part(h1.y, 3);
+                const u64 h2 = my64[4 * bi + 2], hw = my64[4 * bi + wi];
+                u32 n = mypre[bi] + __popcll(low_bits_top(hw, rem - 64 * wi));
+                if (wi > 0) n += __popcll(h0.x);
+                if (wi > 1) n += __popcll(h0.y);
+                if (wi > 2) n += __popcll(h2);
+                return n;
             };
             nbusy += __popcll(busy);
             nleafy += __popcll(leafy);
-            if (leafy & lomask) prefetch(__ffsll((long long)(leafy & lomask)) - 1);
-            __syncwarp();
-            // A run of consecutive busy steps without leaves in this sub-range, all of
-            // primes p with p >= GROUP_P and p^3 > every integer of the segment, is
-            // crossed off in one go: lane = (step of the run, residue class j), four
-            // steps per pass.  A bit still set here is 1, a prime, or a product of primes
-            // that are all >= the run's first prime; below that prime cubed it has at
-            // most two of them, so exactly one lane of the run reaches it: the one of its
-            // least prime factor q, at the cofactor n / q >= q.  That lane's decrement is
-            // therefore the one the steps would make in order, and the per-step counts
-            // follow by a prefix sum.  Lanes of different primes may share a word, hence
-            // the atomics.
-            auto group_cross = [&](u64 run) {
-                const u32 nr = __popcll(run), lo32 = (u32)run, hi32 = (u32)(run >> 32), nlo = __popc(lo32);
-                const u32 slot = lane >> 3, j = lane & 7;
-                for (u32 c = 0; c < nr; c += 4) {
-                    const u32 n = c + slot;
-                    u32 d = 0, tt = 0;
-                    if (n < nr) {
-                        tt = n < nlo ? __fns(lo32, 0, (int)n + 1) : 32 + __fns(hi32, 0, (int)(n - nlo) + 1);
-                        const i32 p = (i32)st[tt].p;
-                        const u32 kmod = kmodw[tt * nw + w];
-                        const u32 bj = st[tt].cbit[j];
-                        i32 by = basew[tt * nw + w] + (i32)st[tt].coff[j] + (r8(j) < kmod ? p : 0);
-                        for (; by < (i32)sub_bytes; by += p) {
-                            const u32 pos = ((u32)by << 3) + bj, mask = 1u << (pos & 31);
-                            const u32 hit = (atomicAnd(&my[pos >> 5], ~mask) & mask) ? 1u : 0u;
-                            d += hit;
-                            atomicSub(&myblk32[pos >> 9], hit << (16 * ((pos >> 8) & 1)));   // 0 or 1
-                            nclears++;
-                        }
-                        const u32 ps = st[tt].pself;
-                        if (j == 0 && ps != ~0u && (ps >> A.sub_shift) == w) {   // p itself
-                            const u32 pos = ps & (sub_bits - 1), mask = 1u << (pos & 31);
-                            if (atomicAnd(&my[pos >> 5], ~mask) & mask) {
-                                d++;
-                                atomicSub(&myblk32[pos >> 9], 1u << (16 * ((pos >> 8) & 1)));
-                            }
-                        }
-                    }
-                    // lanes 8s .. 8s+7 hold step c+s: an inclusive scan over the warp gives,
-                    // at lane 8s+7, the decrement of the steps up to c+s
-                    u32 incl = d;
-                    for (int o = 1; o < 32; o <<= 1) {
-                        const u32 up = __shfl_up_sync(0xffffffffu, incl, o);
-                        if (lane >= o) incl += up;
-                    }
-                    if (j == 7 && n < nr) cw[tt * nw + w] = cnt - incl;
-                    cnt -= __shfl_sync(0xffffffffu, incl, 31);
-                }
+            // counting again at each leaf step against decrementing in each pass of each step (the
+            // middle one of the batch has sub_bytes / 4p passes, at least one)
+            const u32 mid4 = 4 * st[nb >> 1].p;
+            const bool lazy = (u32)__popcll(leafy & lomask) * RECOUNT_COST * (mid4 < sub_bytes ? mid4 : sub_bytes) <
+                              (u32)__popcll(lomask) * 5u * sub_bytes;
+            auto fresh_blocks = [&]() {
+                if (!stale) return;
+                count_blocks();
+                stale = false;
                 __syncwarp();
             };
+            if (leafy & lomask) prefetch(__ffsll((long long)(leafy & lomask)) - 1);
+            __syncwarp();
             // Runs of sparse steps (p >= the sub-range's bytes >> RUN_SHIFT, so each residue
             // class has at most 2^RUN_SHIFT multiples in the sub-range, and p^3 above the
-            // segment's last integer).  As in group_cross, a bit still set when the run starts
-            // is reached by exactly one crossing of the run, that of its least prime factor, so
-            // every crossing of every step of the run is found against the bitset as it is at
+            // segment's last integer).  A bit still set when the run starts is 1, a prime, or a
+            // product of primes that are all >= the run's first prime; below that prime cubed it
+            // has at most two of them, so exactly one crossing of the run reaches it, that of its
+            // least prime factor q, at the cofactor n / q >= q.  So every crossing of every step of the run is found against the bitset as it is at
             // the run's start, in parallel: lane = (step, residue class), four steps per pass.
             // The crossings that hit a set bit go to a log, ordered by step.  A leaf of step t
             // needs the count of set bits up to u after the steps before t; that is the count on
@@ -633,7 +585,7 @@ __global__ void __launch_bounds__(MAXT, MINB) hard_sieve_kernel(HardArgs A0, Mul
                     const u32 loff = incl - n;                             // first leaf of step t0 + lane
                     // leaf g of the run: its step i (the last i < len with loff_i <= g) and its
                     // m-list data (nothing for g >= TL)
-                    auto run_leaf = [&](u32 g, u32& i, u32& info, u32& m32, u64& v, u32& gpf) {
+                    auto run_leaf = [&](u32 g, u32& i, uint4& r) {
                         i = 0;
                         for (u32 stp = 16; stp; stp >>= 1) {
                             const u32 cand = i + stp;
@@ -643,22 +595,7 @@ __global__ void __launch_bounds__(MAXT, MINB) hard_sieve_kernel(HardArgs A0, Mul
                         const u32 ji = __shfl_sync(0xffffffffu, j0, i);
                         const u32 li = __shfl_sync(0xffffffffu, loff, i);
                         const u32 fl = st[t0 + i].flags;
-                        info = 0, m32 = 0, gpf = 0;
-                        v = 0;
-                        if (g < TL) {
-                            const u32 idx = ji + (g - li);
-                            if (fl & 1u) {
-                                info = ~0u;   // a prime: lpf = itself, mu = -1
-                                m32 = A.primes[idx];
-                                v = A.primes_rcp[idx];
-                            } else {
-                                const u32 li2 = (fl >> 2) & 7u;
-                                info = lst_info[li2][idx];
-                                m32 = lst_m[li2][idx];
-                                v = lst_rcp[li2][idx];
-                                gpf = A.trunc ? lst_gpf[li2][idx] : 0;
-                            }
-                        }
+                        r = g < TL ? leaf_rec(fl, ji + (g - li)) : no_leaf;
                     };
 
                     // crossings against the starting bitset; hits logged in step order: each lane
@@ -670,7 +607,7 @@ __global__ void __launch_bounds__(MAXT, MINB) hard_sieve_kernel(HardArgs A0, Mul
                         u32 bj = 0, pp = ~0u;
                         if (i < len && bb + t < Bs) {
                             p = (i32)st[t].p;
-                            by = basew[t * nw + w] + (i32)st[t].coff[j] + (r8(j) < kmodw[t * nw + w] ? p : 0);
+                            by = (i32)first[8 * (t * nw + w) + j];
                             bj = st[t].cbit[j];
                             const u32 ps = st[t].pself;
                             if (j == 0 && ps != ~0u && (ps >> A.sub_shift) == w) pp = ps & (sub_bits - 1);   // p itself
@@ -728,28 +665,28 @@ __global__ void __launch_bounds__(MAXT, MINB) hard_sieve_kernel(HardArgs A0, Mul
                     }
                     __syncwarp();
                     if (TL) {
+                        fresh_blocks();
                         block_prefix();   // of the run's starting bitset
                         // each pass's m-list loads are issued one pass ahead (S2_hard(1e17) kernel
                         // 13.62 -> 13.30 ms with the same for steps taken one at a time)
-                        u32 ci, cinfo, cm, cgpf;
-                        u64 cv;
-                        run_leaf(lane, ci, cinfo, cm, cv, cgpf);
+                        u32 ci;
+                        uint4 cr;
+                        run_leaf(lane, ci, cr);
                         for (u32 g0 = 0; g0 < TL; g0 += 32) {
-                            u32 i, info, m32, gpf;
-                            u64 v;
-                            i = ci, info = cinfo, m32 = cm, gpf = cgpf, v = cv;
-                            if (g0 + 32 < TL) run_leaf(g0 + 32 + lane, ci, cinfo, cm, cv, cgpf);   // next pass in flight
+                            const u32 i = ci;
+                            const uint4 r = cr;
+                            if (g0 + 32 < TL) run_leaf(g0 + 32 + lane, ci, cr);   // next pass in flight
                             const u32 hi = __shfl_sync(0xffffffffu, hoff, i);
                             const u32 t = t0 + i, b = bb + t;
                             const u64 xp = st[t].xp;
-                            const bool valid = m32 && (info >> 1) > b && !(A.trunc && gpf > A.a);
-                            const u32 e = seg_count_end(div_rcp(xp, m32, v), Lw);
+                            const bool valid = (r.z >> 1) > b && !(A.trunc && r.w > A.a);
+                            const u32 e = leaf_end(xp, r);
                             u32 below = 0;   // hits of the run's earlier steps below the count end
                             for (u32 k = 0; k < hi; k++) below += lg[k] < e ? 1u : 0u;
                             const u32 cnt_u = count_to(e) - below;
-                            const i64 sg = valid ? ((info & 1u) ? 1 : -1) : 0;
-                            acc += sg * (i64)cnt_u;
-                            if (valid) atomicAdd(&tw[t * nw + w], (i32)sg);
+                            const i32 sg = valid ? ((r.z & 1u) ? 1 : -1) : 0;
+                            acc += (i64)sg * (i32)cnt_u;
+                            if (valid) atomicAdd(&tw[t * nw + w], sg);
                             nleaves += valid;
                         }
                         __syncwarp();
@@ -758,7 +695,7 @@ __global__ void __launch_bounds__(MAXT, MINB) hard_sieve_kernel(HardArgs A0, Mul
                     for (u32 k = lane; k < nent; k += 32) {
                         const u32 pos = lg[k];
                         atomicAnd(&my[pos >> 5], ~(1u << (pos & 31)));
-                        atomicSub(&myblk32[pos >> 9], 1u << (16 * ((pos >> 8) & 1)));
+                        if (!stale) atomicSub(&myblk32[pos >> 9], 1u << (16 * ((pos >> 8) & 1)));
                     }
                     const u32 hnext = __shfl_down_sync(0xffffffffu, hoff, 1);
                     if (lane < len) cw[(t0 + lane) * nw + w] = cnt - (lane + 1 < len ? hnext : nent);
@@ -767,175 +704,163 @@ __global__ void __launch_bounds__(MAXT, MINB) hard_sieve_kernel(HardArgs A0, Mul
                     t0 += len;
                 }
             };
-            const u32 cnt0 = cnt;
-            for (u64 todo = busy & lomask; todo;) {
-                const u32 t = __ffsll((long long)todo) - 1;
-                if ((grp >> t) & 1u) {
-                    // the run ends below the next busy step that is not in grp
-                    const u64 stop = busy & ~grp & (~0ull << t);
-                    const u64 run = grp & (~0ull << t) & (stop ? (stop & (0ull - stop)) - 1 : ~0ull);
-                    group_cross(run);
-                    todo &= ~run;
-                    continue;
-                }
-                todo &= todo - 1;
-                const u32 b = bb + t;
-                // the step's data, all loaded at once rather than as a chain of loads
-                const u32 fl = st[t].flags, p = st[t].p, ps = st[t].pself;
-                const i32 base = basew[t * nw + w];
-                const u32 kmod = kmodw[t * nw + w];
-                const i32 cj = (i32)st[t].coff[lane & 7];
-                const u32 bj = st[t].cbit[lane & 7];
-                if (b > A.kleaf) {
-                    int tl = 0;
-                    if ((leafy >> t) & 1u) {
-                        u32 j0, j1;
-                        leaf_bounds(t, j0, j1);
-                        block_prefix();
-                        const u64 xp = st[t].xp;
-                        auto one_leaf = [&](u32 info, u32 m32, u64 v, u32 gpf) {
-                            // no early exit: a lane without a leaf of b (no entry, lpf <= p_b, or
-                            // gpf > p_a) runs the same code and adds 0; its block index is clamped
-                            // below and its shifts to 0..64, so its reads stay inside the sub-range
-                            const bool valid = m32 && (info >> 1) > b && !(A.trunc && gpf > A.a);
-                            const bool neg = info & 1u;
-                            const u64 u = div_rcp(xp, m32, v);
-                            const u32 c = count_to(seg_count_end(u, Lw));
-                            const i64 sg = valid ? (neg ? 1 : -1) : 0;
-                            acc += sg * (i64)c;
-                            tl += (int)sg;
-                            nleaves += valid;
-                        };
-                        auto load_at = [&](u32 base, u32& info, u32& m32, u64& v, u32& gpf) {
-                            const u32 i = base + lane;
-                            info = 0, m32 = 0, gpf = 0;
-                            v = 0;
-                            if (i < j1) {
-                                if (fl & 1u) {
-                                    info = ~0u;
-                                    m32 = A.primes[i];
-                                    v = A.primes_rcp[i];
-                                } else {
-                                    const u32 li = (fl >> 2) & 7u;
-                                    info = lst_info[li][i];
-                                    m32 = lst_m[li][i];
-                                    v = lst_rcp[li][i];
-                                    gpf = A.trunc ? lst_gpf[li][i] : 0;
-                                }
-                            }
-                        };
-                        u32 ninfo = 0, nm = 0, ngpf = 0;
-                        u64 nv = 0;
-                        if (j0 + 32 < j1) load_at(j0 + 32, ninfo, nm, nv, ngpf);        // second 32 in flight
-                        one_leaf(pf_info, pf_m, pf_v, pf_gpf);                        // first 32, loaded ahead
-                        const u64 later = leafy & lomask & ~((2ull << t) - 1);
-                        if (later) prefetch(__ffsll((long long)later) - 1);           // next leaf step
-                        for (u32 base = j0 + 32; base < j1; base += 32) {             // the rest
-                            u32 info, m32, gpf;
-                            u64 v;
-                            info = ninfo, m32 = nm, gpf = ngpf, v = nv;
-                            if (base + 32 < j1) load_at(base + 32, ninfo, nm, nv, ngpf);   // next 32 in flight
-                            one_leaf(info, m32, v, gpf);
-                        }
-                        tl = __reduce_add_sync(0xffffffffu, (u32)tl);
-                        if (lane == 0) tw[t * nw + w] = tl;   // steps without leaves keep the 0 set above
+            // Crosses off the steps t0 <= t < t1, one after the other (b < Bs): lane = (class j,
+            // round offset o), four wheel rounds of p per pass, single bytes read and written.
+            // The loop runs for every step of a run without a branch on its data, its passes are
+            // counted by p alone, and the next step's data is loaded ahead: a step costs a few
+            // dozen instructions, which is what bounds the sieve where leaves are few.  With upd
+            // the block counters follow; byte y's is half (y >> 5) & 1 of word y >> 6.
+            // nf, np, nbj: the data of step t0, loaded before its leaves.
+            u32 nf = 0, np = 0, nbj = 0;
+            auto load_step = [&](u32 t) {
+                nf = first[8 * (t * nw + w) + (lane & 7)];
+                np = st[t].p;
+                nbj = st[t].cbit[lane & 7];
+            };
+            auto cross_steps = [&](u32 t0, u32 t1, bool upd) {
+                const u32 j = lane & 7, o = lane >> 3;
+                const u16* fp = first + 8 * (t0 * nw + w) + j;
+                u32* cp = cw + t0 * nw + w;
+                for (u32 t = t0; t < t1; t++, cp += nw) {
+                    const u32 p = np, bj = nbj, bm = 1u << bj, step4 = 4 * p;
+                    u32 by = nf + p * o;
+                    fp += 8 * nw;
+                    if (t + 1 < t1) {
+                        nf = *fp;
+                        np = st[t + 1].p;
+                        nbj = st[t + 1].cbit[j];
                     }
-                }
-                if (b < Bs) {
-                    const bool recount = p < RECOUNT_P;
-                    u32 dec = 0;
-                    auto clear_bit = [&](u32 pos) {   // pos: bit inside this warp's sub-range
-                        const u32 mask = 1u << (pos & 31);
-                        const u32 old = my[pos >> 5];
-                        my[pos >> 5] = old & ~mask;   // written back whether or not the bit was set
-                        const u32 hit = (old & mask) ? 1u : 0u;
-                        dec += hit;
-                        if (!recount) atomicSub(&myblk32[pos >> 9], hit << (16 * ((pos >> 8) & 1)));
-                    };
-                    {
-                        if (base < (i32)sub_bytes) {
-                            if (p >= RECOUNT_P) {
-                                // lane = (class j, round offset o): four rounds per pass.
-                                // Two crossings of one prime p >= 64 by different lanes
-                                // are >= 4 bytes apart, so no two lanes share a word.
-                                const u32 j = lane & 7, o = lane >> 3;
-                                // round o, or o + 4 when round 0 starts below the first cofactor;
-                                // every byte reached from there is >= 0 (k >= klo)
-                                const i32 step4 = 4 * (i32)p;
-                                i32 by = base + (i32)p * (i32)o + cj;
-                                if (o == 0 && r8(j) < kmod) by += step4;
-                                u32 n = 0;
-                                // two rounds at a time, both words loaded before either is written
-                                // (they are 4p bytes apart, so never the same word)
-                                for (; by + step4 < (i32)sub_bytes; by += 2 * step4, n += 2) {
-                                    const u32 pa = ((u32)by << 3) + bj, pb = ((u32)(by + step4) << 3) + bj;
-                                    const u32 ma = 1u << (pa & 31), mb = 1u << (pb & 31);
-                                    // no branch on whether the bit was still set: the word is
-                                    // written back either way and the block counter takes 0 or 1
-                                    const u32 oa = my[pa >> 5], ob = my[pb >> 5];
-                                    my[pa >> 5] = oa & ~ma;
-                                    my[pb >> 5] = ob & ~mb;
-                                    const u32 ca = (oa & ma) ? 1u : 0u, cb = (ob & mb) ? 1u : 0u;
-                                    dec += ca + cb;
-                                    atomicSub(&myblk32[pa >> 9], ca << (16 * ((pa >> 8) & 1)));
-                                    atomicSub(&myblk32[pb >> 9], cb << (16 * ((pb >> 8) & 1)));
-                                }
-                                if (by < (i32)sub_bytes) {
-                                    clear_bit(((u32)by << 3) + bj);
-                                    n++;
-                                }
-                                nclears += n;
-                            } else {
-                                const uint2 bv = *(const uint2*)st[t].cbit;
-                                const uint4 c0 = *(const uint4*)st[t].coff, c1 = *(const uint4*)(st[t].coff + 4);
-                                const u32 cw8[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
-                                // lane = whole wheel rounds, even rounds first, then odd ones.
-                                // The blocks are recounted afterwards (p < RECOUNT_P), so a bit is
-                                // simply cleared; a lane takes rounds r and r + 64 together
-                                // (64 p bytes apart: never the same word) to overlap their loads.
-                                for (u32 ph = 0; ph < 2; ph++) {
-                                    for (u32 r = 2 * lane + ph;; r += 128) {
-                                        const i32 b0 = base + (i32)(p * r);
-                                        if (b0 >= (i32)sub_bytes) break;
-                                        const i32 b1 = b0 + 64 * (i32)p;
-#pragma unroll
-                                        for (int jj = 0; jj < 8; jj++) {
-                                            const i32 by0 = b0 + (i32)cw8[jj], by1 = b1 + (i32)cw8[jj];
-                                            const bool ok0 = by0 < (i32)sub_bytes && !(r == 0 && r8(jj) < kmod);
-                                            const bool ok1 = by1 < (i32)sub_bytes;
-                                            const u32 bit = ((jj < 4 ? bv.x : bv.y) >> (8 * (jj & 3))) & 0xFFu;
-                                            const u32 q0 = ((u32)by0 << 3) + bit, q1 = ((u32)by1 << 3) + bit;
-                                            u32 w0 = 0, w1 = 0;
-                                            if (ok0) w0 = my[q0 >> 5];
-                                            if (ok1) w1 = my[q1 >> 5];
-                                            if (ok0) my[q0 >> 5] = w0 & ~(1u << (q0 & 31));
-                                            if (ok1) my[q1 >> 5] = w1 & ~(1u << (q1 & 31));
-                                            nclears += (u32)ok0 + (u32)ok1;
-                                        }
-                                    }
-                                    __syncwarp();
-                                }
+                    if (step4 >= sub_bytes) {   // one pass: at most one crossing per lane
+                        const bool in = by < sub_bytes;
+                        u32 v = 0;
+                        if (in) {
+                            v = myb[by];
+                            myb[by] = (u8)(v & ~bm);
+                            nclears++;
+                        }
+                        const bool hit = (v & bm) != 0;
+                        if (upd && hit) atomicSub(&myblk32[by >> 6], 1u << ((by >> 1) & 16));
+                        cnt -= __popc(__ballot_sync(0xffffffffu, hit));
+                    } else {
+                        // two passes at a time, both bytes loaded before either is written (4p
+                        // bytes apart).  dec: the hits times 2^bj below bit 16, the crossings above
+                        u32 dec = 0;
+                        for (u32 lim = 0; lim < sub_bytes; lim += 2 * step4, by += 2 * step4) {
+                            const u32 bz = by + step4;
+                            const bool ia = by < sub_bytes, ib = bz < sub_bytes;
+                            u32 va = 0, vb = 0;
+                            if (ia) va = myb[by];
+                            if (ib) vb = myb[bz];
+                            if (ia) myb[by] = (u8)(va & ~bm);
+                            if (ib) myb[bz] = (u8)(vb & ~bm);
+                            if (ia) dec += (va & bm) | 0x10000u;
+                            if (ib) dec += (vb & bm) | 0x10000u;
+                            if (upd) {
+                                if (va & bm) atomicSub(&myblk32[by >> 6], 1u << ((by >> 1) & 16));
+                                if (vb & bm) atomicSub(&myblk32[bz >> 6], 1u << ((bz >> 1) & 16));
                             }
                         }
+                        nclears += dec >> 16;
+                        cnt -= __reduce_add_sync(0xffffffffu, (dec & 0xFFFFu) >> bj);
                     }
                     __syncwarp();
-                    if (lane == 0 && ps != ~0u && (ps >> A.sub_shift) == w) clear_bit(ps & (sub_bits - 1));
-                    if (recount) {
+                    if (s == 0) {   // p itself (p^2 is below the segment's end: in segment 0 only)
+                        const u32 ps = st[t].pself;
+                        u32 own = 0;
+                        if (lane == 0 && ps != ~0u && (ps >> A.sub_shift) == w) {
+                            const u32 pos = ps & (sub_bits - 1), mask = 1u << (pos & 31), old = my[pos >> 5];
+                            my[pos >> 5] = old & ~mask;
+                            own = (old & mask) ? 1u : 0u;
+                            if (upd) atomicSub(&myblk32[pos >> 9], own << (16 * ((pos >> 8) & 1)));
+                        }
+                        cnt -= __shfl_sync(0xffffffffu, own, 0);
                         __syncwarp();
-                        cnt = __reduce_add_sync(0xffffffffu, count_blocks());
-                    } else {
-                        cnt -= __reduce_add_sync(0xffffffffu, dec);
                     }
+                    if (lane == 0) *cp = cnt;
                 }
+            };
+            // Step t of a prime below PATTERN_P: AND with its pattern (p itself included), 16 bytes
+            // a lane, counting the blocks on the way: lanes 2i, 2i + 1 hold the halves of a block
+            auto pattern_step = [&](u32 t) {
+                const u32 p = st[t].p;
+                const u64 g = L / 30 + (u64)w * sub_bytes + 16 * lane;
+                u32 ph = (u32)(g - div_rcp(g, p, st[t].vp) * p);
+                const u32 dph = 512 % p;
+                const uint4* pat = A.pat + (bb + t - 4) * PATTERN_P;   // p_4 = 7
+                uint4* h4 = (uint4*)my;
+                u32 tot = 0;
+                for (u32 k = lane; k < 2 * nbw; k += 32) {
+                    uint4 v = h4[k];
+                    const uint4 m = __ldg(pat + ph);
+                    v.x &= m.x, v.y &= m.y, v.z &= m.z, v.w &= m.w;
+                    h4[k] = v;
+                    u32 c = __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
+                    tot += c;
+                    c += __shfl_xor_sync(0xffffffffu, c, 1);
+                    if (!(k & 1)) myblk[k >> 1] = (u16)c;
+                    ph += dph;
+                    if (ph >= p) ph -= p;
+                }
+                cnt = __reduce_add_sync(0xffffffffu, tot);
+                stale = false;
                 if (lane == 0) cw[t * nw + w] = cnt;
                 __syncwarp();
+            };
+            // the steps below t_sp: the leaves of each step, then its crossings together with those
+            // of the leaf-free steps after it
+            const u32 t_x = Bs - bb < t_sp ? Bs - bb : t_sp;   // steps that cross off: b < Bs
+            u64 lf = leafy & lomask;
+            if (t_x) load_step(0);
+            for (u32 t = 0;;) {
+                const u32 tn = lf ? (u32)__ffsll((long long)lf) - 1 : t_sp;
+                const u32 te = tn < t_x ? tn : t_x;
+                if (t < te && np < PATTERN_P) {
+                    for (; t < te && st[t].p < PATTERN_P; t++) pattern_step(t);
+                    if (t < te) load_step(t);
+                }
+                if (t < te) {
+                    const bool upd = !(lazy || stale);
+                    stale = !upd;
+                    cross_steps(t, te, upd);
+                }
+                t = tn;
+                if (tn >= t_sp) break;
+                lf &= lf - 1;
+                if (t < t_x) load_step(t);
+                const u32 b = bb + t, fl = st[t].flags;
+                int tl = 0;
+                u32 j0, j1;
+                leaf_bounds(t, j0, j1);
+                fresh_blocks();
+                block_prefix();
+                const u64 xp = st[t].xp;
+                auto one_leaf = [&](const uint4& r) {
+                    // no early exit: a lane without a leaf of b (no entry, lpf <= p_b, or
+                    // gpf > p_a) runs the same code and adds 0; its block index is clamped
+                    // in count_to, so its reads stay inside the sub-range
+                    const bool valid = (r.z >> 1) > b && !(A.trunc && r.w > A.a);
+                    const u32 c = count_to(leaf_end(xp, r));
+                    const i32 sg = valid ? ((r.z & 1u) ? 1 : -1) : 0;
+                    acc += (i64)sg * (i32)c;
+                    tl += sg;
+                    nleaves += valid;
+                };
+                uint4 nr = no_leaf;
+                if (j0 + 32 + lane < j1) nr = leaf_rec(fl, j0 + 32 + lane);           // second 32 in flight
+                one_leaf(pf);                                                         // first 32, loaded ahead
+                if (lf) prefetch(__ffsll((long long)lf) - 1);                         // next leaf step
+                for (u32 base = j0 + 32; base < j1; base += 32) {                     // the rest
+                    const uint4 r = nr;
+                    nr = base + 32 + lane < j1 ? leaf_rec(fl, base + 32 + lane) : no_leaf;   // next 32 in flight
+                    one_leaf(r);
+                }
+                tl = __reduce_add_sync(0xffffffffu, (u32)tl);
+                if (lane == 0) tw[t * nw + w] = tl;   // steps without leaves keep the 0 set above
+                __syncwarp();   // its reads before the next step's crossings
             }
+            if (t_x < t_sp && lane == 0) cw[t_x * nw + w] = cnt;   // b = B_s: leaves only
+            __syncwarp();
             if (t_sp < nb) sparse_runs(t_sp);
-            for (u32 t = lane; t < t_sp; t += 32) {
-                if ((busy >> t) & 1u) continue;
-                const u64 before = busy & ((1ull << t) - 1);
-                cw[t * nw + w] = before ? cw[(63 - __clzll((long long)before)) * nw + w] : cnt0;
-            }
             __syncthreads();
             // D: segment rows, and the carries between the CTA's sub-ranges
             for (u32 t = tid; t < nb; t += NT) {
@@ -968,12 +893,13 @@ __global__ void __launch_bounds__(MAXT, MINB) hard_sieve_kernel(HardArgs A0, Mul
     } else {
         if (tid == 0) store_i128(A0.acc + blockIdx.x, tot);
     }
+    unsigned long long nleaves64 = nleaves, nclears64 = nclears;
     for (int o = 16; o; o >>= 1) {
-        nleaves += __shfl_xor_sync(0xffffffffu, nleaves, o);
-        nclears += __shfl_xor_sync(0xffffffffu, nclears, o);
+        nleaves64 += __shfl_xor_sync(0xffffffffu, nleaves64, o);
+        nclears64 += __shfl_xor_sync(0xffffffffu, nclears64, o);
     }
-    if (lane == 0 && nleaves) atomicAdd(A0.stat, nleaves);
-    if (lane == 0 && nclears) atomicAdd(A0.stat + 1, nclears);
+    if (lane == 0 && nleaves64) atomicAdd(A0.stat, nleaves64);
+    if (lane == 0 && nclears64) atomicAdd(A0.stat + 1, nclears64);
     if (lane == 0 && nbusy) atomicAdd(A0.stat + 2, nbusy);     // busy (warp, step) pairs
     if (lane == 0 && nleafy) atomicAdd(A0.stat + 3, nleafy);   // of which with leaves
 }
@@ -1341,7 +1267,7 @@ static size_t hard_smem(const HardArgs& A)
 {
     static_assert(sizeof(StepInfo) % 16 == 0, "StepInfo must keep 16-byte alignment");
     return BATCH * sizeof(StepInfo) + A.seg_bytes + (size_t)A.nw * (A.sub_bytes >> 5) * 4 +
-           (size_t)BATCH * (A.nw + 1) * 4 + 3 * (size_t)BATCH * A.nw * 4 + (size_t)BATCH * A.nw +
+           (size_t)BATCH * (A.nw + 1) * 4 + 2 * (size_t)BATCH * A.nw * 4 + (size_t)BATCH * A.nw * 16 +
            (size_t)A.nw * LOG_CAP * sizeof(u16);
 }
 
@@ -1456,6 +1382,8 @@ int run_hard_sieve(pc_ctx* ctx, const LeafProblem& P, I128Pair* out)
     }
     A.primes = ctx->T.primes.as<u32>();
     A.primes_rcp = ctx->T.primes_rcp.as<u64>();
+    A.primes_dv = ctx->T.primes_dv.as<uint2>();
+    A.pat = ctx->T.pat16.as<uint4>();
 
     const u64 nrows = bmax - A.k0 + 1;
     PC_TRY(buf_reserve(ctx, ctx->seg_b, A.nseg * sizeof(u32) + 2 * (nrows + 1) * sizeof(u32)));
@@ -1665,6 +1593,8 @@ int mq_hard(pc_ctx* ctx, const MQPlan& P)
     }
     T.primes = ctx->T.primes.as<u32>();
     T.primes_rcp = ctx->T.primes_rcp.as<u64>();
+    T.primes_dv = ctx->T.primes_dv.as<uint2>();
+    T.pat = ctx->T.pat16.as<uint4>();
     // per query: segments, count rows b = k0 .. bmax, carried rows b = kleaf + 1 .. bmax
     std::vector<u64> spref(Q + 1, 0), rpref(Q + 1, 0), cpref(Q + 1, 0);
     std::vector<u32> ipref(Q + 1, 0);

@@ -63,11 +63,11 @@ struct Tables {
     u64 ml_limit = 0;
     u32 ml_cmin = 99;
     u64 ml_n = 0;
-    DevBuf ml_m, ml_info, ml_gpf, ml_rcp, rank_bits, rank_cnt;
+    DevBuf ml_m, ml_info, ml_gpf, ml_rcp, ml_rec, rank_bits, rank_cnt;
     // sub-lists of the m-list: entries with lpf index > sl_K[k] (ascending K), so
     // that the leaves of a prime p_b with b >= K need not skip entries with lpf <= p_K
     static constexpr int NSUB = 4;
-    DevBuf sl_m[NSUB], sl_info[NSUB], sl_gpf[NSUB], sl_rcp[NSUB], sl_bits[NSUB], sl_cnt[NSUB];
+    DevBuf sl_rec[NSUB], sl_rcp[NSUB], sl_bits[NSUB], sl_cnt[NSUB];   // MList::rec and rcp only
     u32 sl_K[NSUB] = {0, 0, 0, 0};
     u64 sl_n[NSUB] = {0, 0, 0, 0};
     u32 n_sl = 0;
@@ -78,6 +78,9 @@ struct Tables {
     // presieve pattern of the primes 7, 11, 13, 17, 19 (WHEEL19_PERIOD bytes of the mod-30
     // bitset, then a copy of its start so that any 128 KiB slice is contiguous)
     DevBuf wheel19;
+    // patterns of the primes 7 .. 61 in the mod-30 bitset: entry (k - 4) PATTERN_P + r of p_k
+    // holds the 16 bytes from byte index g = r mod p_k on, a bit clear where p_k divides
+    DevBuf pat16;
     // odd-number pi table over [0, podd_limit] (pi_odd): one uint2 per 64 integers
     DevBuf pi_odd;
     u64 podd_limit = 0;
@@ -89,12 +92,12 @@ struct Tables {
     RankTable rank() const { return RankTable{rank_bits.as<u64>(), rank_cnt.as<u32>(), ml_limit}; }
     MList mlist() const
     {
-        return MList{ml_m.as<u32>(), ml_info.as<u32>(), ml_gpf.as<u32>(), ml_rcp.as<u64>(), ml_n, ml_limit, ml_cmin};
+        return MList{ml_m.as<u32>(), ml_info.as<u32>(), ml_gpf.as<u32>(), ml_rcp.as<u64>(),
+                     ml_rec.as<uint4>(), ml_n, ml_limit, ml_cmin};
     }
     MList sublist(int k) const
     {
-        return MList{sl_m[k].as<u32>(), sl_info[k].as<u32>(), sl_gpf[k].as<u32>(), sl_rcp[k].as<u64>(), sl_n[k],
-                     ml_limit, sl_K[k]};
+        return MList{nullptr, nullptr, nullptr, sl_rcp[k].as<u64>(), sl_rec[k].as<uint4>(), sl_n[k], ml_limit, sl_K[k]};
     }
     RankTable subrank(int k) const { return RankTable{sl_bits[k].as<u64>(), sl_cnt[k].as<u32>(), ml_limit}; }
 };
@@ -183,6 +186,9 @@ int tables_ensure(pc_ctx* ctx, u64 pi_limit, u64 prime_limit, u64 ml_limit, u32 
 // owns its tables (tables_ensure does); a no-op for one that borrows them
 static constexpr u32 WHEEL19_PERIOD = 7u * 11u * 13u * 17u * 19u;   // bytes (30 integers each)
 int tables_wheel19(pc_ctx* ctx);
+static constexpr u32 PATTERN_P = 64;          // Tables::pat16 holds the primes below
+static constexpr u32 PATTERN_PRIMES = 15;     // p_4 = 7 .. p_18 = 61
+int tables_pat16(pc_ctx* ctx);
 int tables_phi_c(pc_ctx* ctx, u32 c);   // phi(., c) residue table
 // values of pi(v) for a handful of v (v <= pi_limit), synchronizing
 int tables_pi_values(pc_ctx* ctx, const u64* v, u64* out, int n);

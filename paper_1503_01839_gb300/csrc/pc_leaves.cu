@@ -474,6 +474,24 @@ __device__ __forceinline__ void easy_chunk(const LeafArgs& A, u64 x, u64 a, u64 
         n_one += k;
         return;
     }
+    if (MODE == PI_ODD) {
+        // m from the list: a 16-byte record per entry, quotients as above
+        const QuotOf of(xp);
+        const uint4* rec = r.ls ? A.sl[r.ls - 1].rec : A.ml.rec;
+        i64 sum = 0;
+        u32 k = 0;
+#pragma unroll 2
+        for (u32 i = start + lane; i < end; i += 32) {
+            const uint4 e = __ldg(rec + i);
+            if ((e.z >> 1) <= b || (A.trunc && e.w > a)) continue;
+            const i32 t2 = (i32)pi_odd1(A.podd, of.by(make_uint2(e.x, e.y), of.shift(e.x)) + 1) - (i32)b + 2;
+            sum += e.z & 1 ? t2 : -t2;
+            k++;
+        }
+        s += sum;
+        n_one += k;
+        return;
+    }
     for (u32 i = start + lane; i < end; i += 32) {
         u64 m, v;
         bool neg = true;
@@ -482,12 +500,12 @@ __device__ __forceinline__ void easy_chunk(const LeafArgs& A, u64 x, u64 a, u64 
             v = A.primes_rcp[i];
         } else {
             const MList& ml = r.ls ? A.sl[r.ls - 1] : A.ml;
-            const u32 info = ml.info[i];
-            if ((info >> 1) <= b) continue;
-            if (A.trunc && ml.gpf[i] > a) continue;
-            m = ml.m[i];
+            const uint4 e = ml.rec[i];
+            if ((e.z >> 1) <= b) continue;
+            if (A.trunc && e.w > a) continue;
+            m = e.x;
             v = ml.rcp[i];
-            neg = info & 1;
+            neg = e.z & 1;
         }
         // easy: p_b <= u < y < 2^32; for b > 3, u >= 7 and pi(u) counts 2, 3, 5
         const u32 u = (u32)div_rcp(xp, m, v);
@@ -495,8 +513,6 @@ __device__ __forceinline__ void easy_chunk(const LeafArgs& A, u64 x, u64 a, u64 
         if (MODE == PI_SAMPLED) {
             u64 pv;
             piu = pi_sampled(A, u, &pv);
-        } else if (MODE == PI_ODD) {
-            piu = pi_odd(A.podd, u);   // u >= p_b >= 2
         } else {
             const u32 q30 = u / 30, w = q30 >> 3;
             const u32 e = 8 * (q30 & 7) + cntle30(u - 30 * q30);   // 0..64

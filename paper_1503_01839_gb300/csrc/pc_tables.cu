@@ -419,6 +419,32 @@ __global__ void wheel19_kernel(u32* words, u32 nwords)
     words[w] = v;
 }
 
+// one CTA per prime p_k, k = 4 + blockIdx.x; thread (r, word)
+__global__ void pat16_kernel(const u32* sp, u32* words)
+{
+    const u32 p = sp[blockIdx.x + 3];   // 0-based
+    const u32 r = threadIdx.x >> 2, wd = threadIdx.x & 3;
+    u32 v = 0;
+    for (u32 i = 0; i < 4; i++) {
+        const u32 g = r + 4 * wd + i;
+        for (u32 j = 0; j < 8; j++)
+            if ((30 * g + r8(j)) % p) v |= 1u << (8 * i + j);
+    }
+    if (r < p) words[(blockIdx.x * PATTERN_P + r) * 4 + wd] = v;
+}
+
+int tables_pat16(pc_ctx* ctx)
+{
+    Tables& T = ctx->T;
+    const size_t bytes = PATTERN_PRIMES * PATTERN_P * 16;
+    if (T.pat16.bytes >= bytes || ctx->borrowed) return PC_OK;
+    PC_TRY(buf_reserve(ctx, T.pat16, bytes));
+    pat16_kernel<<<PATTERN_PRIMES, 4 * PATTERN_P, 0, ctx->stream>>>(T.small_primes.as<u32>(), T.pat16.as<u32>());
+    PC_LAUNCHED(ctx);
+    ctx->stats.kernel_launches++;
+    return PC_OK;
+}
+
 int tables_wheel19(pc_ctx* ctx)
 {
     Tables& T = ctx->T;
@@ -463,18 +489,22 @@ __global__ void sub_flags_kernel(const u32* info, u64 n, u32 K, u32* flags)
     if (i < n) flags[i] = (info[i] >> 1) > K ? 1u : 0u;
 }
 
-__global__ void sub_scatter_kernel(MList src, const u32* flags, const u32* pos, u32* m, u32* info, u32* gpf, u64* rcp,
-                                   u64* bits)
+// the entries as one 16-byte record each
+__global__ void mlist_rec_kernel(MList l, uint4* rec)
+{
+    const u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < l.n) rec[i] = make_uint4(l.m[i], (u32)(pc_dv(l.m[i]) >> 32), l.info[i], l.gpf[i]);
+}
+
+__global__ void sub_scatter_kernel(MList src, const u32* flags, const u32* pos, uint4* rec, u64* rcp, u64* bits)
 {
     const u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= src.n || !flags[i]) return;
     const u32 j = pos[i];
-    const u32 mi = src.m[i];
-    m[j] = mi;
-    info[j] = src.info[i];
-    gpf[j] = src.gpf[i];
+    const uint4 r = src.rec[i];
+    rec[j] = r;
     rcp[j] = src.rcp[i];
-    atomicOr((unsigned long long*)bits + (mi >> 6), 1ull << (mi & 63));
+    atomicOr((unsigned long long*)bits + (r.x >> 6), 1ull << (r.x & 63));
 }
 
 // The entries of the m-list with lpf index > K, for a few K, each with its own
@@ -489,6 +519,10 @@ static int build_sublists(pc_ctx* ctx)
     if (n == 0) return PC_OK;
     const u64 nrw = Y / 64 + 1;
     DevBuf flags, pos, wc;
+    PC_TRY(buf_reserve(ctx, T.ml_rec, (n + 1) * sizeof(uint4)));
+    mlist_rec_kernel<<<(unsigned)((n + 255) / 256), 256, 0, ctx->stream>>>(T.mlist(), T.ml_rec.as<uint4>());
+    PC_LAUNCHED(ctx);
+    ctx->stats.kernel_launches++;
     int rc = buf_reserve(ctx, flags, (n + 1) * sizeof(u32));
     if (rc == PC_OK) rc = buf_reserve(ctx, pos, (n + 1) * sizeof(u32));
     if (rc == PC_OK) rc = buf_reserve(ctx, wc, (nrw + 1) * sizeof(u32));
@@ -501,9 +535,7 @@ static int build_sublists(pc_ctx* ctx)
         if (rc == PC_OK) rc = copy_to_host(ctx, &cnt, pos.as<u32>() + n, sizeof(u32));
         if (rc != PC_OK) break;
         const int s = T.n_sl;
-        rc = buf_reserve(ctx, T.sl_m[s], ((u64)cnt + 1) * sizeof(u32));
-        if (rc == PC_OK) rc = buf_reserve(ctx, T.sl_info[s], ((u64)cnt + 1) * sizeof(u32));
-        if (rc == PC_OK) rc = buf_reserve(ctx, T.sl_gpf[s], ((u64)cnt + 1) * sizeof(u32));
+        rc = buf_reserve(ctx, T.sl_rec[s], ((u64)cnt + 1) * sizeof(uint4));
         if (rc == PC_OK) rc = buf_reserve(ctx, T.sl_rcp[s], ((u64)cnt + 1) * sizeof(u64));
         if (rc == PC_OK) rc = buf_reserve(ctx, T.sl_bits[s], nrw * sizeof(u64));
         if (rc == PC_OK) rc = buf_reserve(ctx, T.sl_cnt[s], (nrw + 1) * sizeof(u32));
@@ -511,8 +543,8 @@ static int build_sublists(pc_ctx* ctx)
         cudaError_t e = cudaMemsetAsync(T.sl_bits[s].p, 0, nrw * sizeof(u64), ctx->stream);
         if (e == cudaSuccess) {
             sub_scatter_kernel<<<(unsigned)((n + 255) / 256), 256, 0, ctx->stream>>>(
-                T.mlist(), flags.as<u32>(), pos.as<u32>(), T.sl_m[s].as<u32>(), T.sl_info[s].as<u32>(),
-                T.sl_gpf[s].as<u32>(), T.sl_rcp[s].as<u64>(), T.sl_bits[s].as<u64>());
+                T.mlist(), flags.as<u32>(), pos.as<u32>(), T.sl_rec[s].as<uint4>(), T.sl_rcp[s].as<u64>(),
+                T.sl_bits[s].as<u64>());
             popc_words_kernel<<<(unsigned)((nrw + 255) / 256), 256, 0, ctx->stream>>>(T.sl_bits[s].as<u64>(), nrw,
                                                                                       wc.as<u32>());
             e = cudaGetLastError();
@@ -849,6 +881,7 @@ int tables_ensure(pc_ctx* ctx, u64 pi_limit, u64 prime_limit, u64 ml_limit, u32 
     }
     PC_TRY(ensure_small(ctx));
     PC_TRY(tables_wheel19(ctx));
+    PC_TRY(tables_pat16(ctx));
     bool new_pi = false;
     // The table is sieved with the bootstrap primes <= 65536, which suffice up to
     // 65536^2 = 2^32 (every query x < 2^63 needs at most isqrt(x) < 3.04e9).

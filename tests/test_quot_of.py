@@ -48,3 +48,24 @@ def test_quotients(dbits):
             for r in (0, 1, d // 2, d - 1):
                 if 0 <= q < (1 << 31) - 2 and 0 < q * d + r < 1 << 63:
                     check(q * d + r, d)
+
+
+def near(n, d):
+    s = d.bit_length() - 1
+    k = max(0, s - 13)
+    v = ((1 << (32 + s)) - 1) // d
+    t = n >> k
+    assert t < 1 << 32
+    q = ((t * v) >> 32) >> (s - k)
+    return q + (n - q * d >= d)
+
+
+@pytest.mark.parametrize("dbits", [1, 2, 13, 14, 15, 27, 31, 32])
+def test_near(dbits):
+    # div_near: quotients below 2^18, any 32-bit divisor (the offset of a leaf in a sub-range)
+    rng = random.Random(dbits)
+    lo, hi = 1 << (dbits - 1), (1 << dbits) - 1
+    for d in {lo, hi, min(lo + 1, hi)} | {rng.randrange(lo, hi + 1) for _ in range(500)}:
+        for q in [0, 1, (1 << 18) - 1, 245759] + [rng.randrange(1 << 18) for _ in range(50)]:
+            for r in {0, d // 2, d - 1}:
+                assert near(q * d + r, d) == q, (q, d, r)
