@@ -63,7 +63,8 @@ static constexpr u32 MAX_SEG = 131072;  // bytes per segment
 // leaves and thresholds of 1, 1/4 and 1/8 of the sub-range)
 static constexpr u32 RUN_SHIFT = 1;
 static constexpr u32 RUN_LEAVES = 512;             // a run ends after the step that brings its leaves to this many
-static constexpr u32 LOG_CAP = 512;                // hit log entries per warp (a run's crossings are bounded by it)
+static constexpr u32 LOG_CAP = 512;                // hit log entries per warp (a run with leaves ends before more)
+static_assert((8u << RUN_SHIFT) <= 32u && (8u << RUN_SHIFT) + 1 <= LOG_CAP, "a step's hits fit in a word and in the log");
 
 // A work item: the steps b_lo <= b < b_hi (and b <= B_s) of segment s.  A light
 // segment is one item with all its steps; a heavy one is split into replicas that
@@ -125,7 +126,7 @@ struct __align__(16) StepInfo {
                    // (see sparse_runs)
     u32 pself;     // segment bit of p_b itself, or ~0
     u32 row;       // off - rlo of b, mod 2^32: the count / tally rows' entry of segment s is row + s
-    u32 runcap;    // bit 6: bound of the step's log entries, 8 ceil(sub_bytes / p) + 1
+    u32 pad;
 };
 
 // leaf range of prime b in the segment [L, L + span): m in (mlo, mhi], u >= p_b^2.
@@ -333,7 +334,7 @@ __global__ void __launch_bounds__(MAXT, MINB) hard_sieve_kernel(HardArgs A0, Mul
                 si.q = div_rcp(L, p, vp);
                 si.r0 = (u32)(L - si.q * p);
                 si.row = (u32)A.off[b - A.k0] - A.rlo[b - A.k0];
-                si.runcap = 0;
+                si.pad = 0;
                 si.flags = 0;
                 si.mlo = si.mhi = 0;
                 si.pself = (p >= L && p < L + A.span) ? seg_pos(p, L) : ~0u;
@@ -344,10 +345,7 @@ __global__ void __launch_bounds__(MAXT, MINB) hard_sieve_kernel(HardArgs A0, Mul
                         if (A.slK[k] <= b) li = k + 1;
                     si.flags = 2u | (p * p > A.y ? 1u : 0u) | (li << 2);
                 }
-                if (p >= (A.sub_bytes >> RUN_SHIFT) && p * p > div_rcp(L + A.span - 1, p, vp)) {
-                    si.flags |= 64u;
-                    si.runcap = 8 * ((A.sub_bytes + (u32)p - 1) / (u32)p) + 1;
-                }
+                if (p >= (A.sub_bytes >> RUN_SHIFT) && p * p > div_rcp(L + A.span - 1, p, vp)) si.flags |= 64u;
                 const u32 p30 = (u32)p % 30;
                 for (int j = 0; j < 8; j++) si.cbit[j] = (u8)idx30(p30 * r8(j) % 30);
                 st[t] = si;
@@ -542,15 +540,18 @@ __global__ void __launch_bounds__(MAXT, MINB) hard_sieve_kernel(HardArgs A0, Mul
             // segment's last integer).  A bit still set when the run starts is 1, a prime, or a
             // product of primes that are all >= the run's first prime; below that prime cubed it
             // has at most two of them, so exactly one crossing of the run reaches it, that of its
-            // least prime factor q, at the cofactor n / q >= q.  So every crossing of every step of the run is found against the bitset as it is at
-            // the run's start, in parallel: lane = (step, residue class), four steps per pass.
-            // The crossings that hit a set bit go to a log, ordered by step.  A leaf of step t
-            // needs the count of set bits up to u after the steps before t; that is the count on
-            // the run's starting bitset less the logged hits of the run's steps before t below
-            // u.  So the leaves of all steps of a run share 32-lane passes, one block prefix
-            // serves the whole run, and the logged bits are cleared once at its end.  A run ends
-            // after the step that brings its leaves to RUN_LEAVES, at 32 steps, or where the
-            // log could overflow, which keeps the log scans short.
+            // least prime factor q, at the cofactor n / q >= q.  So every crossing of every step of
+            // the run is found against the bitset as it is at the run's start, a step per lane (the
+            // first bytes of its eight classes are one 16-byte load): no lane waits for another,
+            // and 32 steps without leaves cost about what two did one after the other (four steps a
+            // pass, lane = (step, class): S2_hard(10^18)'s sieve 45.9 ms, this 42.3).  The
+            // crossings that hit a set bit are cleared at once in a run without leaves; otherwise
+            // they go to a log, ordered by step.  A leaf of step t needs the count of set bits up
+            // to u after the steps before t; that is the count on the run's starting bitset less
+            // the logged hits of the run's steps before t below u.  So the leaves of all steps of a
+            // run share 32-lane passes, one block prefix serves the whole run, and the logged bits
+            // are cleared once at its end.  A run ends after the step that brings its leaves to
+            // RUN_LEAVES, at 32 steps, or where the log is full, which keeps the log scans short.
             auto sparse_runs = [&](u32 t0) {
                 while (t0 < nb) {
                     // the leaf ranges of the next (up to) 32 steps, one per lane
@@ -566,21 +567,73 @@ __global__ void __launch_bounds__(MAXT, MINB) hard_sieve_kernel(HardArgs A0, Mul
                         }
                     }
                     const u32 n = j1 - j0;   // 0 for steps without leaves in this sub-range (or share)
+                    const u32 avail = nb - t0 < 32 ? nb - t0 : 32;
+                    // crossings of step t0 + lane against the starting bitset: bit 8 m + j of hm is
+                    // set when the m-th multiple of class j hits a set bit
+                    const u16* fs = first + 8 * ((lane < avail ? ts : t0) * nw + w);
+                    const StepInfo& ss = st[lane < avail ? ts : t0];
+                    const u32 p = ss.p;
+                    u32 hm = 0, self = ~0u;
+                    if (lane < avail && bb + ts < Bs) {
+                        const uint4 f4 = *(const uint4*)fs;
+                        const uint2 c8 = *(const uint2*)ss.cbit;
+                        const u32 fw[4] = {f4.x, f4.y, f4.z, f4.w};
+#pragma unroll
+                        for (u32 j = 0; j < 8; j++) {
+                            u32 by = (fw[j >> 1] >> (16 * (j & 1))) & 0xFFFFu;
+                            const u32 bj = ((j < 4 ? c8.x : c8.y) >> (8 * (j & 3))) & 0xFFu;
+#pragma unroll
+                            for (u32 m = 0; m < (1u << RUN_SHIFT); m++, by += p) {
+                                if (by < sub_bytes) {
+                                    hm |= ((myb[by] >> bj) & 1u) << (8 * m + j);
+                                    nclears++;
+                                }
+                            }
+                        }
+                        if (s == 0) {   // p itself
+                            const u32 ps = ss.pself;
+                            if (ps != ~0u && (ps >> A.sub_shift) == w) {
+                                const u32 pos = ps & (sub_bits - 1);
+                                if ((my[pos >> 5] >> (pos & 31)) & 1u) self = pos;
+                            }
+                        }
+                    }
+                    const u32 h = __popc(hm) + (self != ~0u ? 1u : 0u);
+                    u32 hin = h;   // hits of the steps up to t0 + lane
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const u32 v = __shfl_up_sync(0xffffffffu, hin, o);
+                        if (lane >= o) hin += v;
+                    }
+                    // the bit positions of this lane's hits, one after the other
+                    auto each_hit = [&](auto&& f) {
+                        for (u32 left = hm; left; left &= left - 1) {
+                            const u32 q = __ffs(left) - 1;
+                            f(((fs[q & 7] + (q >> 3) * p) << 3) + ss.cbit[q & 7]);
+                        }
+                        if (self != ~0u) f(self);
+                    };
+                    auto clear_hit = [&](u32 pos) {
+                        atomicAnd(&my[pos >> 5], ~(1u << (pos & 31)));
+                        if (!stale) atomicSub(&myblk32[pos >> 9], 1u << (16 * ((pos >> 8) & 1)));
+                    };
+                    if (!__any_sync(0xffffffffu, n)) {
+                        __syncwarp();
+                        each_hit(clear_hit);
+                        if (lane < avail) cw[ts * nw + w] = cnt - hin;
+                        cnt -= __shfl_sync(0xffffffffu, hin, 31);
+                        __syncwarp();
+                        t0 += avail;
+                        continue;
+                    }
                     u32 incl = n;
                     for (int o = 1; o < 32; o <<= 1) {
                         const u32 v = __shfl_up_sync(0xffffffffu, incl, o);
                         if (lane >= o) incl += v;
                     }
-                    u32 cap = ts < nb ? st[ts].runcap : 0;   // log entries the step may add
-                    for (int o = 1; o < 32; o <<= 1) {
-                        const u32 v = __shfl_up_sync(0xffffffffu, cap, o);
-                        if (lane >= o) cap += v;
-                    }
-                    u32 avail = nb - t0 < 32 ? nb - t0 : 32;
-                    const u32 fits = __popc(__ballot_sync(0xffffffffu, lane < avail && cap <= LOG_CAP));
-                    if (fits < avail) avail = fits;   // at least 1: a step adds at most 8 * 2^RUN_SHIFT + 1
-                    const u32 enough = __ballot_sync(0xffffffffu, lane < avail && incl >= RUN_LEAVES);
-                    const u32 len = enough ? (u32)__ffs(enough) : avail;   // steps t0 .. t0 + len - 1
+                    // at least one step: a step has at most 8 << RUN_SHIFT hits and its own prime
+                    const u32 fits = __popc(__ballot_sync(0xffffffffu, lane < avail && hin <= LOG_CAP));
+                    const u32 enough = __ballot_sync(0xffffffffu, lane < fits && incl >= RUN_LEAVES);
+                    const u32 len = enough ? (u32)__ffs(enough) : fits;   // steps t0 .. t0 + len - 1
                     const u32 TL = __shfl_sync(0xffffffffu, incl, len - 1);
                     const u32 loff = incl - n;                             // first leaf of step t0 + lane
                     // leaf g of the run: its step i (the last i < len with loff_i <= g) and its
@@ -598,70 +651,10 @@ __global__ void __launch_bounds__(MAXT, MINB) hard_sieve_kernel(HardArgs A0, Mul
                         r = g < TL ? leaf_rec(fl, ji + (g - li)) : no_leaf;
                     };
 
-                    // crossings against the starting bitset; hits logged in step order: each lane
-                    // counts its hits, a warp scan gives its log offset, then it writes them
-                    u32 nent = 0, hoff = 0;                                // hoff: log entries before step t0 + lane
-                    for (u32 c = 0; c < len; c += 4) {
-                        const u32 sl = lane >> 3, j = lane & 7, i = c + sl, t = t0 + i;
-                        i32 by = (i32)sub_bytes, p = 0;
-                        u32 bj = 0, pp = ~0u;
-                        if (i < len && bb + t < Bs) {
-                            p = (i32)st[t].p;
-                            by = (i32)first[8 * (t * nw + w) + j];
-                            bj = st[t].cbit[j];
-                            const u32 ps = st[t].pself;
-                            if (j == 0 && ps != ~0u && (ps >> A.sub_shift) == w) pp = ps & (sub_bits - 1);   // p itself
-                        }
-                        if (st[t0 + c].p >= sub_bytes) {
-                            // every prime of the pass has at most one multiple per class in the
-                            // sub-range: hits found in one go, offsets from two ballots
-                            u32 h = 0, pa = 0, pb = 0;
-                            if (by < (i32)sub_bytes) {
-                                const u32 pos = ((u32)by << 3) + bj;
-                                nclears++;
-                                if ((my[pos >> 5] >> (pos & 31)) & 1u) {
-                                    pa = pos;
-                                    h = 1;
-                                }
-                            }
-                            if (pp != ~0u && ((my[pp >> 5] >> (pp & 31)) & 1u)) {
-                                if (h) pb = pp; else pa = pp;
-                                h++;
-                            }
-                            const u32 m1 = __ballot_sync(0xffffffffu, h >= 1), m2 = __ballot_sync(0xffffffffu, h >= 2);
-                            const u32 below = (1u << lane) - 1u;
-                            const u32 off = nent + __popc(m1 & below) + __popc(m2 & below);
-                            if (h >= 1) lg[off] = (u16)pa;
-                            if (h >= 2) lg[off + 1] = (u16)pb;
-                            const u32 first = __shfl_sync(0xffffffffu, off, ((lane - c) & 3) * 8);
-                            if (lane >= c && lane < c + 4) hoff = first;
-                            nent += __popc(m1) + __popc(m2);
-                            continue;
-                        }
-                        u32 h = 0;
-                        for (i32 q = by; q < (i32)sub_bytes; q += p) {
-                            const u32 pos = ((u32)q << 3) + bj;
-                            h += (my[pos >> 5] >> (pos & 31)) & 1u;
-                            nclears++;
-                        }
-                        if (pp != ~0u) h += (my[pp >> 5] >> (pp & 31)) & 1u;
-                        u32 hin = h;
-                        for (int o = 1; o < 32; o <<= 1) {
-                            const u32 v = __shfl_up_sync(0xffffffffu, hin, o);
-                            if (lane >= o) hin += v;
-                        }
-                        u32 off = nent + hin - h;
-                        // step c + s starts at the entry offset of lane 8 s
-                        const u32 first = __shfl_sync(0xffffffffu, off, ((lane - c) & 3) * 8);
-                        if (lane >= c && lane < c + 4) hoff = first;
-                        if (h) {
-                            for (i32 q = by; q < (i32)sub_bytes; q += p) {
-                                const u32 pos = ((u32)q << 3) + bj;
-                                if ((my[pos >> 5] >> (pos & 31)) & 1u) lg[off++] = (u16)pos;
-                            }
-                            if (pp != ~0u && ((my[pp >> 5] >> (pp & 31)) & 1u)) lg[off] = (u16)pp;
-                        }
-                        nent += __shfl_sync(0xffffffffu, hin, 31);
+                    const u32 nent = __shfl_sync(0xffffffffu, hin, len - 1), hoff = hin - h;   // log entries: all, before the step
+                    if (lane < len) {
+                        u32 off = hoff;
+                        each_hit([&](u32 pos) { lg[off++] = (u16)pos; });
                     }
                     __syncwarp();
                     if (TL) {
@@ -692,13 +685,8 @@ __global__ void __launch_bounds__(MAXT, MINB) hard_sieve_kernel(HardArgs A0, Mul
                         __syncwarp();
                     }
                     // clear the logged bits; counts after every step of the run
-                    for (u32 k = lane; k < nent; k += 32) {
-                        const u32 pos = lg[k];
-                        atomicAnd(&my[pos >> 5], ~(1u << (pos & 31)));
-                        if (!stale) atomicSub(&myblk32[pos >> 9], 1u << (16 * ((pos >> 8) & 1)));
-                    }
-                    const u32 hnext = __shfl_down_sync(0xffffffffu, hoff, 1);
-                    if (lane < len) cw[(t0 + lane) * nw + w] = cnt - (lane + 1 < len ? hnext : nent);
+                    for (u32 k = lane; k < nent; k += 32) clear_hit(lg[k]);
+                    if (lane < len) cw[(t0 + lane) * nw + w] = cnt - hin;
                     cnt -= nent;
                     __syncwarp();
                     t0 += len;
