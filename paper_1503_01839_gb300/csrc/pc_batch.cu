@@ -814,7 +814,10 @@ extern "C" int pc_tuned(pc_ctx* ctx, uint64_t x, uint32_t* alpha, uint32_t* seg_
     if (!ctx || !alpha || !seg_bytes) return PC_EINVAL;
     const int d = decimal_digits(x);
     *alpha = choose_alpha(ctx, x);
-    *seg_bytes = ctx->params.seg_bytes ? ctx->params.seg_bytes : (ctx->tuned_seg[d] ? ctx->tuned_seg[d] : 32768);
+    // y as pc_pi_count picks it (below 2^20 no sieve runs)
+    const u64 r = pc_isqrt(x), y = pc_max(pc_min((u64)*alpha * pc_iroot3(x), r), (u64)1);
+    *seg_bytes = ctx->params.seg_bytes ? ctx->params.seg_bytes
+                                       : (ctx->tuned_seg[d] ? ctx->tuned_seg[d] : hard_seg_for(x / y));
     return PC_OK;
 }
 

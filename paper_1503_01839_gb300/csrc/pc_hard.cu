@@ -1036,10 +1036,27 @@ u32 pc_seg_bytes(pc_ctx* ctx, u32 dflt)
     return sb;
 }
 
-// bytes per warp sub-range: a power of two dividing seg_bytes, at most 16 warps
-static u32 pc_sub_bytes(pc_ctx* ctx, u32 seg_bytes)
+// Geometry of the hard-leaf sieve over [0, z] for one query: segment bytes and warp sub-range
+// bytes.  A warp walks its steps one after the other (a microsecond each), so while the
+// sub-ranges are fewer than the warps the chip holds (152 x 16), smaller ones shorten the
+// chain; once they are many, larger ones do fewer steps per integer.  The lines lie where the
+// sieve's time crosses on GB300 (8 KiB / 1 KiB against 32 KiB / 8 KiB: 0.088 / 0.223 ms at
+// z = 8e5, 0.193 / 0.324 at 6e6, 0.375 / 0.565 at 9e7; 8 KiB / 2 KiB 0.53 / 0.67 at 1.4e8;
+// 16 KiB / 4 KiB 0.825 / 1.03 at 3.3e8, 2.67 / 2.75 at 1.5e9, 4.91 / 4.65 at 3e9).
+static u32 hard_sub_for(u64 z)
 {
-    u32 wb = ctx->params.warp_bytes ? ctx->params.warp_bytes : 8192;
+    return z < 120000000ull ? 1024 : z < 280000000ull ? 2048 : z < 2000000000ull ? 4096 : 8192;
+}
+
+u32 hard_seg_for(u64 z)
+{
+    return z < 400000ull ? 2048 : z < 280000000ull ? 8192 : z < 2000000000ull ? 16384 : 32768;
+}
+
+// bytes per warp sub-range: a power of two dividing seg_bytes, at most 16 warps
+static u32 pc_sub_bytes(pc_ctx* ctx, u32 seg_bytes, u32 dflt)
+{
+    u32 wb = ctx->params.warp_bytes ? ctx->params.warp_bytes : dflt;
     if (wb > MAX_SUB) wb = MAX_SUB;
     if (wb > seg_bytes) wb = seg_bytes;
     while (seg_bytes % wb) wb >>= 1;
@@ -1330,9 +1347,8 @@ int run_hard_sieve(pc_ctx* ctx, const LeafProblem& P, I128Pair* out)
     A.kleaf = P.c > A.k0 ? P.c : A.k0;
     A.a = P.a;
     A.trunc = P.trunc;
-    // 32 KiB segments of four 8 KiB warp sub-ranges: four CTAs fit on an SM
-    A.seg_bytes = pc_seg_bytes(ctx, 32768);
-    A.sub_bytes = pc_sub_bytes(ctx, A.seg_bytes);
+    A.seg_bytes = pc_seg_bytes(ctx, hard_seg_for(P.z));
+    A.sub_bytes = pc_sub_bytes(ctx, A.seg_bytes, hard_sub_for(P.z));
     A.nw = A.seg_bytes / A.sub_bytes;
     A.sub_shift = 3;
     while ((1u << A.sub_shift) < A.sub_bytes * 8) A.sub_shift++;
@@ -1564,7 +1580,7 @@ int mq_hard(pc_ctx* ctx, const MQPlan& P)
     T.k0 = 5;
     T.kleaf = 5;
     T.seg_bytes = pc_seg_bytes(ctx, ctx->batch_seg ? ctx->batch_seg : 16384);
-    T.sub_bytes = pc_sub_bytes(ctx, T.seg_bytes);
+    T.sub_bytes = pc_sub_bytes(ctx, T.seg_bytes, 8192);
     T.nw = T.seg_bytes / T.sub_bytes;
     T.sub_shift = 3;
     while ((1u << T.sub_shift) < T.sub_bytes * 8) T.sub_shift++;

@@ -290,3 +290,5 @@ struct SegGeom {
 
 // segment bytes: the context's fixed size, else the tuned one of the call, else dflt
 u32 pc_seg_bytes(pc_ctx* ctx, u32 dflt);
+// default segment bytes of the hard-leaf sieve over [0, z]
+u32 hard_seg_for(u64 z);

@@ -43,6 +43,22 @@ struct P2Args {
 // residue class); those with fewer than one round per 8 bytes by one thread
 // per prime.
 static constexpr u32 P2_COOP_P = 512;
+// In small segments the line lies lower, at 64 rounds per residue class: the CTA's threads take
+// the primes above it all at once instead of one prime after the other.
+static u32 p2_coop_p(u32 seg_bytes) { return seg_bytes / 64 < P2_COOP_P ? seg_bytes / 64 : P2_COOP_P; }
+
+// Segment bytes of P2's sieve over [0, z]: small z in small segments, so that they spread over
+// the chip's 152 SMs (kernel times on GB300 against 32 KiB: 2 KiB 0.058 / 0.174 ms at z = 6e6,
+// 0.068 / 0.215 at 2.9e7, 8 KiB 0.109 / 0.230 at 9e7, 16 KiB 0.167 / 0.285 at 1.9e8, 0.288 /
+// 0.300 at 5e8), then 32 KiB up to z = 2^30, 64 KiB up to 2^32 and 48 KiB beyond (48 KiB
+// against 64 KiB: pi(1e17) P2 2.45 -> 2.38 ms, pi(1e18) 8.9 -> 8.5 ms).
+static u32 p2_seg_for(u64 z)
+{
+    if (z < 40000000ull) return 2048;
+    if (z < 150000000ull) return 8192;
+    if (z < 700000000ull) return 16384;
+    return z < (1ull << 30) ? 32768 : z < (1ull << 32) ? 65536 : 49152;
+}
 
 // The crossing walks of pc_sieve.cuh with 32-bit offsets, for p < 2^29: a byte offset
 // below 2^17 plus p, or an integer offset below 30 * 2^17 plus 6 p, stays below 2^32.
@@ -556,15 +572,11 @@ int run_p2(pc_ctx* ctx, u64 x, u64 y, u64 a, I128Pair* out)
         A.k0 = 8;
         A.pat = ctx->T.wheel19.as<u32>();
     }
-    // 32 KiB segments up to z = 2^30, 64 KiB up to 2^32, 48 KiB beyond (measured on
-    // GB300: the small segments win by a third at z ~ 1e8 and lose a few percent at
-    // z ~ 1.5e9; 48 KiB against 64 KiB: pi(1e17) P2 2.45 -> 2.38 ms, pi(1e18) 8.9 -> 8.5 ms)
     const bool bucket = ctx->params.p2_bucket != 0;
-    A.seg_bytes = bucket ? pc_seg_bytes(ctx, 4096)
-                         : pc_seg_bytes(ctx, A.z < (1ull << 30) ? 32768 : A.z < (1ull << 32) ? 65536 : 49152);
+    A.seg_bytes = pc_seg_bytes(ctx, bucket ? 4096 : p2_seg_for(A.z));
     A.span = 30ull * A.seg_bytes;
     {
-        u64 v2[2] = {P2_COOP_P - 1, A.seg_bytes / 8}, pv2[2];
+        u64 v2[2] = {p2_coop_p(A.seg_bytes) - 1, A.seg_bytes / 8}, pv2[2];
         PC_TRY(tables_pi_values(ctx, v2, pv2, 2));
         A.b_mid = (u32)pc_min(pc_max(pv2[0] + 1, (u64)A.k0 + 1), B + 1);
         A.b_big = (u32)pc_min(pc_max(pv2[1] + 1, (u64)A.b_mid), B + 1);
