@@ -101,13 +101,17 @@ typedef struct pc_stats {
     uint32_t seg_bytes;
     uint64_t segments;      /* hard-leaf sieve segments */
     uint64_t steps;         /* (segment, prime) steps of the hard-leaf sieve */
-    uint64_t hard_leaves;   /* hard special leaves resolved by the sieve */
-    uint64_t clears;        /* multiples crossed off by the hard-leaf sieve */
+    uint64_t hard_leaves;   /* hard special leaves: those resolved by the sieve (u >= p_b^2) and those
+                               read from the pi table (u < p_b^2) */
+    uint64_t clears;        /* multiples crossed off by the hard-leaf sieve, by primes above 64 (the smaller
+                               ones are applied as bit patterns) */
     uint64_t work_items;    /* sieve work items (segments, heavy ones split into replicas) */
     uint64_t item_steps;    /* (work item, prime) steps the work items own: every (segment,
                                prime) step once, heavy segments split among replicas */
     uint64_t kernel_launches;
-    double ms_tables, ms_s1, ms_trivial, ms_easy, ms_hard, ms_p2, ms_total;
+    double ms_tables, ms_s1, ms_trivial, ms_easy, ms_hard, ms_p2, ms_total;   /* ms_s1: the ordinary and the
+                               trivial leaves (one kernel; ms_trivial stays 0).  The phases of a leaf-sum
+                               call are timed by CUDA events, ms_tables and ms_total on the host. */
     double ms_hard_sieve;   /* the segmented sieve kernel alone (CUDA events) */
     uint64_t warp_steps;      /* (warp sub-range, prime) steps with work in the hard-leaf sieve */
     uint64_t leaf_warp_steps; /* of which resolved leaves */

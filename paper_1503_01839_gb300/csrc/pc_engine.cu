@@ -79,10 +79,10 @@ extern "C" void pc_destroy(pc_ctx* ctx)
     if (ctx->stream) cudaStreamSynchronize(ctx->stream);
     workers_destroy(ctx);
     DevBuf* bufs[] = {&ctx->seg_b, &ctx->seg_off, &ctx->counts, &ctx->tallies,
-                      &ctx->acc_seg, &ctx->partials, &ctx->result, &ctx->misc, &ctx->scan_tmp, &ctx->queue,
-                      &ctx->easy_rng, &ctx->easy_chunk_off, &ctx->easy_cmap, &ctx->starts,
+                      &ctx->acc_seg, &ctx->partials, &ctx->result, &ctx->misc, &ctx->scan_tmp,
+                      &ctx->easy_rng, &ctx->easy_chunk_off, &ctx->starts,
                       &ctx->mq_q, &ctx->mq_pref, &ctx->mq_e, &ctx->mq_h, &ctx->mq_hq, &ctx->mq_p,
-                      &ctx->p2_bkt};
+                      &ctx->p2_seg, &ctx->p2_bkt};
     for (DevBuf* b : bufs) buf_free(*b);
     if (!ctx->borrowed) {
         Tables& T = ctx->T;
@@ -141,42 +141,61 @@ static void stats_begin(pc_ctx* ctx, u64 x)
     ctx->stats.x = x;
 }
 
-// Result slots 0..7 hold i128 parts; slots 8..15 (as u64) the call's counters.
-static int result_slots(pc_ctx* ctx, int n, I128Pair** d)
+// the result buffer of a call (pc_internal.h), zeroed: parts, counters and work queues
+static int result_slots(pc_ctx* ctx, I128Pair** d)
 {
-    (void)n;
-    PC_TRY(buf_reserve(ctx, ctx->result, 16 * sizeof(I128Pair)));
-    PC_CUDA(ctx, cudaMemsetAsync(ctx->result.p, 0, 16 * sizeof(I128Pair), ctx->stream));
+    PC_TRY(buf_reserve(ctx, ctx->result, RES_BYTES));
+    PC_CUDA(ctx, cudaMemsetAsync(ctx->result.p, 0, RES_BYTES, ctx->stream));
     *d = ctx->result.as<I128Pair>();
-    ctx->dstat = (unsigned long long*)(ctx->result.as<I128Pair>() + 8);
-    ctx->easy_timed = ctx->p2_timed = false;
+    ctx->dstat = call_dstat(ctx);
+    ctx->hard_timed = ctx->easy_timed = ctx->p2_timed = false;
+    ctx->marks = 0;
     return PC_OK;
 }
 
+// the end of a phase, on the call's stream
+static int mark(pc_ctx* ctx)
+{
+    PC_CUDA(ctx, cudaEventRecord(ctx->ev[6 + ctx->marks], ctx->stream));
+    ctx->marks++;
+    return PC_OK;
+}
+
+// the call's one wait for its results: parts, counters and kernel times
 static int read_slots(pc_ctx* ctx, int n, i128* out)
 {
-    I128Pair h[16];
-    PC_TRY(copy_to_host(ctx, h, ctx->result.p, 16 * sizeof(I128Pair)));
-    for (int i = 0; i < n; i++) out[i] = from_pair(h[i]);
-    const u64* c = (const u64*)(h + 8);
+    alignas(16) unsigned char h[RES_QUEUE];
+    PC_TRY(copy_to_host(ctx, h, ctx->result.p, sizeof(h)));
+    for (int i = 0; i < n; i++) out[i] = from_pair(((const I128Pair*)h)[i]);
+    const u64* c = (const u64*)(h + RES_DSTAT);
+    const u64* hs = (const u64*)(h + RES_HARD);
+    if (hs[6]) {
+        pc_set_error(ctx, "hard-leaf sieve: work items exceed the planned slots");
+        return PC_EOVERFLOW;
+    }
+    ctx->stats.hard_leaves += hs[0];
+    ctx->stats.clears += hs[1];
+    ctx->stats.warp_steps += hs[2];
+    ctx->stats.leaf_warp_steps += hs[3];
+    ctx->stats.work_items = hs[4];
+    ctx->stats.item_steps += hs[5];
+    ctx->stats.presieve_steps += hs[7];
+    if (hs[8]) ctx->stats.steps = hs[8];
     ctx->stats.easy_leaves += c[0];
     ctx->stats.easy_runs += c[1];
     ctx->stats.easy_run_leaves += c[2];
     ctx->stats.p2_clears += c[3];
     ctx->stats.hard_leaves += c[4];   // those read from the pi table
     float ms = 0;
+    if (ctx->hard_timed && cudaEventElapsedTime(&ms, ctx->ev[0], ctx->ev[1]) == cudaSuccess) ctx->stats.ms_hard_sieve += ms;
     if (ctx->easy_timed && cudaEventElapsedTime(&ms, ctx->ev[2], ctx->ev[3]) == cudaSuccess) ctx->stats.ms_easy_kernel += ms;
     if (ctx->p2_timed && cudaEventElapsedTime(&ms, ctx->ev[4], ctx->ev[5]) == cudaSuccess) ctx->stats.ms_p2_kernel += ms;
-    ctx->easy_timed = ctx->p2_timed = false;
+    double* phase[] = {&ctx->stats.ms_s1, &ctx->stats.ms_easy, &ctx->stats.ms_hard, &ctx->stats.ms_p2};
+    for (int i = 0; i + 1 < ctx->marks; i++)
+        if (cudaEventElapsedTime(&ms, ctx->ev[6 + i], ctx->ev[7 + i]) == cudaSuccess) *phase[i] += ms;
+    ctx->hard_timed = ctx->easy_timed = ctx->p2_timed = false;
+    ctx->marks = 0;
     ctx->dstat = nullptr;
-    return PC_OK;
-}
-
-static int sync_timed(pc_ctx* ctx, double* acc, Timer& t)
-{
-    PC_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-    *acc += t.ms();
-    t = Timer();
     return PC_OK;
 }
 
@@ -245,8 +264,10 @@ static int leaf_parts(pc_ctx* ctx, u64 x, u64 y, u32 c, u64 a, bool want_p2, boo
     const u64 z = x / y;
     const u64 r = pc_isqrt(x);
     PC_TRY(tables_ensure(ctx, r > y ? r : y, pc_max(y, pc_isqrt(z)), y, c));
-    u64 vals[3] = {y, pc_isqrt(z), pc_isqrt(r)}, pv[3];
-    PC_TRY(tables_pi_values(ctx, vals, pv, 3));
+    // every pi value the phases need, in one lookup
+    u64 vals[4 + P2_ASK] = {y, pc_isqrt(z), pc_isqrt(r), pc_iroot3(x)}, pv[4 + P2_ASK];
+    const int n_ask = 4 + (want_p2 ? p2_ask(ctx, x, y, vals + 4) : 0);
+    PC_TRY(tables_pi_values(ctx, vals, pv, n_ask));
     const u64 piy = pv[0], B = pv[1];
     if (a == 0) a = piy;
     if (a > piy || c > a) {
@@ -254,8 +275,8 @@ static int leaf_parts(pc_ctx* ctx, u64 x, u64 y, u32 c, u64 a, bool want_p2, boo
                      (unsigned long long)piy);
         return PC_EINVAL;
     }
-    PC_TRY(sync_timed(ctx, &ctx->stats.ms_tables, t));
-    LeafProblem P{x, y, z, c, a, a < piy, piy, B, pv[2]};
+    ctx->stats.ms_tables += t.ms();
+    LeafProblem P{x, y, z, c, a, a < piy, piy, B, pv[2], pv[3]};
     P.table_in_easy = total_only;
     ctx->stats.y = y;
     ctx->stats.z = z;
@@ -263,19 +284,19 @@ static int leaf_parts(pc_ctx* ctx, u64 x, u64 y, u32 c, u64 a, bool want_p2, boo
     ctx->stats.B = B;
     ctx->stats.c = c;
     I128Pair* d;
-    PC_TRY(result_slots(ctx, 5, &d));
-    PC_TRY(run_s1(ctx, P, d + 0));
-    PC_TRY(sync_timed(ctx, &ctx->stats.ms_s1, t));
-    PC_TRY(run_trivial(ctx, P, d + 1));
-    PC_TRY(sync_timed(ctx, &ctx->stats.ms_trivial, t));
+    // the phases follow one another on the stream, with no wait in between
+    PC_TRY(result_slots(ctx, &d));
+    PC_TRY(mark(ctx));
+    PC_TRY(run_s1_trivial(ctx, P, d + 0, d + 1));
+    PC_TRY(mark(ctx));
     PC_TRY(run_easy(ctx, P, d + 2));
-    PC_TRY(sync_timed(ctx, &ctx->stats.ms_easy, t));
+    PC_TRY(mark(ctx));
     PC_TRY(run_hard_smallb(ctx, P, d + 3));
     PC_TRY(run_hard_sieve(ctx, P, d + 3));
-    PC_TRY(sync_timed(ctx, &ctx->stats.ms_hard, t));
+    PC_TRY(mark(ctx));
     if (want_p2) {
-        PC_TRY(run_p2(ctx, x, y, a, d + 4));
-        PC_TRY(sync_timed(ctx, &ctx->stats.ms_p2, t));
+        PC_TRY(run_p2(ctx, x, y, a, pv + 4, d + 4));
+        PC_TRY(mark(ctx));
     }
     PC_TRY(read_slots(ctx, 5, parts));
     if (!want_p2) parts[4] = 0;
@@ -326,15 +347,16 @@ static int s2_hard_impl(pc_ctx* ctx, uint64_t x, uint64_t y, uint32_t c, u32 sha
     const u64 z = x / y;
     const u64 r = pc_isqrt(x);
     PC_TRY(tables_ensure(ctx, r > y ? r : y, pc_max(y, pc_isqrt(z)), y, c));
-    u64 vals[3] = {y, pc_isqrt(z), pc_isqrt(r)}, pv[3];
-    PC_TRY(tables_pi_values(ctx, vals, pv, 3));
+    u64 vals[4] = {y, pc_isqrt(z), pc_isqrt(r), pc_iroot3(x)}, pv[4];
+    PC_TRY(tables_pi_values(ctx, vals, pv, 4));
     const u64 piy = pv[0], B = pv[1];
     if (c > piy) {
         pc_set_error(ctx, "c=%u exceeds pi(y)=%llu", c, (unsigned long long)piy);
         return PC_EINVAL;
     }
-    PC_TRY(sync_timed(ctx, &ctx->stats.ms_tables, ph));
-    LeafProblem P{x, y, z, c, piy, false, piy, B, pv[2]};
+    ctx->stats.ms_tables += ph.ms();
+    ph = Timer();
+    LeafProblem P{x, y, z, c, piy, false, piy, B, pv[2], pv[3]};
     P.shard_k = shard_k;
     P.shard_n = shard_n;
     ctx->stats.y = y;
@@ -343,7 +365,7 @@ static int s2_hard_impl(pc_ctx* ctx, uint64_t x, uint64_t y, uint32_t c, u32 sha
     ctx->stats.B = B;
     ctx->stats.c = c;
     I128Pair* d;
-    PC_TRY(result_slots(ctx, 1, &d));
+    PC_TRY(result_slots(ctx, &d));
     if (shard_n == 0 || shard_k == 0)
         PC_TRY(run_hard_smallb(ctx, P, d));   // closed-form leaves (b <= 3): counted once, in shard 0
     PC_TRY(run_hard_sieve(ctx, P, d));
@@ -369,11 +391,11 @@ extern "C" int pc_p2(pc_ctx* ctx, uint64_t x, uint64_t y, uint64_t* out)
     const u64 z = x / y;
     const u64 r = pc_isqrt(x);
     PC_TRY(tables_ensure(ctx, r > y ? r : y, pc_max(y, pc_isqrt(z)), 0, 7));
-    u64 vals[1] = {y}, pv[1];
-    PC_TRY(tables_pi_values(ctx, vals, pv, 1));
+    u64 vals[1 + P2_ASK] = {y}, pv[1 + P2_ASK];
+    PC_TRY(tables_pi_values(ctx, vals, pv, 1 + p2_ask(ctx, x, y, vals + 1)));
     I128Pair* d;
-    PC_TRY(result_slots(ctx, 1, &d));
-    PC_TRY(run_p2(ctx, x, y, pv[0], d));
+    PC_TRY(result_slots(ctx, &d));
+    PC_TRY(run_p2(ctx, x, y, pv[0], pv + 1, d));
     i128 v;
     PC_TRY(read_slots(ctx, 1, &v));
     if (v < 0 || (v >> 64) != 0) return PC_EOVERFLOW;

@@ -100,7 +100,6 @@ struct HardArgs {
     const uint2* primes_dv;   // p_k and its 32-bit reciprocal (pc_dv)
     const uint4* pat;     // patterns of the primes 7 .. 61 (Tables::pat16)
     const u32* segB;
-    const u64* rcp_seg;   // per segment: reciprocals of L_s and L_s + span (0 for L = 0)
     const u64* off;
     const u32* rlo;     // first segment of row b (index b - k0): entry s of the row is off + s - rlo
     const u64* start;   // phi(L_{s0} - 1, b) for b = k0 .. bmax (index b - k0), or null for s0 = 0
@@ -108,9 +107,9 @@ struct HardArgs {
     i32* tallies;
     const HardItem* items;
     const unsigned long long* nitems;   // number of items, written by the planner
-    I128Pair* acc;                 // one slot per CTA
+    I128Pair* acc;                 // the hard sum
     u32* queue;
-    unsigned long long* stat;      // [0] hard leaves, [1] multiples crossed off
+    unsigned long long* stat;      // [0] hard leaves, [1] multiples crossed off (from p >= PATTERN_P on)
 };
 
 struct __align__(16) StepInfo {
@@ -867,7 +866,7 @@ __global__ void __launch_bounds__(MAXT, MINB) hard_sieve_kernel(HardArgs A0, Mul
                         intra += (i64)tk * run;
                         run += cp[k];
                     }
-                    if (T) atomicAdd(&A.tallies[at], T);
+                    A.tallies[at] = T;   // one item owns the step
                     acc += intra;
                 }
             }
@@ -879,7 +878,7 @@ __global__ void __launch_bounds__(MAXT, MINB) hard_sieve_kernel(HardArgs A0, Mul
     if (MULTI) {
         if (tid == 0 && cur_q != ~0u) mq_atomic_add_i128(M.qacc + (u64)cur_q * M.qstride, tot);
     } else {
-        if (tid == 0) store_i128(A0.acc + blockIdx.x, tot);
+        if (tid == 0 && tot != 0) mq_atomic_add_i128(A0.acc, tot);
     }
     unsigned long long nleaves64 = nleaves, nclears64 = nclears;
     for (int o = 16; o; o >>= 1) {
@@ -924,34 +923,30 @@ __device__ __forceinline__ u64 row_start(const HardArgs& A, u32 b)
     return n >= b ? n - b + 2 : 1;
 }
 
-__global__ void seg_b_kernel(u64 x, u64 nseg, u64 span, u32 bmax, PiTable pit, u32* segB, u64* rcp_seg)
+// The run's schedule in one launch.  The first segblocks blocks take a warp per segment s in
+// [s0, s1): B_s, and an upper bound of its hard leaves (the lpf filter of the m-list is not
+// applied), its lanes over the segment's leaf primes b (kleaf < b <= min(B_s, a)).  The others
+// take a thread per row b: its segments.
+__global__ void __launch_bounds__(256) hard_prep_kernel(HardArgs A, u32 segblocks, u32* segB, unsigned long long* est,
+                                                        u32* len, u32* rlo)
 {
-    u64 s = (u64)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= nseg) return;
-    rcp_seg[2 * s] = s ? ~0ull / (s * span) : 0;
-    rcp_seg[2 * s + 1] = ~0ull / ((s + 1) * span);
-    segB[s] = seg_b(x, s, span, bmax, pit);
-}
-
-__global__ void row_len_kernel(u64 x, const u32* primes, u64 span, u64 nseg, u64 s0, u64 s1, u32 k0, u32 bmax,
-                               u32* len, u32* rlo)
-{
-    u32 t = blockIdx.x * blockDim.x + threadIdx.x;
-    u32 b = k0 + t;
-    if (b > bmax) return;
-    len[t] = row_range(x, primes[b], span, nseg, s0, s1, rlo + t);
-}
-
-// Upper bound of the hard leaves of every segment (the lpf filter of the
-// m-list is not applied): a warp per segment s in [s0, s1), its lanes over the
-// segment's leaf primes b (kleaf < b <= min(B_s, a)), one store per segment.
-__global__ void hard_estimate_kernel(HardArgs A, unsigned long long* est)
-{
+    if (blockIdx.x >= segblocks) {
+        const u32 t = (blockIdx.x - segblocks) * blockDim.x + threadIdx.x, b = A.k0 + t;
+        if (b <= A.bmax) len[t] = row_range(A.x, A.primes[b], A.span, A.nseg, A.s0, A.s1, rlo + t);
+        return;
+    }
     const u64 s = A.s0 + ((u64)blockIdx.x * blockDim.x + threadIdx.x) / 32;
     const u32 lane = threadIdx.x & 31;
     if (s >= A.s1) return;   // the whole warp
-    const u64 L = s * A.span, vL = A.rcp_seg[2 * s], vLs = A.rcp_seg[2 * s + 1];
-    const u64 bhi = pc_min((u64)A.segB[s], A.a);
+    const u64 L = s * A.span;
+    u32 B = 0;
+    u64 v = 0;
+    if (lane == 0) B = seg_b(A.x, s, A.span, A.bmax, A.pit);
+    if (lane < 2) v = L + lane * A.span;
+    v = v ? ~0ull / v : 0;   // reciprocals of L (0 for L = 0) and L + span
+    B = __shfl_sync(0xffffffffu, B, 0);
+    const u64 vL = __shfl_sync(0xffffffffu, v, 0), vLs = __shfl_sync(0xffffffffu, v, 1);
+    const u64 bhi = pc_min((u64)B, A.a);
     u64 n = 0;
     for (u64 b = A.kleaf + 1 + lane; b <= bhi; b += 32) {
         const u64 p = A.primes[b];
@@ -968,13 +963,16 @@ __global__ void hard_estimate_kernel(HardArgs A, unsigned long long* est)
         }
     }
     for (int o = 16; o; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
-    if (lane == 0) est[s] = n;
+    if (lane == 0) {
+        segB[s] = B;
+        est[s] = n;
+    }
 }
 
 // S2_hard carries: for each leaf prime b, the exclusive scan over segments
 // of count(., b-1) dotted with tally(., b).
 template <int NT>
-__global__ void __launch_bounds__(NT) hard_combine_kernel(HardArgs A, I128Pair* part)
+__global__ void __launch_bounds__(NT) hard_combine_kernel(HardArgs A, I128Pair* out)
 {
     __shared__ u64 wsum[NT / 32];
     __shared__ u64 s_carry;
@@ -1020,7 +1018,7 @@ __global__ void __launch_bounds__(NT) hard_combine_kernel(HardArgs A, I128Pair* 
         }
     }
     dot = block_sum_i128(dot, red);
-    if (threadIdx.x == 0) store_i128(part + blockIdx.x, dot);
+    if (threadIdx.x == 0 && dot != 0) mq_atomic_add_i128(out, dot);
 }
 
 // ---------------------------------------------------------------- host
@@ -1052,6 +1050,10 @@ u32 hard_seg_for(u64 z)
 {
     return z < 400000ull ? 2048 : z < 280000000ull ? 8192 : z < 2000000000ull ? 16384 : 32768;
 }
+
+// count-row entries (8 bytes each with their tallies) up to which a run takes rows x segments as
+// their bound instead of reading the exact number back: 64 MiB
+static constexpr u64 ROWS_UNREAD = 1ull << 23;
 
 // bytes per warp sub-range: a power of two dividing seg_bytes, at most 16 warps
 static u32 pc_sub_bytes(pc_ctx* ctx, u32 seg_bytes, u32 dflt)
@@ -1099,7 +1101,7 @@ struct PlanArgs {
     const u32* segB;
     const unsigned long long* est;
     u32 k0;
-    double x, z;
+    float x, z;
     u64 span, s0, s1;
     double inv_ctas4;           // 1 / (4 * resident CTAs)
     u64 cap;                    // slots in items
@@ -1111,14 +1113,30 @@ struct PlanArgs {
                                 // [7] steps replicas cross off before their own
 };
 
-__device__ __forceinline__ double seg_cost(const PlanArgs& P, u64 s)
+__device__ __forceinline__ float seg_cost(const PlanArgs& P, u64 s)
 {
-    const double steps = (double)(P.segB[s] - P.k0);
-    const double sz = sqrt(P.z);
-    const double top = fmin(sqrt((double)(s + 1) * (double)P.span), sz);
-    const double pm = s ? fmin(sqrt(P.x / ((double)s * (double)P.span)), top) : top;
-    const double ll = pm > 16.0 ? log(log(pm)) - 1.0056 : 0.0;
-    return 128.0 * steps + 0.08 * (double)P.span * (8.0 / 30.0) * (ll > 0.0 ? ll : 0.0);
+    const float steps = (float)(P.segB[s] - P.k0);
+    const float sz = sqrtf(P.z);
+    const float top = fminf(sqrtf((float)(s + 1) * (float)P.span), sz);
+    const float pm = s ? fminf(sqrtf(P.x / ((float)s * (float)P.span)), top) : top;
+    const float ll = pm > 16.0f ? logf(logf(pm)) - 1.0056f : 0.0f;
+    return 128.0f * steps + 0.08f * (float)P.span * (8.0f / 30.0f) * (ll > 0.0f ? ll : 0.0f);
+}
+
+// R and the cost bucket of segment s: R | bucket << 16, or 0 for a segment without steps
+__device__ __forceinline__ u32 seg_split(const PlanArgs& P, u64 s, float target)
+{
+    if (P.segB[s] <= P.k0) return 0;
+    const float base = seg_cost(P, s), e = (float)P.est[s];
+    u32 R = 1;
+    if (base + e > target && e > base) {
+        const float room = fmaxf(target - base, base);
+        R = (u32)fminf(1024.0f, ceilf(e / fmaxf(room, 1.0f)));
+        if (R < 1) R = 1;
+    }
+    const int k = (int)floorf(4.0f * log2f((base + e) / R));   // a replica's share
+    const u32 key = (u32)(k < 0 ? 0 : (k >= PLAN_BUCKETS ? PLAN_BUCKETS - 1 : k));
+    return R | (key << 16);
 }
 
 __global__ void plan_cost_kernel(PlanArgs P)
@@ -1137,24 +1155,14 @@ __global__ void plan_cost_kernel(PlanArgs P)
     }
 }
 
-// R and the cost bucket of every segment, decided once and stored
+// the split of every segment, decided once and stored
 __global__ void plan_split_kernel(PlanArgs P)
 {
-    const double target = fmax(P.scr->total * P.inv_ctas4, 1.0);
+    const float target = fmaxf((float)(P.scr->total * P.inv_ctas4), 1.0f);
     for (u64 s = P.s0 + (u64)blockIdx.x * blockDim.x + threadIdx.x; s < P.s1; s += (u64)gridDim.x * blockDim.x) {
-        u32 v = 0;
-        if (P.segB[s] > P.k0) {
-            const double base = seg_cost(P, s), e = (double)P.est[s];
-            u32 R = 1;
-            if (base + e > target && e > base) {
-                const double room = fmax(target - base, base);
-                R = (u32)fmin(1024.0, ceil(e / fmax(room, 1.0)));
-                if (R < 1) R = 1;
-            }
-            const int k = (int)floor(4.0 * log2((base + e) / R));   // a replica's share
-            const u32 key = (u32)(k < 0 ? 0 : (k >= PLAN_BUCKETS ? PLAN_BUCKETS - 1 : k));
-            v = R | (key << 16);
-            atomicAdd(&P.scr->cnt[key], R);
+        const u32 v = seg_split(P, s, target);
+        if (v) {
+            atomicAdd(&P.scr->cnt[v >> 16], v & 0xFFFFu);
             atomicAdd(&P.stat[5], (unsigned long long)(P.segB[s] - P.k0));
         }
         P.split[s] = v;
@@ -1189,6 +1197,64 @@ __global__ void plan_scatter_kernel(PlanArgs P)
         for (u32 r = 0; r < R; r++) P.items[pos + r] = HardItem{(u32)s, r ? ~0u : P.k0 + 1, ~0u, 0u};
         if (R > 1) P.heavy[atomicAdd(&P.scr->nheavy, 1u)] = HeavySeg{(u32)s, pos, R, 0u};
     }
+}
+
+// The planner in one launch (one CTA) for up to PLAN_ONE segments: the same decisions, with the
+// buckets in shared memory.  Also the number of count-row entries, for the caller's statistics.
+// (Four launches and their gaps cost more than the work: pi(10^12) plans 26 segments.)
+static constexpr u64 PLAN_ONE = 8192;
+__global__ void __launch_bounds__(1024) plan_one_kernel(PlanArgs P, const u64* rows)
+{
+    __shared__ double part[32];
+    __shared__ u32 cnt[PLAN_BUCKETS], cur[PLAN_BUCKETS];
+    __shared__ u32 nheavy, ok;
+    __shared__ unsigned long long steps;
+    const u32 tid = threadIdx.x;
+    if (tid < PLAN_BUCKETS) cnt[tid] = 0;
+    if (tid == 0) nheavy = 0, steps = 0;
+    double t = 0;
+    unsigned long long st = 0;
+    for (u64 s = P.s0 + tid; s < P.s1; s += 1024)
+        if (P.segB[s] > P.k0) {
+            t += seg_cost(P, s) + (double)P.est[s];
+            st += P.segB[s] - P.k0;
+        }
+    for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if ((tid & 31) == 0) part[tid >> 5] = t;
+    __syncthreads();
+    if (st) atomicAdd(&steps, st);
+    double total = 0;
+    for (u32 k = 0; k < 32; k++) total += part[k];
+    const float target = fmaxf((float)(total * P.inv_ctas4), 1.0f);
+    for (u64 s = P.s0 + tid; s < P.s1; s += 1024) {
+        const u32 v = seg_split(P, s, target);
+        P.split[s] = v;
+        if (v) atomicAdd(&cnt[v >> 16], v & 0xFFFFu);
+    }
+    __syncthreads();
+    if (tid == 0) {   // first slot of every bucket, the most costly bucket first
+        unsigned long long run = 0;
+        for (int k = PLAN_BUCKETS - 1; k >= 0; k--) {
+            cur[k] = (u32)run;
+            run += cnt[k];
+        }
+        ok = run <= P.cap;   // always, with cap = segments + 8 * CTAs; the run reports it if not
+        P.scr->nitems = P.stat[4] = ok ? run : 0;
+        P.stat[5] = steps;
+        P.stat[6] = ok ? 0 : 1;
+        P.stat[8] = *rows;
+    }
+    __syncthreads();
+    if (ok)
+        for (u64 s = P.s0 + tid; s < P.s1; s += 1024) {
+            const u32 v = P.split[s], R = v & 0xFFFFu;
+            if (!R) continue;
+            const u32 pos = atomicAdd(&cur[v >> 16], R);
+            for (u32 r = 0; r < R; r++) P.items[pos + r] = HardItem{(u32)s, r ? ~0u : P.k0 + 1, ~0u, 0u};
+            if (R > 1) P.heavy[atomicAdd(&nheavy, 1u)] = HeavySeg{(u32)s, pos, R, 0u};
+        }
+    __syncthreads();
+    if (tid == 0) P.scr->nheavy = nheavy;
 }
 
 // Estimated cost of step b of the segment [L, L + span), in the units of seg_cost (one
@@ -1362,19 +1428,17 @@ int run_hard_sieve(pc_ctx* ctx, const LeafProblem& P, I128Pair* out)
         A.s1 = A.nseg * (P.shard_k + 1) / P.shard_n;
         if (A.s1 <= A.s0) return PC_OK;   // an empty shard
     }
-    if (!P.table_in_easy) PC_TRY(run_hard_table(ctx, P, A.kleaf, A.s0 * A.span, A.s1 * A.span, out));
     const u64 bmax = pc_min(pc_min(P.B, P.a), P.R4);
+    std::vector<u64> hstart;
+    if (P.shard_n && A.s0 && bmax > A.kleaf) {
+        // carries into the shard: phi(L - 1, b) for every b (Section 4), computed before
+        // this run launches anything (the queries may grow the tables) or claims scratch
+        hstart.resize(bmax - A.k0 + 1);
+        PC_TRY(phi_starts(ctx, A.s0 * A.span - 1, A.k0, bmax, hstart.data()));
+    }
+    if (!P.table_in_easy) PC_TRY(run_hard_table(ctx, P, A.kleaf, A.s0 * A.span, A.s1 * A.span, out));
     if (bmax <= A.kleaf) return PC_OK;   // no hard leaf needs the sieve
     A.bmax = (u32)bmax;
-    std::vector<u64> hstart;
-    if (P.shard_n) {
-        if (A.s0) {
-            // carries into the shard: phi(L - 1, b) for every b (Section 4), computed
-            // before this run claims the context's scratch
-            hstart.resize(bmax - A.k0 + 1);
-            PC_TRY(phi_starts(ctx, A.s0 * A.span - 1, A.k0, bmax, hstart.data()));
-        }
-    }
     A.pit = ctx->T.pi();
     A.rk = ctx->T.rank();
     A.ml = ctx->T.mlist();
@@ -1390,25 +1454,22 @@ int run_hard_sieve(pc_ctx* ctx, const LeafProblem& P, I128Pair* out)
     A.pat = ctx->T.pat16.as<uint4>();
 
     const u64 nrows = bmax - A.k0 + 1;
+    const u64 ns = A.s1 - A.s0;
     PC_TRY(buf_reserve(ctx, ctx->seg_b, A.nseg * sizeof(u32) + 2 * (nrows + 1) * sizeof(u32)));
-    PC_TRY(buf_reserve(ctx, ctx->seg_off, (nrows + 1) * sizeof(u64) + 3 * A.nseg * sizeof(u64) + A.nseg * sizeof(u32) +
+    PC_TRY(buf_reserve(ctx, ctx->seg_off, (nrows + 1) * sizeof(u64) + A.nseg * sizeof(u64) + A.nseg * sizeof(u32) +
                                               A.nseg * sizeof(HeavySeg) + 16));
     u32* segB = ctx->seg_b.as<u32>();
     u32* rowlen = segB + A.nseg;
     u32* rlo = rowlen + nrows + 1;
     u64* off = ctx->seg_off.as<u64>();
     unsigned long long* est = (unsigned long long*)(off + nrows + 1);
-    u64* rcp_seg = (u64*)(est + A.nseg);
-    u32* split = (u32*)(rcp_seg + 2 * A.nseg);   // the work-item split of every segment
+    u32* split = (u32*)(est + A.nseg);   // the work-item split of every segment
     HeavySeg* heavy = (HeavySeg*)(((uintptr_t)(split + A.nseg) + 15) & ~(uintptr_t)15);
-    A.rcp_seg = rcp_seg;
-    seg_b_kernel<<<(unsigned)((A.nseg + 255) / 256), 256, 0, ctx->stream>>>(P.x, A.nseg, A.span, A.bmax, A.pit, segB,
-                                                                            rcp_seg);
+    const u32 segblocks = (u32)((ns + 7) / 8);
+    hard_prep_kernel<<<segblocks + (unsigned)((nrows + 255) / 256), 256, 0, ctx->stream>>>(A, segblocks, segB, est,
+                                                                                          rowlen, rlo);
     PC_LAUNCHED(ctx);
-    row_len_kernel<<<(unsigned)((nrows + 255) / 256), 256, 0, ctx->stream>>>(P.x, A.primes, A.span, A.nseg, A.s0,
-                                                                              A.s1, A.k0, A.bmax, rowlen, rlo);
-    PC_LAUNCHED(ctx);
-    ctx->stats.kernel_launches += 2;
+    ctx->stats.kernel_launches++;
     PC_TRY(scan_exclusive_u32_to_u64(ctx, rowlen, off, nrows));
     A.segB = segB;
     A.off = off;
@@ -1419,9 +1480,15 @@ int run_hard_sieve(pc_ctx* ctx, const LeafProblem& P, I128Pair* out)
         PC_CUDA(ctx, cudaMemcpyAsync(ctx->starts.p, hstart.data(), hstart.size() * sizeof(u64),
                                      cudaMemcpyHostToDevice, ctx->stream));
         A.start = ctx->starts.as<u64>();
+        PC_CUDA(ctx, cudaStreamSynchronize(ctx->stream));   // hstart is pageable memory of this call
     }
-    u64 total = 0;
-    PC_TRY(copy_to_host(ctx, &total, off + nrows, sizeof(u64)));
+    // The count and tally rows: rows x segments bounds them; where that is small the exact number
+    // stays on the device, and the launches below follow without a wait.
+    u64 total = ns * nrows;
+    if (total > ROWS_UNREAD || ns > PLAN_ONE) {
+        PC_TRY(copy_to_host(ctx, &total, off + nrows, sizeof(u64)));
+        ctx->stats.steps = total;
+    }
     if (total >> 32) {
         pc_set_error(ctx, "hard-leaf sieve: %llu count rows exceed 32-bit offsets", (unsigned long long)total);
         return PC_EOVERFLOW;
@@ -1433,79 +1500,53 @@ int run_hard_sieve(pc_ctx* ctx, const LeafProblem& P, I128Pair* out)
     PC_TRY(choose_hard_kernel<false>(ctx, A, smem, &kern, &per_sm));
     int ctas = ctx->sm_count * per_sm;
 
-    // per-segment leaf estimate, then the work items, all on the device
-    PC_CUDA(ctx, cudaMemsetAsync(est, 0, A.nseg * sizeof(u64), ctx->stream));
-    if (A.s1 > A.s0) {
-        hard_estimate_kernel<<<(unsigned)(((A.s1 - A.s0) * 32 + 255) / 256), 256, 0, ctx->stream>>>(A, est);
-        PC_LAUNCHED(ctx);
-        ctx->stats.kernel_launches++;
-    }
-    const u64 cap = (A.s1 - A.s0) + 8ull * (u64)ctas + 64;
-    const size_t items_bytes = (size_t)ctas * sizeof(I128Pair) + cap * sizeof(HardItem);
+    // the work items, planned on the device
+    const u64 cap = ns + 8ull * (u64)ctas + 64;
+    const size_t items_bytes = (cap * sizeof(HardItem) + 15) / 16 * 16;
     PC_TRY(buf_reserve(ctx, ctx->counts, total * sizeof(u32)));
     PC_TRY(buf_reserve(ctx, ctx->tallies, total * sizeof(i32)));
-    PC_TRY(buf_reserve(ctx, ctx->acc_seg, (items_bytes + 15) / 16 * 16 + sizeof(PlanScratch)));
-    PC_TRY(buf_reserve(ctx, ctx->queue, 128));
-    HardItem* ditems = (HardItem*)(ctx->acc_seg.as<I128Pair>() + ctas);
-    PlanScratch* scr = (PlanScratch*)(ctx->acc_seg.as<unsigned char>() + (items_bytes + 15) / 16 * 16);
+    PC_TRY(buf_reserve(ctx, ctx->acc_seg, items_bytes + sizeof(PlanScratch)));
+    HardItem* ditems = ctx->acc_seg.as<HardItem>();
+    PlanScratch* scr = (PlanScratch*)(ctx->acc_seg.as<unsigned char>() + items_bytes);
     A.counts = ctx->counts.as<u32>();
     A.tallies = ctx->tallies.as<i32>();
     A.items = ditems;
     A.nitems = &scr->nitems;
-    A.acc = ctx->acc_seg.as<I128Pair>();
-    A.queue = ctx->queue.as<u32>();
-    A.stat = (unsigned long long*)(ctx->queue.as<u32>() + 2);
-    PC_CUDA(ctx, cudaMemsetAsync(ctx->queue.p, 0, 128, ctx->stream));
-    PC_CUDA(ctx, cudaMemsetAsync(scr, 0, sizeof(PlanScratch), ctx->stream));
-    PC_CUDA(ctx, cudaMemsetAsync(ctx->tallies.p, 0, total * sizeof(i32), ctx->stream));
-    PlanArgs PA{segB, est, A.k0, (double)P.x, (double)P.z, A.span, A.s0, A.s1, 1.0 / (4.0 * ctas), cap,
+    A.acc = out;
+    A.queue = (u32*)call_queue(ctx, Q_HARD);
+    A.stat = call_hard_stat(ctx);
+    PlanArgs PA{segB, est, A.k0, (float)P.x, (float)P.z, A.span, A.s0, A.s1, 1.0 / (4.0 * ctas), cap,
                 scr, split, ditems, heavy, A.stat};
-    const unsigned pg = (unsigned)pc_min((A.s1 - A.s0 + 255) / 256, (u64)ctx->sm_count * 4);
-    plan_cost_kernel<<<pg, 256, 0, ctx->stream>>>(PA);
+    if (ns <= PLAN_ONE) {
+        plan_one_kernel<<<1, 1024, 0, ctx->stream>>>(PA, off + nrows);
+        PC_LAUNCHED(ctx);
+        ctx->stats.kernel_launches++;
+    } else {
+        const unsigned pg = (unsigned)pc_min((ns + 255) / 256, (u64)ctx->sm_count * 4);
+        PC_CUDA(ctx, cudaMemsetAsync(scr, 0, sizeof(PlanScratch), ctx->stream));
+        plan_cost_kernel<<<pg, 256, 0, ctx->stream>>>(PA);
+        PC_LAUNCHED(ctx);
+        plan_split_kernel<<<pg, 256, 0, ctx->stream>>>(PA);
+        PC_LAUNCHED(ctx);
+        plan_offsets_kernel<<<1, 32, 0, ctx->stream>>>(PA);
+        PC_LAUNCHED(ctx);
+        plan_scatter_kernel<<<pg, 256, 0, ctx->stream>>>(PA);
+        PC_LAUNCHED(ctx);
+        ctx->stats.kernel_launches += 4;
+    }
+    plan_bsplit_kernel<<<(unsigned)pc_min(ns, (u64)ctx->sm_count * 2), 256, 0, ctx->stream>>>(A, PA);
     PC_LAUNCHED(ctx);
-    plan_split_kernel<<<pg, 256, 0, ctx->stream>>>(PA);
-    PC_LAUNCHED(ctx);
-    plan_offsets_kernel<<<1, 32, 0, ctx->stream>>>(PA);
-    PC_LAUNCHED(ctx);
-    plan_scatter_kernel<<<pg, 256, 0, ctx->stream>>>(PA);
-    PC_LAUNCHED(ctx);
-    plan_bsplit_kernel<<<ctx->sm_count * 2, 256, 0, ctx->stream>>>(A, PA);
-    PC_LAUNCHED(ctx);
-    ctx->stats.kernel_launches += 5;
+    ctx->stats.kernel_launches++;
 
-    cudaEvent_t e0 = ctx->ev[0], e1 = ctx->ev[1];
-    PC_CUDA(ctx, cudaEventRecord(e0, ctx->stream));
+    PC_CUDA(ctx, cudaEventRecord(ctx->ev[0], ctx->stream));
     kern<<<ctas, 32 * A.nw, smem, ctx->stream>>>(A, MultiArgs{});
     PC_LAUNCHED(ctx);
-    PC_CUDA(ctx, cudaEventRecord(e1, ctx->stream));
-    ctx->stats.kernel_launches++;
-
-    int g = (int)pc_min(bmax - A.kleaf, 4096);
-    PC_TRY(buf_reserve(ctx, ctx->partials, g * sizeof(I128Pair)));
-    hard_combine_kernel<256><<<g, 256, 0, ctx->stream>>>(A, ctx->partials.as<I128Pair>());
+    PC_CUDA(ctx, cudaEventRecord(ctx->ev[1], ctx->stream));
+    ctx->hard_timed = true;
+    hard_combine_kernel<256><<<(int)pc_min(bmax - A.kleaf, 4096), 256, 0, ctx->stream>>>(A, out);
     PC_LAUNCHED(ctx);
-    ctx->stats.kernel_launches++;
-    PC_TRY(reduce_i128(ctx, ctx->partials.as<I128Pair>(), g, out));
-    PC_TRY(reduce_i128(ctx, A.acc, ctas, out));
-
-    u64 nl[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    PC_TRY(copy_to_host(ctx, nl, A.stat, 8 * sizeof(u64)));
-    if (nl[6]) {
-        pc_set_error(ctx, "hard-leaf sieve: work items exceed the planned %llu slots", (unsigned long long)cap);
-        return PC_EOVERFLOW;
-    }
-    ctx->stats.work_items = nl[4];
-    ctx->stats.item_steps += nl[5];
-    ctx->stats.presieve_steps += nl[7];
-    ctx->stats.warp_steps += nl[2];
-    ctx->stats.leaf_warp_steps += nl[3];
-    float ms = 0;
-    PC_CUDA(ctx, cudaEventElapsedTime(&ms, e0, e1));
-    ctx->stats.ms_hard_sieve = ms;
-    ctx->stats.hard_leaves += nl[0];
-    ctx->stats.clears += nl[1];
+    ctx->stats.kernel_launches += 2;
     ctx->stats.segments = A.nseg;
-    ctx->stats.steps = total;
     ctx->stats.seg_bytes = A.seg_bytes;
     return PC_OK;
 }
@@ -1515,16 +1556,14 @@ int run_hard_sieve(pc_ctx* ctx, const LeafProblem& P, I128Pair* out)
 // segments (largest queries first, since the batch sorts them so), with the segment
 // schedule and the count rows of every query built by one launch each.
 
-// B_s and the reciprocals of L_s, L_s + span for segment g - pref[q] of query q
-__global__ void mq_seg_b_kernel(const HardArgs* qa, const u64* pref, u32 Q, u32* segB, u64* rcp_seg)
+// B_s for segment g - pref[q] of query q
+__global__ void mq_seg_b_kernel(const HardArgs* qa, const u64* pref, u32 Q, u32* segB)
 {
     const u64 g = (u64)blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= pref[Q]) return;
     const u64 q = mq_find(pref, Q + 1, g);
     const HardArgs& A = qa[q];
     const u64 s = g - pref[q];
-    rcp_seg[2 * g] = s ? ~0ull / (s * A.span) : 0;
-    rcp_seg[2 * g + 1] = ~0ull / ((s + 1) * A.span);
     segB[g] = seg_b(A.x, s, A.span, A.bmax, A.pit);
 }
 
@@ -1621,11 +1660,11 @@ int mq_hard(pc_ctx* ctx, const MQPlan& P)
         return PC_EOVERFLOW;
     }
     for (u32 q = 0; q <= Q; q++) ipref[q] = (u32)spref[q];
-    // mq_h: spref | rpref | cpref (Q+1 u64 each) | ipref (Q+1 u32) | segB (S u32) | rcp_seg (2S u64) |
+    // mq_h: spref | rpref | cpref (Q+1 u64 each) | ipref (Q+1 u32) | segB (S u32) |
     // rowlen (R u32) | rlo (R u32) | off (R+1 u64) | queue + counters (128 B)
     auto al = [](size_t v) { return (v + 15) / 16 * 16; };
     const size_t o_r = al((Q + 1) * 8), o_c = o_r + al((Q + 1) * 8), o_i = o_c + al((Q + 1) * 8);
-    const size_t o_sb = o_i + al((Q + 1) * 4), o_rc = o_sb + al(S * 4), o_rl = o_rc + al(2 * S * 8);
+    const size_t o_sb = o_i + al((Q + 1) * 4), o_rl = o_sb + al(S * 4);
     const size_t o_ro = o_rl + al(R * 4), o_off = o_ro + al(R * 4), o_q = o_off + al((R + 1) * 8), total = o_q + 128;
     PC_TRY(buf_reserve(ctx, ctx->mq_h, total));
     PC_TRY(buf_reserve(ctx, ctx->mq_hq, Q * sizeof(HardArgs)));
@@ -1637,7 +1676,6 @@ int mq_hard(pc_ctx* ctx, const MQPlan& P)
     u64* d_cpref = (u64*)(base + o_c);
     u32* d_ipref = (u32*)(base + o_i);
     u32* d_segB = (u32*)(base + o_sb);
-    u64* d_rcp = (u64*)(base + o_rc);
     u32* d_rowlen = (u32*)(base + o_rl);
     u32* d_rlo = (u32*)(base + o_ro);
     u64* d_off = (u64*)(base + o_off);
@@ -1659,7 +1697,6 @@ int mq_hard(pc_ctx* ctx, const MQPlan& P)
         A.s0 = 0;
         A.s1 = A.nseg;
         A.segB = d_segB + spref[q];
-        A.rcp_seg = d_rcp + 2 * spref[q];
         A.off = d_off + rpref[q];
         A.rlo = d_rlo + rpref[q];
         A.start = nullptr;
@@ -1692,8 +1729,7 @@ int mq_hard(pc_ctx* ctx, const MQPlan& P)
     }
     if (!mq_device_work(ctx)) return scan_exclusive_u32_to_u64(ctx, d_rowlen, d_off, R);   // its scratch only
     PC_CUDA(ctx, cudaMemsetAsync(d_queue, 0, 128, st));
-    PC_CUDA(ctx, cudaMemsetAsync(ctx->tallies.p, 0, bound * sizeof(i32), st));
-    mq_seg_b_kernel<<<(unsigned)((S + 255) / 256), 256, 0, st>>>(d_qa, d_spref, Q, d_segB, d_rcp);
+    mq_seg_b_kernel<<<(unsigned)((S + 255) / 256), 256, 0, st>>>(d_qa, d_spref, Q, d_segB);
     PC_LAUNCHED(ctx);
     mq_row_len_kernel<<<(unsigned)((R + 255) / 256), 256, 0, st>>>(d_qa, d_rpref, Q, d_rowlen, d_rlo);
     PC_LAUNCHED(ctx);

@@ -112,9 +112,10 @@ struct pc_ctx {
     size_t smem_optin = 0;
     Tables T;
     // scratch (grow-only)
-    DevBuf seg_b, seg_off, counts, tallies, acc_seg, partials, result, misc, scan_tmp, queue;
-    DevBuf easy_rng, easy_chunk_off, easy_cmap, starts;
+    DevBuf seg_b, seg_off, counts, tallies, acc_seg, partials, result, misc, scan_tmp;
+    DevBuf easy_rng, easy_chunk_off, starts;
     DevBuf mq_q, mq_pref, mq_e, mq_h, mq_hq, mq_p;   // batched queries (pc_pi_count_batch)
+    DevBuf p2_seg;   // P2: per-segment sums, counts and tallies
     DevBuf p2_bkt;   // P2 bucket sieve: the buckets of one wave of segments and their fill counts
     // pinned host staging for small results
     void* host_stage = nullptr;
@@ -134,10 +135,11 @@ struct pc_ctx {
     u32 seg_call = 0;   // segment bytes chosen for the running pi(x) call (0 = default)
     u32 tuned_ctas[21] = {0};   // autotuned resident CTAs per SM of the hard-leaf sieve (0 = most)
     u32 ctas_call = 0;          // the value for the running call
-    // device counters of the running call (easy leaves, runs, their leaves, P2 crossings),
-    // beside the result slots; null outside a leaf-sum call
+    // device counters of the running call (easy leaves, runs, their leaves, P2 crossings, table
+    // leaves), beside the result slots; null outside a leaf-sum call
     unsigned long long* dstat = nullptr;
-    bool easy_timed = false, p2_timed = false;   // ev[2..3] / ev[4..5] hold kernel times
+    bool hard_timed = false, easy_timed = false, p2_timed = false;   // ev[0..1] / ev[2..3] / ev[4..5] hold kernel times
+    int marks = 0;   // ev[6 ..] hold the ends of the call's phases
     // How the batched phases (mq_*) run: MQ_DIRECT launches as it goes; MQ_PREPARE reserves
     // scratch, uploads the arrays built on the host and reads back table values, with no
     // device work; MQ_CAPTURE then enqueues only device work (kernels, memsets), into a
@@ -190,10 +192,20 @@ static constexpr u32 PATTERN_P = 64;          // Tables::pat16 holds the primes 
 static constexpr u32 PATTERN_PRIMES = 15;     // p_4 = 7 .. p_18 = 61
 int tables_pat16(pc_ctx* ctx);
 int tables_phi_c(pc_ctx* ctx, u32 c);   // phi(., c) residue table
-// values of pi(v) for a handful of v (v <= pi_limit), synchronizing
+// values of pi(v) for a handful of v (v <= pi_limit, at most PI_ASK_MAX), synchronizing
+static constexpr int PI_ASK_MAX = 16;
 int tables_pi_values(pc_ctx* ctx, const u64* v, u64* out, int n);
 // pi(v) for any number of v (every v <= the table limit), synchronizing
 int tables_pi_many(pc_ctx* ctx, const u64* v, u64* out, size_t n);
+
+// The running call's result buffer, zeroed once per call and read back once at its end: eight
+// I128Pair parts, then (as u64) the call's counters (dstat), the hard-leaf sieve's (HardArgs::stat;
+// [8] = its count rows) and the work queues, each on a line of its own.
+static constexpr size_t RES_DSTAT = 128, RES_HARD = 256, RES_QUEUE = 384, RES_BYTES = 768;
+enum { Q_EASY = 0, Q_HARD = 1, Q_P2 = 2, Q_TABLE = 3 };
+inline unsigned long long* call_dstat(pc_ctx* c) { return (unsigned long long*)(c->result.as<unsigned char>() + RES_DSTAT); }
+inline unsigned long long* call_hard_stat(pc_ctx* c) { return (unsigned long long*)(c->result.as<unsigned char>() + RES_HARD); }
+inline unsigned long long* call_queue(pc_ctx* c, int q) { return (unsigned long long*)(c->result.as<unsigned char>() + RES_QUEUE + 64 * q); }
 
 // ----------------------------------------------------------------- leaves
 struct LeafProblem {
@@ -204,6 +216,7 @@ struct LeafProblem {
     u64 piy;      // pi(y)
     u64 B;        // pi(isqrt z)
     u64 R4;       // pi(x^(1/4)): a leaf with u >= p_b^2 and m > p_b has p_b^4 < x
+    u64 E;        // pi(iroot3 x): a leaf with u >= p_b has p_b^3 < x
     // hard-leaf sieve over segments [shard_k * nseg / shard_n, (shard_k + 1) * nseg / shard_n) only
     // (shard_n = 0: all of them); the leaves' carries then start from phi(L - 1, b)
     u32 shard_k = 0, shard_n = 0;
@@ -219,14 +232,17 @@ int phi_starts(pc_ctx* ctx, u64 m, u32 c, u64 b_max, u64* out);
 u64 hard_segments(pc_ctx* ctx, u64 z);
 
 // Each adds its sum to *out (device I128Pair) -- out must be zeroed first.
-int run_s1(pc_ctx* ctx, const LeafProblem& P, I128Pair* out);
-int run_trivial(pc_ctx* ctx, const LeafProblem& P, I128Pair* out);
+int run_s1_trivial(pc_ctx* ctx, const LeafProblem& P, I128Pair* out_s1, I128Pair* out_trivial);
 int run_easy(pc_ctx* ctx, const LeafProblem& P, I128Pair* out);
 int run_hard_smallb(pc_ctx* ctx, const LeafProblem& P, I128Pair* out);
 int run_hard_sieve(pc_ctx* ctx, const LeafProblem& P, I128Pair* out);
 // the hard leaves with y <= u < p_b^2, b > b_min, whose u lies in [u_lo, u_hi)
 int run_hard_table(pc_ctx* ctx, const LeafProblem& P, u64 b_min, u64 u_lo, u64 u_hi, I128Pair* out);
-int run_p2(pc_ctx* ctx, u64 x, u64 y, u64 a, I128Pair* out);
+// P2 takes the pi values it needs from the caller's one lookup: p2_ask writes the arguments (at
+// most P2_ASK), run_p2 gets their pi values in the same order
+static constexpr int P2_ASK = 5;
+int p2_ask(pc_ctx* ctx, u64 x, u64 y, u64* v);
+int run_p2(pc_ctx* ctx, u64 x, u64 y, u64 a, const u64* pv, I128Pair* out);
 
 // ------------------------------------------------------- batched queries
 // One pi(x) query of a batched launch (pc_pi_count_batch): its parameters, and the
@@ -259,6 +275,21 @@ __device__ __forceinline__ void mq_atomic_add_i128(I128Pair* p, i128 v)
     const unsigned long long old = atomicAdd((unsigned long long*)&p->lo, lo);
     const u64 carry = old + lo < old ? 1u : 0u;
     atomicAdd((unsigned long long*)&p->hi, (unsigned long long)((u64)(i64)(v >> 64) + carry));
+}
+
+// The last index k < n with pref[k] <= v (pref ascending, pref[0] <= v), by a whole warp: 32
+// probes a round, so 10^5 entries take four dependent loads instead of seventeen.
+__device__ __forceinline__ u64 warp_find(const u64* pref, u64 n, u64 v, u32 lane)
+{
+    u64 lo = 0;
+    while (n > 1) {
+        const u64 step = (n + 31) / 32, at = lane * step;
+        const bool le = at < n && pref[lo + at] <= v;
+        const u64 c = (u64)__popc(__ballot_sync(0xffffffffu, le)) - 1;   // lane 0's is true
+        lo += c * step;
+        n = pc_min(step, n - c * step);
+    }
+    return lo;
 }
 
 // the last index k < n with pref[k] <= v (pref ascending, pref[0] <= v)

@@ -38,7 +38,6 @@ struct LeafArgs {
     const u64* primes_rcp;   // floor((2^64 - 1) / p_k)
     const u64* primes_dv;    // p_k and its 32-bit reciprocal (div_dv)
     const uint2* podd;       // odd-number pi table (pi_odd) over [0, y]
-    u64 n_lim;   // list entries with m <= y: [0, n_lim)
     // easy-leaf gathers from the sampled table of Section 2.1 instead of the pi table
     const u32* samp;
     u32 samp_s;
@@ -65,7 +64,7 @@ __device__ __forceinline__ u64 pi_sampled(const LeafArgs& A, u64 v, u64* pv)
 // more of a run in one lane, short ones balance the warps when there are few
 PC_HD u32 clust_chunk_for(u64 x) { return x >= 100000000000000000ull ? 16384 : 8192; }
 
-static LeafArgs make_args(pc_ctx* ctx, const LeafProblem& P, u64 n_lim)
+static LeafArgs make_args(pc_ctx* ctx, const LeafProblem& P)
 {
     LeafArgs A;
     A.x = P.x;
@@ -85,7 +84,6 @@ static LeafArgs make_args(pc_ctx* ctx, const LeafProblem& P, u64 n_lim)
     A.primes_rcp = ctx->T.primes_rcp.as<u64>();
     A.primes_dv = ctx->T.primes_dv.as<u64>();
     A.podd = ctx->T.pi_odd.as<uint2>();
-    A.n_lim = n_lim;
     A.samp = ctx->T.samp.as<u32>();
     A.samp_s = ctx->T.samp_s;
     A.sampled = ctx->params.pi_gather == 1;
@@ -93,102 +91,62 @@ static LeafArgs make_args(pc_ctx* ctx, const LeafProblem& P, u64 n_lim)
     return A;
 }
 
-// list index range of entries with m <= y
-__global__ void rank_of_kernel(RankTable rk, u64 v, u64* out) { *out = rank_lookup(rk, v); }
-
-static int list_count_upto(pc_ctx* ctx, u64 y, u64* n)
-{
-    PC_TRY(buf_reserve(ctx, ctx->misc, 64 * sizeof(u64)));
-    rank_of_kernel<<<1, 1, 0, ctx->stream>>>(ctx->T.rank(), y, ctx->misc.as<u64>());
-    PC_LAUNCHED(ctx);
-    ctx->stats.kernel_launches++;
-    return copy_to_host(ctx, n, ctx->misc.p, sizeof(u64));
-}
-
 static int grid_for(pc_ctx* ctx) { return ctx->sm_count * 4; }
 
-// ------------------------------------------------------------------- S1
-__global__ void s1_kernel(LeafArgs A, const u32* phiT, u32 Q, I128Pair* part)
+// -------------------------------------------------------- S1 and trivial
+// One pass over the list entries m <= y for both sums.  S1 adds mu(m) phi(x/m, c).  For m the
+// trivial leaves are the b with max(c, pi(T)) < b < lpf_index(m), b <= a,
+// T = max(y/m, isqrt(x/m)): p_b > y/m makes m > y/p_b, and p_b > isqrt(x/m) makes
+// p_b^2 m > x, i.e. u < p_b.  None when lpf(m)^2 <= x/m, as for most composite m.
+__global__ void s1_trivial_kernel(LeafArgs A, const u32* phiT, u32 Q, u64 rcpQ, I128Pair* out_s1, I128Pair* out_tr)
 {
     __shared__ i128 scratch[32];
+    const u64 n_lim = rank_lookup(A.rk, A.y);   // list entries with m <= y
     i128 s = 0;
+    i64 tr = 0;
     auto phic = [&](u64 v) -> u64 {
         if (A.c == 0) return v;
-        u64 q = v / Q;
-        u32 r = (u32)(v - q * Q);
-        return q * phiT[Q] + phiT[r + 1];
+        const u64 q = div_rcp(v, Q, rcpQ);
+        return q * phiT[Q] + phiT[(u32)(v - q * Q) + 1];
     };
-    u64 tid = (u64)blockIdx.x * blockDim.x + threadIdx.x;
+    const u64 tid = (u64)blockIdx.x * blockDim.x + threadIdx.x;
     if (tid == 0) s += (i128)phic(A.x);   // n = 1
-    for (u64 i = tid; i < A.n_lim; i += (u64)gridDim.x * blockDim.x) {
-        u32 info = A.ml.info[i];
-        if ((info >> 1) <= A.c) continue;
+    for (u64 i = tid; i < n_lim; i += (u64)gridDim.x * blockDim.x) {
+        const u32 info = A.ml.info[i];
+        const u64 k = info >> 1;
+        if (k <= A.c) continue;
         if (A.trunc && A.ml.gpf[i] > A.a) continue;
-        u64 m = A.ml.m[i];
-        u64 f = phic(A.x / m);
+        const u64 m = A.ml.m[i], rc = A.ml.rcp[i], xm = div_rcp(A.x, m, rc);
+        const u64 f = phic(xm);
         if (info & 1) s -= (i128)f; else s += (i128)f;
+        if (k <= A.c + 1) continue;
+        const u64 lp = A.primes[k];
+        if (lp * lp <= xm) continue;
+        const u64 T = pc_max(div_rcp(A.y, m, rc), pc_isqrt(xm));
+        const u64 hi = pc_min(k - 1, A.a);
+        u64 lo = A.c;
+        if (T >= 2) lo = pc_max(lo, pi_lookup(A.pit, T));
+        if (hi > lo) tr += (info & 1) ? (i64)(hi - lo) : -(i64)(hi - lo);
     }
     s = block_sum_i128(s, scratch);
-    if (threadIdx.x == 0) store_i128(part + blockIdx.x, s);
+    if (threadIdx.x == 0 && s != 0) mq_atomic_add_i128(out_s1, s);
+    const i128 t = block_sum_i128((i128)tr, scratch);
+    if (threadIdx.x == 0 && t != 0) mq_atomic_add_i128(out_tr, t);
 }
 
-int run_s1(pc_ctx* ctx, const LeafProblem& P, I128Pair* out)
+int run_s1_trivial(pc_ctx* ctx, const LeafProblem& P, I128Pair* out_s1, I128Pair* out_tr)
 {
     PC_TRY(tables_phi_c(ctx, P.c));
-    u64 n_lim = 0;
-    PC_TRY(list_count_upto(ctx, P.y, &n_lim));
-    int g = grid_for(ctx);
-    PC_TRY(buf_reserve(ctx, ctx->partials, g * sizeof(I128Pair)));
     u32 Q = 1;
     static const u32 P8[8] = {1, 2, 3, 5, 7, 11, 13, 17};
     for (u32 i = 1; i <= P.c; i++) Q *= P8[i];
-    s1_kernel<<<g, 256, 0, ctx->stream>>>(make_args(ctx, P, n_lim), P.c ? ctx->T.phiT[P.c].as<u32>() : nullptr, Q,
-                                          ctx->partials.as<I128Pair>());
+    // a thread per eight integers up to y (about one list entry), up to four CTAs per SM
+    const int g = (int)pc_min((u64)grid_for(ctx), P.y / 2048 + 1);
+    s1_trivial_kernel<<<g, 256, 0, ctx->stream>>>(make_args(ctx, P), P.c ? ctx->T.phiT[P.c].as<u32>() : nullptr, Q,
+                                                  ~0ull / Q, out_s1, out_tr);
     PC_LAUNCHED(ctx);
     ctx->stats.kernel_launches++;
-    return reduce_i128(ctx, ctx->partials.as<I128Pair>(), g, out);
-}
-
-// -------------------------------------------------------------- trivial
-// For m the trivial leaves are the b with max(c, pi(T)) < b < lpf_index(m),
-// b <= a, T = max(y/m, isqrt(x/m)): p_b > y/m makes m > y/p_b, and
-// p_b > isqrt(x/m) makes p_b^2 m > x, i.e. u < p_b.
-__global__ void trivial_kernel(LeafArgs A, I128Pair* part)
-{
-    __shared__ i128 scratch[32];
-    i64 s = 0;
-    for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < A.n_lim; i += (u64)gridDim.x * blockDim.x) {
-        u32 info = A.ml.info[i];
-        u64 k = info >> 1;
-        if (k <= A.c + 1) continue;
-        if (A.trunc && A.ml.gpf[i] > A.a) continue;
-        u64 m = A.ml.m[i];
-        u64 T = pc_max(A.y / m, pc_isqrt(A.x / m));
-        u64 hi = pc_min(k - 1, A.a);
-        u64 lo = A.c;
-        if (T >= 2) {
-            u64 pt = pi_lookup(A.pit, T);
-            if (pt > lo) lo = pt;
-        }
-        if (hi > lo) {
-            i64 cnt = (i64)(hi - lo);
-            s += (info & 1) ? cnt : -cnt;
-        }
-    }
-    i128 v = block_sum_i128((i128)s, scratch);
-    if (threadIdx.x == 0) store_i128(part + blockIdx.x, v);
-}
-
-int run_trivial(pc_ctx* ctx, const LeafProblem& P, I128Pair* out)
-{
-    u64 n_lim = 0;
-    PC_TRY(list_count_upto(ctx, P.y, &n_lim));
-    int g = grid_for(ctx);
-    PC_TRY(buf_reserve(ctx, ctx->partials, g * sizeof(I128Pair)));
-    trivial_kernel<<<g, 256, 0, ctx->stream>>>(make_args(ctx, P, n_lim), ctx->partials.as<I128Pair>());
-    PC_LAUNCHED(ctx);
-    ctx->stats.kernel_launches++;
-    return reduce_i128(ctx, ctx->partials.as<I128Pair>(), g, out);
+    return PC_OK;
 }
 
 // ----------------------------------------------------------------- easy
@@ -301,14 +259,6 @@ __global__ void easy_ranges_kernel(LeafArgs A, u64 b_lo, u64 nb, u32 what, u64 u
     const EasyRange r = easy_range(A, A.x, A.y, A.a, b_lo + t, what, u_lo, u_hi);
     rng[t] = r;
     nchunk[t] = (u32)easy_chunks(r, A.clust_chunk);
-}
-
-// chunk -> index t = b - b_lo of the prime whose leaves it holds
-__global__ void easy_chunk_map_kernel(u64 nb, const u64* choff, u32* cmap)
-{
-    const u64 t = (u64)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= nb) return;
-    for (u64 ch = choff[t]; ch < choff[t + 1]; ch++) cmap[ch] = (u32)t;
 }
 
 // How an easy leaf reads pi(u): from the popcount pi table (PI_REC), from the
@@ -529,10 +479,11 @@ __device__ __forceinline__ void easy_chunk(const LeafArgs& A, u64 x, u64 a, u64 
 
 // MODE: how pi(u) is read (PI_REC, PI_SAMPLED, PI_ODD)
 template <int MODE>
-__global__ void easy_kernel(LeafArgs A, u64 b_lo, const EasyRange* rng, const u64* choff, const u32* cmap,
-                            u64 nchunks, unsigned long long* queue, I128Pair* part, unsigned long long* stat)
+__global__ void easy_kernel(LeafArgs A, u64 b_lo, u64 nb, const EasyRange* rng, const u64* choff,
+                            unsigned long long* queue, I128Pair* out, unsigned long long* stat)
 {
     __shared__ i128 scratch[32];
+    const u64 nchunks = choff[nb];
     const u32 lane = threadIdx.x & 31;
     i64 s = 0;
     u32 n_table = 0, n_one = 0, n_runs = 0, n_run_leaves = 0;   // hard leaves from the table, leaves one at a time,
@@ -543,7 +494,7 @@ __global__ void easy_kernel(LeafArgs A, u64 b_lo, const EasyRange* rng, const u6
         if (lane == 0) ch = atomicAdd(queue, 1ull);
         ch = __shfl_sync(0xffffffffu, ch, 0);
         if (ch >= nchunks) break;
-        const u64 t = cmap[ch];
+        const u64 t = warp_find(choff, nb, ch, lane);   // the prime whose leaves the chunk holds
         const EasyRange r = rng[t];
         easy_chunk<MODE>(A, A.x, A.a, b_lo + t, r, ch - choff[t], A.clust_chunk, lane, s, n_table, n_one, n_runs,
                             n_run_leaves);
@@ -559,7 +510,7 @@ __global__ void easy_kernel(LeafArgs A, u64 b_lo, const EasyRange* rng, const u6
         }
     }
     i128 v = block_sum_i128((i128)s, scratch);
-    if (threadIdx.x == 0) store_i128(part + blockIdx.x, v);
+    if (threadIdx.x == 0 && v != 0) mq_atomic_add_i128(out, v);
 }
 
 // The leaves of the primes b_lo <= b < b_lo + nb (see easy_range for what, u_lo, u_hi)
@@ -570,7 +521,7 @@ static int leaf_pass(pc_ctx* ctx, const LeafProblem& P, u64 b_lo, u64 nb, u32 wh
     PC_TRY(buf_reserve(ctx, ctx->easy_chunk_off, (nb + 1) * sizeof(u64) + (nb + 1) * sizeof(u32)));
     u64* choff = ctx->easy_chunk_off.as<u64>();
     u32* nch = (u32*)(choff + nb + 1);
-    LeafArgs A = make_args(ctx, P, 0);
+    LeafArgs A = make_args(ctx, P);
     const bool odd = !A.sampled && P.y < PI_ODD_Y && ctx->T.podd_limit >= P.y;
     if (odd) A.clust_chunk = 0;   // clustered chunks by pi value
     easy_ranges_kernel<<<(unsigned)((nb + 255) / 256), 256, 0, ctx->stream>>>(A, b_lo, nb, what, u_lo, u_hi,
@@ -578,50 +529,33 @@ static int leaf_pass(pc_ctx* ctx, const LeafProblem& P, u64 b_lo, u64 nb, u32 wh
     PC_LAUNCHED(ctx);
     ctx->stats.kernel_launches++;
     PC_TRY(scan_exclusive_u32_to_u64(ctx, nch, choff, nb));
-    u64 nchunks = 0;
-    PC_TRY(copy_to_host(ctx, &nchunks, choff + nb, sizeof(u64)));
-    if (nchunks == 0) return PC_OK;
-    if (nchunks >> 32) {
-        pc_set_error(ctx, "easy leaves: %llu chunks", (unsigned long long)nchunks);
-        return PC_EOVERFLOW;
-    }
-    PC_TRY(buf_reserve(ctx, ctx->easy_cmap, nchunks * sizeof(u32)));
-    easy_chunk_map_kernel<<<(unsigned)((nb + 255) / 256), 256, 0, ctx->stream>>>(nb, choff,
-                                                                                 ctx->easy_cmap.as<u32>());
-    PC_LAUNCHED(ctx);
-    ctx->stats.kernel_launches++;
-    int g = (int)pc_min((u64)ctx->sm_count * 8, nchunks);
-    PC_TRY(buf_reserve(ctx, ctx->partials, g * sizeof(I128Pair)));
-    PC_TRY(buf_reserve(ctx, ctx->queue, 64));
-    PC_CUDA(ctx, cudaMemsetAsync(ctx->queue.p, 0, 64, ctx->stream));
     const bool timed = what != LEAVES_TABLE;
+    // the number of chunks stays on the device: warps take them from a queue
+    const int g = (int)pc_min((u64)ctx->sm_count * 8, nb);
     if (timed) PC_CUDA(ctx, cudaEventRecord(ctx->ev[2], ctx->stream));
     const EasyRange* rng = ctx->easy_rng.as<EasyRange>();
-    const u32* cmap = ctx->easy_cmap.as<u32>();
-    unsigned long long* queue = (unsigned long long*)ctx->queue.p;
+    unsigned long long* queue = call_queue(ctx, timed ? Q_EASY : Q_TABLE);
     if (A.sampled)
-        easy_kernel<PI_SAMPLED><<<g, 256, 0, ctx->stream>>>(A, b_lo, rng, choff, cmap, nchunks, queue,
-                                                            ctx->partials.as<I128Pair>(), ctx->dstat);
+        easy_kernel<PI_SAMPLED><<<g, 256, 0, ctx->stream>>>(A, b_lo, nb, rng, choff, queue, out, ctx->dstat);
     else if (odd)
-        easy_kernel<PI_ODD><<<g, 256, 0, ctx->stream>>>(A, b_lo, rng, choff, cmap, nchunks, queue,
-                                                        ctx->partials.as<I128Pair>(), ctx->dstat);
+        easy_kernel<PI_ODD><<<g, 256, 0, ctx->stream>>>(A, b_lo, nb, rng, choff, queue, out, ctx->dstat);
     else
-        easy_kernel<PI_REC><<<g, 256, 0, ctx->stream>>>(A, b_lo, rng, choff, cmap, nchunks, queue,
-                                                        ctx->partials.as<I128Pair>(), ctx->dstat);
+        easy_kernel<PI_REC><<<g, 256, 0, ctx->stream>>>(A, b_lo, nb, rng, choff, queue, out, ctx->dstat);
     PC_LAUNCHED(ctx);
     if (timed) {
         PC_CUDA(ctx, cudaEventRecord(ctx->ev[3], ctx->stream));
         ctx->easy_timed = true;
     }
     ctx->stats.kernel_launches++;
-    return reduce_i128(ctx, ctx->partials.as<I128Pair>(), g, out);
+    return PC_OK;
 }
 
 int run_easy(pc_ctx* ctx, const LeafProblem& P, I128Pair* out)
 {
     const u64 b_lo = (u64)P.c + 1;
-    if (P.a < b_lo) return PC_OK;
-    return leaf_pass(ctx, P, b_lo, P.a - b_lo + 1, P.table_in_easy ? LEAVES_BOTH : LEAVES_EASY, 0, ~0ull, out);
+    const u64 b_hi = pc_min(P.a, P.E);
+    if (b_hi < b_lo) return PC_OK;
+    return leaf_pass(ctx, P, b_lo, b_hi - b_lo + 1, P.table_in_easy ? LEAVES_BOTH : LEAVES_EASY, 0, ~0ull, out);
 }
 
 int run_hard_table(pc_ctx* ctx, const LeafProblem& P, u64 b_min, u64 u_lo, u64 u_hi, I128Pair* out)
@@ -670,7 +604,7 @@ int run_hard_smallb(pc_ctx* ctx, const LeafProblem& P, I128Pair* out)
     int g = grid_for(ctx);
     PC_TRY(buf_reserve(ctx, ctx->partials, g * sizeof(I128Pair)));
     PC_CUDA(ctx, cudaMemsetAsync(ctx->partials.p, 0, g * sizeof(I128Pair), ctx->stream));
-    LeafArgs A = make_args(ctx, P, 0);
+    LeafArgs A = make_args(ctx, P);
     for (u64 b = (u64)P.c + 1; b <= 3 && b <= P.a; b++) {
         PC_TRY(buf_reserve(ctx, ctx->misc, 64 * sizeof(u64)));
         smallb_range_kernel<<<1, 1, 0, ctx->stream>>>(A, b, ctx->misc.as<u64>());
@@ -696,7 +630,7 @@ static LeafArgs table_args(pc_ctx* ctx)
 {
     LeafProblem P{};
     P.x = 0;
-    return make_args(ctx, P, 0);
+    return make_args(ctx, P);
 }
 
 // per query: pi(y), pi(isqrt z), pi(isqrt x), the m-list entries up to y, pi(iroot3 x);
@@ -811,8 +745,8 @@ __global__ void mq_easy_kernel(LeafArgs T, const MQ* qs, const u64* pref, u32 Q,
         if (lane == 0) ch = atomicAdd(queue, 1ull);
         ch = __shfl_sync(0xffffffffu, ch, 0);
         if (ch >= nchunks) break;
-        const u64 g = mq_find(choff, npairs + 1, ch);   // the pair of the chunk
-        const u64 q = mq_find(pref, Q + 1, g);
+        const u64 g = warp_find(choff, npairs, ch, lane);   // the pair of the chunk
+        const u64 q = warp_find(pref, Q, g, lane);
         const MQ m = qs[q];
         const EasyRange r = rng[g];
         i64 s = 0;

@@ -293,8 +293,10 @@ __global__ void __launch_bounds__(NT, 4) p2_sieve_kernel(P2Args A0, P2Multi M)
     }
 }
 
-// sum_s acc[s] + tally[s] * phi(L_s - 1, B), phi(L_s - 1, B) = sum_{s'<s} cnt[s']
-__global__ void p2_combine_kernel(P2Args A, I128Pair* out)
+// sum_s acc[s] + tally[s] * phi(L_s - 1, B), phi(L_s - 1, B) = sum_{s'<s} cnt[s'], and the
+// constant part of P2, (K - a)(B - 1) - sum_{k=a+1}^{K} (k - 1), K = pi(isqrt x): every
+// pi(x/p_k) = phi(x/p_k, B) + B - 1 and pi(p_k) = k.
+__global__ void p2_combine_kernel(P2Args A, u64 K, u64 a, I128Pair* out)
 {
     __shared__ u64 wsum[32];
     __shared__ u64 s_carry;
@@ -339,7 +341,10 @@ __global__ void p2_combine_kernel(P2Args A, I128Pair* out)
         __syncthreads();
     }
     dot = block_sum_i128(dot, red);
-    if (threadIdx.x == 0) store_i128(out, load_i128(out) + dot);
+    if (threadIdx.x == 0) {
+        const i128 sum_k1 = ((i128)K * (i128)(K - 1) - (i128)a * (i128)(a ? a - 1 : 0)) / 2;   // sum_{k=a+1}^{K} (k - 1)
+        store_i128(out, load_i128(out) + dot + (i128)(K - a) * (i128)(A.B - 1) - sum_k1);
+    }
 }
 
 // tiny z (fewer than 3 sieving primes): every pi(x/p) straight from the pi table
@@ -354,15 +359,6 @@ __global__ void p2_lookup_kernel(u64 x, u64 y, u64 r, PiTable pit, I128Pair* out
     }
     s = block_sum_i128(s, red);
     if (threadIdx.x == 0) store_i128(out, load_i128(out) + s);
-}
-
-// The constant part of P2, (K - a)(B - 1) - sum_{k=a+1}^{K} (k - 1), K = pi(isqrt x),
-// B = pi(isqrt z), added to *out: every pi(x/p_k) = phi(x/p_k, B) + B - 1 and pi(p_k) = k.
-__global__ void p2_constant_kernel(u64 K, u64 a, u64 B, I128Pair* out)
-{
-    const i128 n = (i128)(K - a);
-    const i128 sum_k1 = ((i128)K * (i128)(K - 1) - (i128)a * (i128)(a ? a - 1 : 0)) / 2;   // sum_{k=a+1}^{K} (k - 1)
-    store_i128(out, load_i128(out) + n * (i128)(B - 1) - sum_k1);
 }
 
 // ------------------------------------------------------------- bucket sieve
@@ -542,14 +538,26 @@ static int run_p2_buckets(pc_ctx* ctx, const P2Args& A, int ctas, size_t smem)
     return PC_OK;
 }
 
-int run_p2(pc_ctx* ctx, u64 x, u64 y, u64 a, I128Pair* out)
+static u32 p2_seg(pc_ctx* ctx, u64 z) { return pc_seg_bytes(ctx, ctx->params.p2_bucket ? 4096 : p2_seg_for(z)); }
+
+int p2_ask(pc_ctx* ctx, u64 x, u64 y, u64* v)
+{
+    const u64 z = x / y;
+    const u32 seg = p2_seg(ctx, z);
+    int n = 0;
+    v[n++] = pc_isqrt(x);
+    v[n++] = pc_isqrt(z);
+    v[n++] = p2_coop_p(seg) - 1;
+    v[n++] = seg / 8;
+    if (ctx->params.p2_bucket) v[n++] = seg;
+    return n;
+}
+
+int run_p2(pc_ctx* ctx, u64 x, u64 y, u64 a, const u64* pv, I128Pair* out)
 {
     const u64 r = pc_isqrt(x);
     if (r <= y) return PC_OK;
     const u64 z = x / y;
-    u64 vals[3] = {r, pc_isqrt(z), 0};
-    u64 pv[3];
-    PC_TRY(tables_pi_values(ctx, vals, pv, 2));
     const u64 K = pv[0], B = pv[1];
     if (K <= a) return PC_OK;
     if (B < 3) {
@@ -573,36 +581,26 @@ int run_p2(pc_ctx* ctx, u64 x, u64 y, u64 a, I128Pair* out)
         A.pat = ctx->T.wheel19.as<u32>();
     }
     const bool bucket = ctx->params.p2_bucket != 0;
-    A.seg_bytes = pc_seg_bytes(ctx, bucket ? 4096 : p2_seg_for(A.z));
+    A.seg_bytes = p2_seg(ctx, z);
     A.span = 30ull * A.seg_bytes;
-    {
-        u64 v2[2] = {p2_coop_p(A.seg_bytes) - 1, A.seg_bytes / 8}, pv2[2];
-        PC_TRY(tables_pi_values(ctx, v2, pv2, 2));
-        A.b_mid = (u32)pc_min(pc_max(pv2[0] + 1, (u64)A.k0 + 1), B + 1);
-        A.b_big = (u32)pc_min(pc_max(pv2[1] + 1, (u64)A.b_mid), B + 1);
-    }
+    A.b_mid = (u32)pc_min(pc_max(pv[2] + 1, (u64)A.k0 + 1), B + 1);
+    A.b_big = (u32)pc_min(pc_max(pv[3] + 1, (u64)A.b_mid), B + 1);
     A.s0 = r / A.span;                   // r <= z since y < r
     A.nseg = z / A.span + 1 - A.s0;
     A.bkt = nullptr;
     A.bkt_n = nullptr;
     A.bkt_cap = 0;
     A.b_bkt = (u32)B + 1;
-    if (bucket) {   // bucket primes: p > seg_bytes, at most one multiple per residue class in a segment
-        u64 v1 = A.seg_bytes, pv1 = 0;
-        PC_TRY(tables_pi_values(ctx, &v1, &pv1, 1));
-        A.b_bkt = (u32)pc_min(pc_max(pv1 + 1, (u64)A.b_big), B + 1);
-    }
+    if (bucket)   // bucket primes: p > seg_bytes, at most one multiple per residue class in a segment
+        A.b_bkt = (u32)pc_min(pc_max(pv[4] + 1, (u64)A.b_big), B + 1);
     A.pit = ctx->T.pi();
     A.primes = ctx->T.primes.as<u32>();
     A.primes_rcp = ctx->T.primes_rcp.as<u64>();
-    PC_TRY(buf_reserve(ctx, ctx->counts, A.nseg * 2 * sizeof(u32)));
-    PC_TRY(buf_reserve(ctx, ctx->acc_seg, A.nseg * sizeof(I128Pair)));
-    PC_TRY(buf_reserve(ctx, ctx->queue, 64));
-    PC_CUDA(ctx, cudaMemsetAsync(ctx->queue.p, 0, 64, ctx->stream));
-    A.cnt = ctx->counts.as<u32>();
+    PC_TRY(buf_reserve(ctx, ctx->p2_seg, A.nseg * (sizeof(I128Pair) + 2 * sizeof(u32))));
+    A.acc = ctx->p2_seg.as<I128Pair>();
+    A.cnt = (u32*)(A.acc + A.nseg);
     A.tally = A.cnt + A.nseg;
-    A.acc = ctx->acc_seg.as<I128Pair>();
-    A.queue = ctx->queue.as<u32>();
+    A.queue = (u32*)call_queue(ctx, Q_P2);
     const u32 nblk = A.seg_bytes >> 7;
     size_t smem = A.seg_bytes + (2 * (size_t)nblk + 2) * sizeof(u32);
     // the kernel's limit is shared by every host thread: set the device maximum
@@ -634,11 +632,9 @@ int run_p2(pc_ctx* ctx, u64 x, u64 y, u64 a, I128Pair* out)
         PC_CUDA(ctx, cudaEventRecord(ctx->ev[5], ctx->stream));
     }
     ctx->p2_timed = true;
-    p2_combine_kernel<<<1, 1024, 0, ctx->stream>>>(A, out);
+    p2_combine_kernel<<<1, 1024, 0, ctx->stream>>>(A, K, a, out);
     PC_LAUNCHED(ctx);
-    p2_constant_kernel<<<1, 1, 0, ctx->stream>>>(K, a, B, out);
-    PC_LAUNCHED(ctx);
-    ctx->stats.kernel_launches += 3;
+    ctx->stats.kernel_launches += 2;
     return PC_OK;
 }
 

@@ -923,28 +923,36 @@ int tables_ensure(pc_ctx* ctx, u64 pi_limit, u64 prime_limit, u64 ml_limit, u32 
     return PC_OK;
 }
 
-__global__ void pi_values_kernel(PiTable t, const u64* v, u64* out, int n)
+struct PiAsk {
+    u64 v[PI_ASK_MAX];
+};
+
+__global__ void pi_values_kernel(PiTable t, PiAsk ask, u64* out, int n)
 {
     int i = threadIdx.x;
-    if (i < n) out[i] = pi_lookup(t, v[i]);
+    if (i < n) out[i] = pi_lookup(t, ask.v[i]);
 }
 
 int tables_pi_values(pc_ctx* ctx, const u64* v, u64* out, int n)
 {
-    if (n > 32) return PC_EINVAL;
+    if (n > PI_ASK_MAX) return PC_EINVAL;
+    PiAsk ask{};
     for (int i = 0; i < n; i++)
         if (v[i] > ctx->T.pi_limit) {
             pc_set_error(ctx, "pi lookup %llu beyond table %llu", (unsigned long long)v[i],
                          (unsigned long long)ctx->T.pi_limit);
             return PC_EINVAL;
         }
-    PC_TRY(buf_reserve(ctx, ctx->misc, 64 * sizeof(u64)));
-    u64* d = ctx->misc.as<u64>();
-    PC_CUDA(ctx, cudaMemcpyAsync(d, v, n * sizeof(u64), cudaMemcpyHostToDevice, ctx->stream));
-    pi_values_kernel<<<1, 32, 0, ctx->stream>>>(ctx->T.pi(), d, d + 32, n);
+    for (int i = 0; i < n; i++) ask.v[i] = v[i];
+    // the arguments travel with the launch and the results straight to the pinned staging
+    // memory: one launch and one wait
+    u64* h = (u64*)ctx->host_stage;
+    pi_values_kernel<<<1, 32, 0, ctx->stream>>>(ctx->T.pi(), ask, h, n);
     PC_LAUNCHED(ctx);
     ctx->stats.kernel_launches++;
-    return copy_to_host(ctx, out, d + 32, n * sizeof(u64));
+    PC_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    for (int i = 0; i < n; i++) out[i] = h[i];
+    return PC_OK;
 }
 
 __global__ void pi_many_kernel(PiTable t, const u64* v, u64* out, u64 n)

@@ -118,7 +118,7 @@ __global__ void scan_sums_one_cta(TO* sums, u64 m)
 }
 
 template <class TO>
-__global__ void scan_tiles(const u32* in, TO* out, u64 n, const TO* sums)
+__global__ void scan_tiles(const u32* in, TO* out, u64 n, const TO* sums)   // and out[n] = the total
 {
     __shared__ TO wsum[SCAN_THREADS / 32];
     __shared__ TO carry;
@@ -152,19 +152,59 @@ __global__ void scan_tiles(const u32* in, TO* out, u64 n, const TO* sums)
         if (threadIdx.x == SCAN_THREADS - 1) carry = c0 + wsum[wid] + incl;
         __syncthreads();
     }
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[n] = sums[gridDim.x];
 }
 
+// short arrays: one CTA, one launch (4 launches for the phases above cost more than the scan)
+static constexpr u64 SCAN_ONE = 16384;
 template <class TO>
-__global__ void scan_write_total(TO* out, u64 n, const TO* sums, u64 m)
+__global__ void __launch_bounds__(1024) scan_one_kernel(const u32* in, TO* out, u64 n)
 {
-    out[n] = sums[m];
+    __shared__ TO wsum[32];
+    __shared__ TO carry;
+    const u32 lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (threadIdx.x == 0) carry = 0;
+    __syncthreads();
+    for (u64 base = 0; base < n; base += 1024) {
+        const u64 i = base + threadIdx.x;
+        const TO v = i < n ? (TO)in[i] : 0;
+        TO incl = v;
+        for (int o = 1; o < 32; o <<= 1) {
+            const TO t = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += t;
+        }
+        if (lane == 31) wsum[wid] = incl;
+        __syncthreads();
+        if (wid == 0) {
+            const TO w = wsum[lane];
+            TO wi = w;
+            for (int o = 1; o < 32; o <<= 1) {
+                const TO t = __shfl_up_sync(0xffffffffu, wi, o);
+                if (lane >= o) wi += t;
+            }
+            wsum[lane] = wi - w;
+        }
+        __syncthreads();
+        const TO c0 = carry;
+        if (i < n) out[i] = c0 + wsum[wid] + incl - v;
+        __syncthreads();
+        if (threadIdx.x == 1023) carry = c0 + wsum[wid] + incl;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) out[n] = carry;
 }
 
 template <class TO>
 static int scan_impl(pc_ctx* ctx, const u32* in, TO* out, u64 n)
 {
-    u64 tiles = (n + SCAN_TILE - 1) / SCAN_TILE;
-    if (tiles == 0) tiles = 1;
+    if (n <= SCAN_ONE) {
+        if (!mq_device_work(ctx)) return PC_OK;
+        scan_one_kernel<TO><<<1, 1024, 0, ctx->stream>>>(in, out, n);
+        PC_LAUNCHED(ctx);
+        ctx->stats.kernel_launches++;
+        return PC_OK;
+    }
+    const u64 tiles = (n + SCAN_TILE - 1) / SCAN_TILE;
     PC_TRY(buf_reserve(ctx, ctx->scan_tmp, (tiles + 1) * sizeof(TO)));
     TO* sums = ctx->scan_tmp.as<TO>();
     if (!mq_device_work(ctx)) return PC_OK;
@@ -174,9 +214,7 @@ static int scan_impl(pc_ctx* ctx, const u32* in, TO* out, u64 n)
     PC_LAUNCHED(ctx);
     scan_tiles<TO><<<(unsigned)tiles, SCAN_THREADS, 0, ctx->stream>>>(in, out, n, sums);
     PC_LAUNCHED(ctx);
-    scan_write_total<TO><<<1, 1, 0, ctx->stream>>>(out, n, sums, tiles);
-    PC_LAUNCHED(ctx);
-    ctx->stats.kernel_launches += 4;
+    ctx->stats.kernel_launches += 3;
     return PC_OK;
 }
 
