@@ -292,6 +292,19 @@ __device__ __forceinline__ u64 warp_find(const u64* pref, u64 n, u64 v, u32 lane
     return lo;
 }
 
+// The same for a v that never falls below the last call's, whose answer is hint: usually a
+// little ahead, two loads away.
+__device__ __forceinline__ u64 warp_find_from(const u64* pref, u64 n, u64 v, u32 lane, u64 hint)
+{
+    constexpr u64 step = 16;
+    const u64 at = hint + lane * step;
+    const u64 c = (u64)__popc(__ballot_sync(0xffffffffu, at < n && pref[at] <= v)) - 1;   // lane 0's is true
+    const u64 lo = hint + c * step;
+    if (c == 31) return lo + warp_find(pref + lo, n - lo, v, lane);   // past the window
+    const u64 m = pc_min(step, n - lo);
+    return lo + (u64)__popc(__ballot_sync(0xffffffffu, lane < m && pref[lo + lane] <= v)) - 1;
+}
+
 // the last index k < n with pref[k] <= v (pref ascending, pref[0] <= v)
 __device__ __forceinline__ u64 mq_find(const u64* pref, u64 n, u64 v)
 {

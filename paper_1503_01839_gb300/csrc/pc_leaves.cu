@@ -477,9 +477,11 @@ __device__ __forceinline__ void easy_chunk(const LeafArgs& A, u64 x, u64 a, u64 
     }
 }
 
-// MODE: how pi(u) is read (PI_REC, PI_SAMPLED, PI_ODD)
+// MODE: how pi(u) is read (PI_REC, PI_SAMPLED, PI_ODD).  Eight CTAs per SM (32 registers): the
+// gathers want every warp slot (pi(10^18), alpha 56: 18.6 ms; 20.3 with six CTAs at 40 registers,
+// 21.4 with five at 48).
 template <int MODE>
-__global__ void easy_kernel(LeafArgs A, u64 b_lo, u64 nb, const EasyRange* rng, const u64* choff,
+__global__ void __launch_bounds__(256, 8) easy_kernel(LeafArgs A, u64 b_lo, u64 nb, const EasyRange* rng, const u64* choff,
                             unsigned long long* queue, I128Pair* out, unsigned long long* stat)
 {
     __shared__ i128 scratch[32];
@@ -488,13 +490,16 @@ __global__ void easy_kernel(LeafArgs A, u64 b_lo, u64 nb, const EasyRange* rng, 
     i64 s = 0;
     u32 n_table = 0, n_one = 0, n_runs = 0, n_run_leaves = 0;   // hard leaves from the table, leaves one at a time,
                                                                 // runs, leaves in runs
-    // chunks are handed out one at a time to warps (their costs differ widely)
+    // chunks are handed out one at a time to warps (their costs differ widely), each asked for
+    // while the one before it is worked on
+    unsigned long long next = 0;
+    u64 t = 0;
+    if (lane == 0) next = atomicAdd(queue, 1ull);
     for (;;) {
-        u64 ch = 0;
-        if (lane == 0) ch = atomicAdd(queue, 1ull);
-        ch = __shfl_sync(0xffffffffu, ch, 0);
+        const u64 ch = __shfl_sync(0xffffffffu, next, 0);
         if (ch >= nchunks) break;
-        const u64 t = warp_find(choff, nb, ch, lane);   // the prime whose leaves the chunk holds
+        if (lane == 0) next = atomicAdd(queue, 1ull);
+        t = warp_find_from(choff, nb, ch, lane, t);   // the prime whose leaves the chunk holds
         const EasyRange r = rng[t];
         easy_chunk<MODE>(A, A.x, A.a, b_lo + t, r, ch - choff[t], A.clust_chunk, lane, s, n_table, n_one, n_runs,
                             n_run_leaves);
@@ -740,13 +745,15 @@ __global__ void mq_easy_kernel(LeafArgs T, const MQ* qs, const u64* pref, u32 Q,
 {
     const u32 lane = threadIdx.x & 31;
     const u64 nchunks = choff[npairs];
+    unsigned long long next = 0;
+    u64 g = 0, q = 0;
+    if (lane == 0) next = atomicAdd(queue, 1ull);
     for (;;) {
-        u64 ch = 0;
-        if (lane == 0) ch = atomicAdd(queue, 1ull);
-        ch = __shfl_sync(0xffffffffu, ch, 0);
+        const u64 ch = __shfl_sync(0xffffffffu, next, 0);
         if (ch >= nchunks) break;
-        const u64 g = warp_find(choff, npairs, ch, lane);   // the pair of the chunk
-        const u64 q = warp_find(pref, Q, g, lane);
+        if (lane == 0) next = atomicAdd(queue, 1ull);
+        g = warp_find_from(choff, npairs, ch, lane, g);   // the pair of the chunk
+        q = warp_find_from(pref, Q, g, lane, q);
         const MQ m = qs[q];
         const EasyRange r = rng[g];
         i64 s = 0;
