@@ -21,8 +21,10 @@
  *   - A context is not thread-safe: use one context per host thread.
  *   - Every function returns PC_OK (0) or a negative PC_E* code; the message
  *     of the last failure is available from pc_last_error().
- *   - All GPU work of a context runs on one CUDA stream (pc_set_stream), and
- *     each call synchronizes that stream before it returns.
+ *   - All GPU work of a context is ordered on one CUDA stream (pc_set_stream):
+ *     independent phases of one call may run beside it, on streams of the
+ *     context's own that wait for it and that it waits for, and each call
+ *     synchronizes that stream before it returns.
  */
 #ifndef PICOUNT_H
 #define PICOUNT_H
@@ -111,7 +113,8 @@ typedef struct pc_stats {
     uint64_t kernel_launches;
     double ms_tables, ms_s1, ms_trivial, ms_easy, ms_hard, ms_p2, ms_total;   /* ms_s1: the ordinary and the
                                trivial leaves (one kernel; ms_trivial stays 0).  The phases of a leaf-sum
-                               call are timed by CUDA events, ms_tables and ms_total on the host. */
+                               call are timed by CUDA events and may overlap; ms_tables and ms_total
+                               on the host. */
     double ms_hard_sieve;   /* the segmented sieve kernel alone (CUDA events) */
     uint64_t warp_steps;      /* (warp sub-range, prime) steps with work in the hard-leaf sieve */
     uint64_t leaf_warp_steps; /* of which resolved leaves */

@@ -79,8 +79,9 @@ extern "C" void pc_destroy(pc_ctx* ctx)
     if (ctx->stream) cudaStreamSynchronize(ctx->stream);
     workers_destroy(ctx);
     DevBuf* bufs[] = {&ctx->seg_b, &ctx->seg_off, &ctx->counts, &ctx->tallies,
-                      &ctx->acc_seg, &ctx->partials, &ctx->result, &ctx->misc, &ctx->scan_tmp,
-                      &ctx->easy_rng, &ctx->easy_chunk_off, &ctx->starts,
+                      &ctx->acc_seg, &ctx->partials, &ctx->result, &ctx->misc, &ctx->scan_tmp[0],
+                      &ctx->scan_tmp[1], &ctx->scan_tmp[2],
+                      &ctx->easy_rng[0], &ctx->easy_rng[1], &ctx->easy_chunk_off[0], &ctx->easy_chunk_off[1], &ctx->starts,
                       &ctx->mq_q, &ctx->mq_pref, &ctx->mq_e, &ctx->mq_h, &ctx->mq_hq, &ctx->mq_p,
                       &ctx->p2_seg, &ctx->p2_bkt};
     for (DevBuf* b : bufs) buf_free(*b);
@@ -98,6 +99,10 @@ extern "C" void pc_destroy(pc_ctx* ctx)
     if (ctx->ev_ok)
         for (int i = 0; i < 16; i++) cudaEventDestroy(ctx->ev[i]);
     if (ctx->host_stage) cudaFreeHost(ctx->host_stage);
+    for (cudaStream_t s : ctx->side)
+        if (s) cudaStreamDestroy(s);
+    for (cudaEvent_t e : {ctx->ev_fork, ctx->ev_join[0], ctx->ev_join[1]})
+        if (e) cudaEventDestroy(e);
     if (ctx->own_stream) cudaStreamDestroy(ctx->own_stream);
     delete ctx;
 }
@@ -149,17 +154,43 @@ static int result_slots(pc_ctx* ctx, I128Pair** d)
     *d = ctx->result.as<I128Pair>();
     ctx->dstat = call_dstat(ctx);
     ctx->hard_timed = ctx->easy_timed = ctx->p2_timed = false;
-    ctx->marks = 0;
     return PC_OK;
 }
 
-// the end of a phase, on the call's stream
-static int mark(pc_ctx* ctx)
+// --------------------------------------------------------- side streams
+static int sides_ensure(pc_ctx* ctx)
 {
-    PC_CUDA(ctx, cudaEventRecord(ctx->ev[6 + ctx->marks], ctx->stream));
-    ctx->marks++;
+    for (cudaStream_t& s : ctx->side)
+        if (!s) PC_CUDA(ctx, cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
+    for (cudaEvent_t* e : {&ctx->ev_fork, &ctx->ev_join[0], &ctx->ev_join[1]})
+        if (!*e) PC_CUDA(ctx, cudaEventCreateWithFlags(e, cudaEventDisableTiming));
     return PC_OK;
 }
+
+// Enqueues on side stream k until it goes out of scope; the side waits for the call's start
+// (ev_fork), and join() makes the call's stream wait for it.
+struct SideScope {
+    pc_ctx* ctx;
+    cudaStream_t main;
+    int k;
+    SideScope(pc_ctx* c, int kk) : ctx(c), main(c->stream), k(kk)
+    {
+        ctx->stream = ctx->side[k];
+        ctx->scan_sel = 1 + k;
+    }
+    ~SideScope()
+    {
+        ctx->stream = main;
+        ctx->scan_sel = 0;
+    }
+    int begin() { PC_CUDA(ctx, cudaStreamWaitEvent(ctx->side[k], ctx->ev_fork, 0)); return PC_OK; }
+    int join()
+    {
+        PC_CUDA(ctx, cudaEventRecord(ctx->ev_join[k], ctx->side[k]));
+        PC_CUDA(ctx, cudaStreamWaitEvent(main, ctx->ev_join[k], 0));
+        return PC_OK;
+    }
+};
 
 // the call's one wait for its results: parts, counters and kernel times
 static int read_slots(pc_ctx* ctx, int n, i128* out)
@@ -190,11 +221,7 @@ static int read_slots(pc_ctx* ctx, int n, i128* out)
     if (ctx->hard_timed && cudaEventElapsedTime(&ms, ctx->ev[0], ctx->ev[1]) == cudaSuccess) ctx->stats.ms_hard_sieve += ms;
     if (ctx->easy_timed && cudaEventElapsedTime(&ms, ctx->ev[2], ctx->ev[3]) == cudaSuccess) ctx->stats.ms_easy_kernel += ms;
     if (ctx->p2_timed && cudaEventElapsedTime(&ms, ctx->ev[4], ctx->ev[5]) == cudaSuccess) ctx->stats.ms_p2_kernel += ms;
-    double* phase[] = {&ctx->stats.ms_s1, &ctx->stats.ms_easy, &ctx->stats.ms_hard, &ctx->stats.ms_p2};
-    for (int i = 0; i + 1 < ctx->marks; i++)
-        if (cudaEventElapsedTime(&ms, ctx->ev[6 + i], ctx->ev[7 + i]) == cudaSuccess) *phase[i] += ms;
     ctx->hard_timed = ctx->easy_timed = ctx->p2_timed = false;
-    ctx->marks = 0;
     ctx->dstat = nullptr;
     return PC_OK;
 }
@@ -250,6 +277,51 @@ static u32 choose_seg(const pc_ctx* ctx, u64 x)
     return ctx->tuned_seg[decimal_digits(x)];
 }
 
+// One phase of a call on its stream, or on side stream k (0 or 1), between events ev[e], ev[e + 1]
+template <class F>
+static int timed_phase(pc_ctx* ctx, int e, int k, F&& enqueue)
+{
+    if (k < 0) {
+        PC_CUDA(ctx, cudaEventRecord(ctx->ev[e], ctx->stream));
+        PC_TRY(enqueue());
+        PC_CUDA(ctx, cudaEventRecord(ctx->ev[e + 1], ctx->stream));
+        return PC_OK;
+    }
+    SideScope side(ctx, k);
+    PC_TRY(side.begin());
+    PC_TRY(timed_phase(ctx, e, -1, enqueue));
+    return PC_OK;
+}
+
+// The phases of a leaf-sum call, all enqueued without a wait: the hard leaves on the call's
+// stream; below SIDES_Z, where no phase fills the chip, P2 and the other leaves beside them
+// (pi(3e7) 0.19 -> 0.11 ms, pi(1e12) 0.40 -> 0.26, pi(1e14) 0.72 -> 0.61; from z = 2e9 on
+// one after the other: pi(1e17) with P2 beside 16.8 ms against 15.4, and the easy leaves beside
+// the sieve, which leaves them no L1, gain nothing either, 67.6 and 62.5 against 61.4 ms at
+// pi(1e18) with a full grid and with two or three CTAs per SM).
+static constexpr u64 SIDES_Z = 2000000000ull;
+static int phases(pc_ctx* ctx, const LeafProblem& P, const u64* p2_pv)
+{
+    const bool sides = P.z < SIDES_Z;
+    I128Pair* d;
+    if (sides) PC_TRY(sides_ensure(ctx));
+    PC_TRY(result_slots(ctx, &d));
+    if (sides) PC_CUDA(ctx, cudaEventRecord(ctx->ev_fork, ctx->stream));
+    PC_TRY(timed_phase(ctx, 10, -1, [&]() -> int {
+        PC_TRY(run_hard_smallb(ctx, P, d + 3));
+        return run_hard_sieve(ctx, P, d + 3);
+    }));
+    if (p2_pv)
+        PC_TRY(timed_phase(ctx, 12, sides ? 1 : -1, [&] { return run_p2(ctx, P.x, P.y, P.a, p2_pv, d + 4); }));
+    PC_TRY(timed_phase(ctx, 6, sides ? 0 : -1, [&] { return run_s1_trivial(ctx, P, d + 0, d + 1); }));
+    PC_TRY(timed_phase(ctx, 8, sides ? 0 : -1, [&] { return run_easy(ctx, P, d + 2); }));
+    for (int k = 0; sides && k < (p2_pv ? 2 : 1); k++) {
+        SideScope side(ctx, k);
+        PC_TRY(side.join());
+    }
+    return PC_OK;
+}
+
 // Leaf decomposition of phi(x, a) and P2(x, a); a == 0 selects pi(y).
 // parts: S1, trivial, easy, hard, P2 (P2 only when want_p2).
 // total_only: the caller wants the sum of the leaves, not how it splits into easy and hard.
@@ -283,22 +355,19 @@ static int leaf_parts(pc_ctx* ctx, u64 x, u64 y, u32 c, u64 a, bool want_p2, boo
     ctx->stats.a = a;
     ctx->stats.B = B;
     ctx->stats.c = c;
-    I128Pair* d;
-    // the phases follow one another on the stream, with no wait in between
-    PC_TRY(result_slots(ctx, &d));
-    PC_TRY(mark(ctx));
-    PC_TRY(run_s1_trivial(ctx, P, d + 0, d + 1));
-    PC_TRY(mark(ctx));
-    PC_TRY(run_easy(ctx, P, d + 2));
-    PC_TRY(mark(ctx));
-    PC_TRY(run_hard_smallb(ctx, P, d + 3));
-    PC_TRY(run_hard_sieve(ctx, P, d + 3));
-    PC_TRY(mark(ctx));
-    if (want_p2) {
-        PC_TRY(run_p2(ctx, x, y, a, pv + 4, d + 4));
-        PC_TRY(mark(ctx));
+    int rc = phases(ctx, P, want_p2 ? pv + 4 : nullptr);
+    if (rc == PC_OK) rc = read_slots(ctx, 5, parts);
+    if (rc != PC_OK) {
+        // nothing of this call may still run when the next one takes its scratch
+        for (cudaStream_t s : ctx->side)
+            if (s) cudaStreamSynchronize(s);
+        cudaStreamSynchronize(ctx->stream);
+        return rc;
     }
-    PC_TRY(read_slots(ctx, 5, parts));
+    float ms = 0;
+    double* phase[] = {&ctx->stats.ms_s1, &ctx->stats.ms_easy, &ctx->stats.ms_hard, &ctx->stats.ms_p2};
+    for (int i = 0; i < (want_p2 ? 4 : 3); i++)
+        if (cudaEventElapsedTime(&ms, ctx->ev[6 + 2 * i], ctx->ev[7 + 2 * i]) == cudaSuccess) *phase[i] += ms;
     if (!want_p2) parts[4] = 0;
     if (a_out) *a_out = a;
     return PC_OK;

@@ -904,7 +904,7 @@ __device__ __forceinline__ u32 seg_b(u64 x, u64 s, u64 span, u32 bmax, const PiT
 
 // The segments of row b in [s0, s1), those with B_s >= b: first segment and number.
 // p_b^2 <= L + span - 1 from segment p_b^2 / span on, p_b^2 <= x / L up to L = x / p_b^2.
-__device__ __forceinline__ u32 row_range(u64 x, u64 p, u64 span, u64 nseg, u64 s0, u64 s1, u32* first)
+PC_HD u32 row_range(u64 x, u64 p, u64 span, u64 nseg, u64 s0, u64 s1, u32* first)
 {
     const u64 lo = pc_max(p * p / span, s0);
     const u64 hi = pc_min(pc_min(x / (p * p) / span + 1, nseg), s1);
@@ -1051,10 +1051,6 @@ u32 hard_seg_for(u64 z)
     return z < 400000ull ? 2048 : z < 280000000ull ? 8192 : z < 2000000000ull ? 16384 : 32768;
 }
 
-// count-row entries (8 bytes each with their tallies) up to which a run takes rows x segments as
-// their bound instead of reading the exact number back: 64 MiB
-static constexpr u64 ROWS_UNREAD = 1ull << 23;
-
 // bytes per warp sub-range: a power of two dividing seg_bytes, at most 16 warps
 static u32 pc_sub_bytes(pc_ctx* ctx, u32 seg_bytes, u32 dflt)
 {
@@ -1200,10 +1196,10 @@ __global__ void plan_scatter_kernel(PlanArgs P)
 }
 
 // The planner in one launch (one CTA) for up to PLAN_ONE segments: the same decisions, with the
-// buckets in shared memory.  Also the number of count-row entries, for the caller's statistics.
+// buckets in shared memory.
 // (Four launches and their gaps cost more than the work: pi(10^12) plans 26 segments.)
 static constexpr u64 PLAN_ONE = 8192;
-__global__ void __launch_bounds__(1024) plan_one_kernel(PlanArgs P, const u64* rows)
+__global__ void __launch_bounds__(1024) plan_one_kernel(PlanArgs P)
 {
     __shared__ double part[32];
     __shared__ u32 cnt[PLAN_BUCKETS], cur[PLAN_BUCKETS];
@@ -1242,7 +1238,6 @@ __global__ void __launch_bounds__(1024) plan_one_kernel(PlanArgs P, const u64* r
         P.scr->nitems = P.stat[4] = ok ? run : 0;
         P.stat[5] = steps;
         P.stat[6] = ok ? 0 : 1;
-        P.stat[8] = *rows;
     }
     __syncthreads();
     if (ok)
@@ -1358,6 +1353,11 @@ static int choose_hard_kernel(pc_ctx* ctx, const HardArgs& A, size_t smem, void 
                                        {hard_sieve_kernel<256, 4, MULTI>, 256, 4}};
     const int nt = 32 * (int)A.nw;
     const int want = (int)(ctx->params.ctas_per_sm ? ctx->params.ctas_per_sm : ctx->ctas_call);
+    if (!MULTI && ctx->hk.fn && ctx->hk.nt == nt && ctx->hk.smem == smem && ctx->hk.want == want) {
+        *out = (void (*)(HardArgs, MultiArgs))ctx->hk.fn;
+        *out_per_sm = ctx->hk.per_sm;
+        return PC_OK;
+    }
     void (*kern)(HardArgs, MultiArgs) = nullptr;
     int per_sm = 0;
     for (const Variant& v : variants) {
@@ -1399,7 +1399,27 @@ static int choose_hard_kernel(pc_ctx* ctx, const HardArgs& A, size_t smem, void 
     if (per_sm > 8) per_sm = 8;   // 32 KiB segments fit 4; smaller ones (autotuned, or set) up to 8
     *out = kern;
     *out_per_sm = per_sm;
+    if (!MULTI) {
+        ctx->hk.nt = nt, ctx->hk.smem = smem, ctx->hk.want = want;
+        ctx->hk.fn = (void*)kern, ctx->hk.per_sm = per_sm;
+    }
     return PC_OK;
+}
+
+// primes below 2^16 (a run's sieving primes are at most x^(1/4) < 55109), p_1 at index 1
+static const std::vector<u32>& host_primes()
+{
+    static const std::vector<u32> ps = [] {
+        std::vector<u32> v(1, 1);
+        std::vector<char> comp(65536, 0);
+        for (u32 i = 2; i < 65536; i++) {
+            if (comp[i]) continue;
+            v.push_back(i);
+            for (u64 j = (u64)i * i; j < 65536; j += i) comp[j] = 1;
+        }
+        return v;
+    }();
+    return ps;
 }
 
 int run_hard_sieve(pc_ctx* ctx, const LeafProblem& P, I128Pair* out)
@@ -1482,13 +1502,14 @@ int run_hard_sieve(pc_ctx* ctx, const LeafProblem& P, I128Pair* out)
         A.start = ctx->starts.as<u64>();
         PC_CUDA(ctx, cudaStreamSynchronize(ctx->stream));   // hstart is pageable memory of this call
     }
-    // The count and tally rows: rows x segments bounds them; where that is small the exact number
-    // stays on the device, and the launches below follow without a wait.
-    u64 total = ns * nrows;
-    if (total > ROWS_UNREAD || ns > PLAN_ONE) {
-        PC_TRY(copy_to_host(ctx, &total, off + nrows, sizeof(u64)));
-        ctx->stats.steps = total;
+    // entries of the count and tally rows, as the device lays them out
+    u64 total = 0;
+    const std::vector<u32>& hp = host_primes();
+    for (u64 b = A.k0; b <= bmax; b++) {
+        u32 first;
+        total += row_range(P.x, hp[b], A.span, A.nseg, A.s0, A.s1, &first);
     }
+    ctx->stats.steps = total;
     if (total >> 32) {
         pc_set_error(ctx, "hard-leaf sieve: %llu count rows exceed 32-bit offsets", (unsigned long long)total);
         return PC_EOVERFLOW;
@@ -1518,7 +1539,7 @@ int run_hard_sieve(pc_ctx* ctx, const LeafProblem& P, I128Pair* out)
     PlanArgs PA{segB, est, A.k0, (float)P.x, (float)P.z, A.span, A.s0, A.s1, 1.0 / (4.0 * ctas), cap,
                 scr, split, ditems, heavy, A.stat};
     if (ns <= PLAN_ONE) {
-        plan_one_kernel<<<1, 1024, 0, ctx->stream>>>(PA, off + nrows);
+        plan_one_kernel<<<1, 1024, 0, ctx->stream>>>(PA);
         PC_LAUNCHED(ctx);
         ctx->stats.kernel_launches++;
     } else {

@@ -107,13 +107,20 @@ struct pc_ctx {
     int device = 0;
     cudaStream_t stream = nullptr;   // stream every kernel of this context uses
     cudaStream_t own_stream = nullptr;
+    // Independent phases of one call run beside its stream: on side streams that wait for the
+    // call's start and that its stream waits for before the results are read (pc_engine.cu).
+    // While a phase is enqueued there, stream is the side stream and scan_sel its scan scratch.
+    cudaStream_t side[2] = {nullptr, nullptr};
+    cudaEvent_t ev_fork = nullptr, ev_join[2] = {nullptr, nullptr};
+    int scan_sel = 0;
     pc_params params{};
     int sm_count = 0;
     size_t smem_optin = 0;
     Tables T;
     // scratch (grow-only)
-    DevBuf seg_b, seg_off, counts, tallies, acc_seg, partials, result, misc, scan_tmp;
-    DevBuf easy_rng, easy_chunk_off, starts;
+    DevBuf seg_b, seg_off, counts, tallies, acc_seg, partials, result, misc, scan_tmp[3];
+    DevBuf easy_rng[2], easy_chunk_off[2];   // of the easy pass, of the table leaves' pass
+    DevBuf starts;
     DevBuf mq_q, mq_pref, mq_e, mq_h, mq_hq, mq_p;   // batched queries (pc_pi_count_batch)
     DevBuf p2_seg;   // P2: per-segment sums, counts and tallies
     DevBuf p2_bkt;   // P2 bucket sieve: the buckets of one wave of segments and their fill counts
@@ -139,7 +146,9 @@ struct pc_ctx {
     // leaves), beside the result slots; null outside a leaf-sum call
     unsigned long long* dstat = nullptr;
     bool hard_timed = false, easy_timed = false, p2_timed = false;   // ev[0..1] / ev[2..3] / ev[4..5] hold kernel times
-    int marks = 0;   // ev[6 ..] hold the ends of the call's phases
+    // the hard-leaf sieve's instantiation for the last (threads, shared memory, residency) asked for
+    struct { int nt = 0, want = -1, per_sm = 0; size_t smem = 0; void* fn = nullptr; } hk;
+    bool p2_smem_set = false;   // the P2 sieve's shared-memory limit has been raised
     // How the batched phases (mq_*) run: MQ_DIRECT launches as it goes; MQ_PREPARE reserves
     // scratch, uploads the arrays built on the host and reads back table values, with no
     // device work; MQ_CAPTURE then enqueues only device work (kernels, memsets), into a

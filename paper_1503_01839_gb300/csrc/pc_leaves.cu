@@ -522,24 +522,24 @@ __global__ void __launch_bounds__(256, 8) easy_kernel(LeafArgs A, u64 b_lo, u64 
 static int leaf_pass(pc_ctx* ctx, const LeafProblem& P, u64 b_lo, u64 nb, u32 what, u64 u_lo, u64 u_hi,
                      I128Pair* out)
 {
-    PC_TRY(buf_reserve(ctx, ctx->easy_rng, nb * sizeof(EasyRange)));
-    PC_TRY(buf_reserve(ctx, ctx->easy_chunk_off, (nb + 1) * sizeof(u64) + (nb + 1) * sizeof(u32)));
-    u64* choff = ctx->easy_chunk_off.as<u64>();
+    const bool table = what == LEAVES_TABLE;   // such a pass may run beside the easy leaves': its own scratch
+    DevBuf &range_buf = ctx->easy_rng[table], &off_buf = ctx->easy_chunk_off[table];
+    PC_TRY(buf_reserve(ctx, range_buf, nb * sizeof(EasyRange)));
+    PC_TRY(buf_reserve(ctx, off_buf, (nb + 1) * (sizeof(u64) + sizeof(u32))));
+    EasyRange* rng = range_buf.as<EasyRange>();
+    u64* choff = off_buf.as<u64>();
     u32* nch = (u32*)(choff + nb + 1);
     LeafArgs A = make_args(ctx, P);
     const bool odd = !A.sampled && P.y < PI_ODD_Y && ctx->T.podd_limit >= P.y;
     if (odd) A.clust_chunk = 0;   // clustered chunks by pi value
-    easy_ranges_kernel<<<(unsigned)((nb + 255) / 256), 256, 0, ctx->stream>>>(A, b_lo, nb, what, u_lo, u_hi,
-                                                                              ctx->easy_rng.as<EasyRange>(), nch);
+    easy_ranges_kernel<<<(unsigned)((nb + 255) / 256), 256, 0, ctx->stream>>>(A, b_lo, nb, what, u_lo, u_hi, rng, nch);
     PC_LAUNCHED(ctx);
     ctx->stats.kernel_launches++;
     PC_TRY(scan_exclusive_u32_to_u64(ctx, nch, choff, nb));
-    const bool timed = what != LEAVES_TABLE;
     // the number of chunks stays on the device: warps take them from a queue
     const int g = (int)pc_min((u64)ctx->sm_count * 8, nb);
-    if (timed) PC_CUDA(ctx, cudaEventRecord(ctx->ev[2], ctx->stream));
-    const EasyRange* rng = ctx->easy_rng.as<EasyRange>();
-    unsigned long long* queue = call_queue(ctx, timed ? Q_EASY : Q_TABLE);
+    if (!table) PC_CUDA(ctx, cudaEventRecord(ctx->ev[2], ctx->stream));
+    unsigned long long* queue = call_queue(ctx, table ? Q_TABLE : Q_EASY);
     if (A.sampled)
         easy_kernel<PI_SAMPLED><<<g, 256, 0, ctx->stream>>>(A, b_lo, nb, rng, choff, queue, out, ctx->dstat);
     else if (odd)
@@ -547,7 +547,7 @@ static int leaf_pass(pc_ctx* ctx, const LeafProblem& P, u64 b_lo, u64 nb, u32 wh
     else
         easy_kernel<PI_REC><<<g, 256, 0, ctx->stream>>>(A, b_lo, nb, rng, choff, queue, out, ctx->dstat);
     PC_LAUNCHED(ctx);
-    if (timed) {
+    if (!table) {
         PC_CUDA(ctx, cudaEventRecord(ctx->ev[3], ctx->stream));
         ctx->easy_timed = true;
     }
@@ -557,8 +557,7 @@ static int leaf_pass(pc_ctx* ctx, const LeafProblem& P, u64 b_lo, u64 nb, u32 wh
 
 int run_easy(pc_ctx* ctx, const LeafProblem& P, I128Pair* out)
 {
-    const u64 b_lo = (u64)P.c + 1;
-    const u64 b_hi = pc_min(P.a, P.E);
+    const u64 b_lo = (u64)P.c + 1, b_hi = pc_min(P.a, P.E);
     if (b_hi < b_lo) return PC_OK;
     return leaf_pass(ctx, P, b_lo, b_hi - b_lo + 1, P.table_in_easy ? LEAVES_BOTH : LEAVES_EASY, 0, ~0ull, out);
 }

@@ -603,19 +603,19 @@ int run_p2(pc_ctx* ctx, u64 x, u64 y, u64 a, const u64* pv, I128Pair* out)
     A.queue = (u32*)call_queue(ctx, Q_P2);
     const u32 nblk = A.seg_bytes >> 7;
     size_t smem = A.seg_bytes + (2 * (size_t)nblk + 2) * sizeof(u32);
-    // the kernel's limit is shared by every host thread: set the device maximum
-    cudaFuncAttributes fa;
-    PC_CUDA(ctx, cudaFuncGetAttributes(&fa, p2_sieve_kernel<512, false>));
-    const size_t dyn_max = ctx->smem_optin - fa.sharedSizeBytes;
-    if (smem > dyn_max) {
-        pc_set_error(ctx, "p2 sieve: %zu bytes of shared memory per CTA", smem);
-        return PC_EINVAL;
-    }
-    cudaError_t e = cudaFuncSetAttribute(p2_sieve_kernel<512, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)dyn_max);
-    if (e != cudaSuccess) {
-        pc_set_error(ctx, "p2 smem attribute: %s", cudaGetErrorString(e));
-        return PC_ECUDA;
+    // the kernel's limit is shared by every host thread: set the device maximum (segments of at
+    // most MAX_SEG bytes and their block counts fit in it)
+    if (!ctx->p2_smem_set) {
+        cudaFuncAttributes fa;
+        PC_CUDA(ctx, cudaFuncGetAttributes(&fa, p2_sieve_kernel<512, false>));
+        const size_t dyn_max = ctx->smem_optin - fa.sharedSizeBytes;
+        cudaError_t e = cudaFuncSetAttribute(p2_sieve_kernel<512, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)dyn_max);
+        if (e != cudaSuccess) {
+            pc_set_error(ctx, "p2 smem attribute: %s", cudaGetErrorString(e));
+            return PC_ECUDA;
+        }
+        ctx->p2_smem_set = true;
     }
     int per_sm = (int)(ctx->smem_optin / (smem + 4096));
     if (per_sm < 1) per_sm = 1;

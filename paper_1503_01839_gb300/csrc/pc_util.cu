@@ -205,8 +205,9 @@ static int scan_impl(pc_ctx* ctx, const u32* in, TO* out, u64 n)
         return PC_OK;
     }
     const u64 tiles = (n + SCAN_TILE - 1) / SCAN_TILE;
-    PC_TRY(buf_reserve(ctx, ctx->scan_tmp, (tiles + 1) * sizeof(TO)));
-    TO* sums = ctx->scan_tmp.as<TO>();
+    DevBuf& tmp = ctx->scan_tmp[ctx->scan_sel];
+    PC_TRY(buf_reserve(ctx, tmp, (tiles + 1) * sizeof(TO)));
+    TO* sums = tmp.as<TO>();
     if (!mq_device_work(ctx)) return PC_OK;
     scan_tile_sums<TO><<<(unsigned)tiles, SCAN_THREADS, 0, ctx->stream>>>(in, n, sums);
     PC_LAUNCHED(ctx);
