@@ -15,7 +15,7 @@
 struct P2Args {
     u64 x, y, z, r;   // r = isqrt(x)
     u32 B, k0;
-    u32 b_mid, b_big;   // first prime index >= P2_COOP_P, and with 8 p > seg_bytes
+    u32 b_mid, b_big;   // first prime index with p >= p2_coop_p, with p > p2_big_p
     u64 nseg;         // segments sieved: s0 .. s0 + nseg - 1 (arrays below indexed from s0)
     u64 s0;           // first segment sieved: those below isqrt(x) hold no x/p (x/p >= isqrt x)
     u32 seg_bytes;
@@ -38,34 +38,46 @@ struct P2Args {
     u32 b_bkt;
 };
 
-// Primes below P2_COOP_P have many wheel rounds per segment and are crossed
-// off by the whole CTA at once; the medium ones by one thread per (prime,
-// residue class); those with fewer than one round per 8 bytes by one thread
-// per prime.
-static constexpr u32 P2_COOP_P = 512;
-// In small segments the line lies lower, at 64 rounds per residue class: the CTA's threads take
-// the primes above it all at once instead of one prime after the other.
-static u32 p2_coop_p(u32 seg_bytes) { return seg_bytes / 64 < P2_COOP_P ? seg_bytes / 64 : P2_COOP_P; }
+// The smallest primes have many wheel rounds per segment and are crossed off by the whole CTA at
+// once, up to p2_coop_p (each class's first byte from a table in shared memory, below 2^10); the
+// medium ones, up to p2_big_p, by one thread per (prime, residue class); those with a round or two
+// by one thread per prime.  A thread's work between two barriers should not exceed its share of
+// the whole, hence 32 rounds per class at the first line (64 in large segments, where the CTA's
+// loop over one prime is long enough), two rounds at the second (P2 of pi(10^18) in 48 KiB segments: 7.6 ms
+// at 512 and seg / 8, i.e. 96 and 8 rounds, 7.0 at seg / 4, 6.7 at seg / 2, 5.74 with 768; 11.7 at 256).
+static constexpr u32 P2_COOP_MAX = 1024;
+static u32 p2_coop_p(u32 seg_bytes)
+{
+    const u32 c = seg_bytes >= 49152 ? seg_bytes / 64 : seg_bytes / 32;
+    return c < P2_COOP_MAX ? c : P2_COOP_MAX;
+}
+static u32 p2_big_p(u32 seg_bytes) { return seg_bytes / 2; }
+// Bytes of shared memory: the bitset, then the table of the cooperative primes (at most 164 of
+// eight u16; the bitset's fill needs none) and, after the crossings, the block counts.
+static size_t p2_smem(u32 seg_bytes, u64 n_coop)
+{
+    const size_t counts = (2 * (size_t)(seg_bytes >> 7) + 2) * sizeof(u32), table = n_coop * 8 * sizeof(u16);
+    return seg_bytes + ((counts > table ? counts : table) + 15) / 16 * 16;
+}
 
 // Segment bytes of P2's sieve over [0, z]: small z in small segments, so that they spread over
-// the chip's 152 SMs (kernel times on GB300 against 32 KiB: 2 KiB 0.058 / 0.174 ms at z = 6e6,
-// 0.068 / 0.215 at 2.9e7, 8 KiB 0.109 / 0.230 at 9e7, 16 KiB 0.167 / 0.285 at 1.9e8, 0.288 /
-// 0.300 at 5e8), then 32 KiB up to z = 2^30, 64 KiB up to 2^32 and 48 KiB beyond (48 KiB
-// against 64 KiB: pi(1e17) P2 2.45 -> 2.38 ms, pi(1e18) 8.9 -> 8.5 ms).
+// the chip's 152 SMs (kernel times on GB300 against 32 KiB: 2 KiB 0.039 / 0.217 ms at z = 6e6,
+// 4 KiB 0.052 / 0.206 at 2.9e7, 8 KiB 0.088 / 0.238 at 9e7, 0.106 / 0.265 at 1.9e8, 16 KiB
+// 0.209 / 0.314 at 5e8, 40 KiB 0.468 / 0.502 at 1.5e9, 64 KiB 5.04 / 6.23 at 1.8e10; 48 KiB
+// there, with a fourth CTA per SM: 5.72).  Half these sizes are a little faster alone at z < 1e8
+// but slow the hard-leaf sieve beside them (pi(1e12) 0.255 ms, 0.285 at 1 KiB).
 static u32 p2_seg_for(u64 z)
 {
-    if (z < 40000000ull) return 2048;
-    if (z < 150000000ull) return 8192;
-    if (z < 700000000ull) return 16384;
-    return z < (1ull << 30) ? 32768 : z < (1ull << 32) ? 65536 : 49152;
+    if (z < 12000000ull) return 2048;
+    if (z < 40000000ull) return 4096;
+    if (z < 300000000ull) return 8192;
+    if (z < 800000000ull) return 16384;
+    return z < 1200000000ull ? 32768 : z < 2200000000ull ? 40960 : 65536;
 }
 
 // The crossing walks of pc_sieve.cuh with 32-bit offsets, for p < 2^29: a byte offset
 // below 2^17 plus p, or an integer offset below 30 * 2^17 plus 6 p, stays below 2^32.
 // (P2's primes are at most isqrt(z) < 2^21 whenever y >= iroot3(x).)
-#ifndef P2_NARROW
-#define P2_NARROW 1
-#endif
 __device__ __forceinline__ u32 p2_cross_class(u32* bits, u32 seg_bytes, u64 L, u32 p, u64 kstart, u32 j)
 {
     const u32 rj = r8(j);
@@ -84,24 +96,76 @@ __device__ __forceinline__ u32 p2_cross_class(u32* bits, u32 seg_bytes, u64 L, u
     return n;
 }
 
-__device__ __forceinline__ u32 p2_cross_single(u32* bits, u32 seg_bytes, u64 L, u32 p, u64 kstart)
+// The constants of the primes p = 30 P + R8[i]: their multiple of class j, cofactor 30 q + R8[j],
+// lies in byte p q + P R8[j] + floor(R8[i] R8[j] / 30), at bit idx30(R8[i] R8[j] mod 30).
+struct P2Wheel {
+    u64 off[8];   // [i]: floor(R8[i] R8[j] / 30), 5 bits a class
+    u32 bit[8];   // [i]: the bits, 4 bits a class
+};
+
+__device__ __forceinline__ void make_p2_wheel(P2Wheel* w)
 {
-    const u64 k = coprime30_at_or_after(kstart);
-    const u64 n0 = (u64)p * k;
-    const u32 span = 30 * seg_bytes;
-    if (n0 - L >= span) return 0;
-    u32 r = (u32)(k % 30), rel = (u32)(n0 - L), cnt = 0;
-    while (rel < span) {
-        cnt++;
-        const u32 q30 = rel / 30;
-        const u32 pos = q30 * 8 + idx30(rel - 30 * q30);
-        atomicAnd(&bits[pos >> 5], ~(1u << (pos & 31)));
-        const u32 d = next30(r);
-        r += d;
-        if (r >= 30) r -= 30;
-        rel += p * d;
+    if (threadIdx.x < 8) {
+        const u32 ri = r8(threadIdx.x);
+        u64 o = 0;
+        u32 b = 0;
+        for (u32 j = 0; j < 8; j++) {
+            o |= (u64)(ri * r8(j) / 30) << (5 * j);
+            b |= idx30(ri * r8(j) % 30) << (4 * j);
+        }
+        w->off[threadIdx.x] = o;
+        w->bit[threadIdx.x] = b;
     }
-    return cnt;
+}
+
+// One thread crosses off all multiples k p, k >= kstart coprime to 30, of a prime p < 2^29 with
+// few rounds in the segment: class by class from its first byte, so that a crossing costs a
+// few instructions and not a step along the wheel.  Lb = L / 30.
+__device__ __forceinline__ u32 p2_cross_prime(u32* bits, u32 seg_bytes, u64 Lb, u32 p, u64 kstart, const P2Wheel& w)
+{
+    const u64 q = kstart / 30;
+    const u32 kmod = (u32)(kstart - 30 * q);
+    const i64 base64 = (i64)(p * q) - (i64)Lb;   // the round of kstart: it may begin before the segment
+    if (base64 >= (i64)seg_bytes) return 0;
+    const i32 base = (i32)base64;
+    const u32 P30 = p / 30, i = idx30(p - 30 * P30);
+    const u64 off = w.off[i];
+    const u32 bit = w.bit[i];
+    u32 n = 0;
+#pragma unroll
+    for (u32 j = 0; j < 8; j++) {
+        const u32 R = (u32)(PC_R8PACK >> (5 * j)) & 31u;
+        i32 by = base + (i32)(P30 * R + ((u32)(off >> (5 * j)) & 31u));
+        if (R < kmod) by += (i32)p;
+        const u32 b = (bit >> (4 * j)) & 7u;
+        for (; by < (i32)seg_bytes; by += (i32)p, n++) {
+            const u32 pos = ((u32)by << 3) + b;
+            atomicAnd(&bits[pos >> 5], ~(1u << (pos & 31)));
+        }
+    }
+    return n;
+}
+
+// floor(n / d) for n < 2^22 d: two steps with the reciprocal of d's top 16 bits, from below (the
+// first leaves n < 2^9 d, the second a few d), then the exact remainder.
+__device__ __forceinline__ u32 p2_div(u64 n, u32 d)
+{
+    const int s = 31 - __clz((int)d);                        // 2^s <= d
+    const u32 top = s >= 15 ? d >> (s - 15) : d << (15 - s);   // 2^15 <= top < 2^16
+    const u32 v = 0xFFFFFFFFu / (top + 1);                   // 2^32 / (top + 1), below 2^17: from below
+    // n / d > n v / 2^(17 + s): from below again
+    const int k = s > 9 ? s - 9 : 0;                         // n >> k < 2^32
+    u32 q = (u32)(((u64)(u32)(n >> k) * v) >> (17 + s - k));
+    u64 r = n - (u64)q * d;                                  // below 2^9 d
+    const int k2 = s > 21 ? s - 21 : 0;
+    const u32 q2 = (u32)(((u64)(u32)(r >> k2) * v) >> (17 + s - k2));
+    q += q2;
+    r -= (u64)q2 * d;
+    while (r >= d) {
+        r -= d;
+        q++;
+    }
+    return q;
 }
 
 // A launch over the segments of many queries (the batched form): item g is segment
@@ -133,6 +197,11 @@ __global__ void __launch_bounds__(NT, 4) p2_sieve_kernel(P2Args A0, P2Multi M)
     __shared__ i128 red[32];
     const u32 tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     make_pattern_words(patw, A0.k0);
+    // the cooperative primes of a segment: first byte of every class, and its bit in the top 3
+    // bits (in the place of the block counts, which the crossings do not need yet)
+    u16* coop = (u16*)blk;
+    __shared__ P2Wheel wheel;
+    make_p2_wheel(&wheel);
     __shared__ __align__(16) unsigned char sA_raw[MULTI ? sizeof(P2Args) : 16];
     __shared__ u32 s_q;
     u32 cur_q = ~0u;
@@ -169,22 +238,45 @@ __global__ void __launch_bounds__(NT, 4) p2_sieve_kernel(P2Args A0, P2Multi M)
         if (A.pat) fill_pattern_global(bits, seg_words, L, A.pat, WHEEL19_PERIOD);
         else fill_pattern(bits, seg_words, L, patw, A.k0);
         u32 ncl = 0;
+        const u64 end = L + A.span, Lb = L / 30;
+        // from p^2 <= L on for every cooperative prime, a class's first byte is below p < 2^10
+        const bool table = L >= (u64)P2_COOP_MAX * P2_COOP_MAX;
+        const u32 n_coop = A.b_mid - A.k0 - 1;
+        if (table)
+            for (u32 t = tid; t < 8 * n_coop; t += NT) {
+                const u32 b = A.k0 + 1 + (t >> 3), j = t & 7;
+                const u32 p = A.primes[b], rj = r8(j);
+                const u64 ks = div_rcp(L + p - 1, p, A.primes_rcp[b]), q = ks / 30;
+                const u32 pr = p * rj;
+                const i32 by = (i32)((i64)(p * q) - (i64)Lb) + (i32)(pr / 30) + (rj < (u32)(ks - 30 * q) ? (i32)p : 0);
+                coop[t] = (u16)((u32)by | idx30(pr % 30) << 13);
+            }
         __syncthreads();
-        const u64 end = L + A.span;
         // cross off p_b, k0 < b <= B (the prime itself included)
         auto none = [](u32) {};
-        for (u32 b = A.k0 + 1; b < A.b_mid; b++) {
-            const u64 p = A.primes[b];
-            u64 ks = L ? div_rcp(L + p - 1, p, A.primes_rcp[b]) : 0;
-            if (ks < p) ks = p;
-            ncl += cross_off_coop(bits, A.seg_bytes, L, (u32)p, ks, tid, NT, none);
+        if (table) {   // thread = (class, every 64th round), the same for every prime
+            const u32 j = tid / (NT / 8), o = tid % (NT / 8);
+            for (u32 c = 0; c < n_coop; c++) {
+                const u32 p = A.primes[A.k0 + 1 + c], e = coop[8 * c + j], bit = e >> 13, step = p * (NT / 8);
+                for (u32 by = (e & 0x1FFFu) + o * p; by < A.seg_bytes; by += step, ncl++) {
+                    const u32 pos = (by << 3) + bit;
+                    atomicAnd(&bits[pos >> 5], ~(1u << (pos & 31)));
+                }
+            }
+        } else {
+            for (u32 b = A.k0 + 1; b < A.b_mid; b++) {
+                const u64 p = A.primes[b];
+                u64 ks = L ? div_rcp(L + p - 1, p, A.primes_rcp[b]) : 0;
+                if (ks < p) ks = p;
+                ncl += cross_off_coop(bits, A.seg_bytes, L, (u32)p, ks, tid, NT, none);
+            }
         }
         for (u32 task = tid; task < 8 * (A.b_big - A.b_mid); task += NT) {
             const u32 bb = A.b_mid + (task >> 3);
             const u64 p = A.primes[bb];
             u64 ks = L ? div_rcp(L + p - 1, p, A.primes_rcp[bb]) : 0;
             if (ks < p) ks = p;
-            ncl += P2_NARROW && p < (1u << 29) ? p2_cross_class(bits, A.seg_bytes, L, (u32)p, ks, task & 7)
+            ncl += p < (1u << 29) ? p2_cross_class(bits, A.seg_bytes, L, (u32)p, ks, task & 7)
                              : cross_off_class(bits, A.seg_bytes, L, (u32)p, ks, task & 7, none);
         }
         const u32 b_end = A.bkt ? A.b_bkt : A.B + 1;
@@ -192,8 +284,8 @@ __global__ void __launch_bounds__(NT, 4) p2_sieve_kernel(P2Args A0, P2Multi M)
             const u64 p = A.primes[bb];
             u64 ks = L ? div_rcp(L + p - 1, p, A.primes_rcp[bb]) : 0;
             if (ks < p) ks = p;
-            ncl += P2_NARROW && p < (1u << 29) ? p2_cross_single(bits, A.seg_bytes, L, (u32)p, ks)
-                             : cross_off_single(bits, A.seg_bytes, L, (u32)p, ks, none);
+            ncl += p < (1u << 29) ? p2_cross_prime(bits, A.seg_bytes, Lb, (u32)p, ks, wheel)
+                                  : cross_off_single(bits, A.seg_bytes, L, (u32)p, ks, none);
         }
         if (A.bkt) {   // the larger primes: only the multiples filed in this segment's bucket
             const u32 nf = pc_min(A.bkt_n[s], A.bkt_cap);
@@ -205,7 +297,7 @@ __global__ void __launch_bounds__(NT, 4) p2_sieve_kernel(P2Args A0, P2Multi M)
             }
         }
         // the sieving primes themselves (only in the first segments)
-        for (u32 bb = A.k0 + 1 + tid; bb <= A.B; bb += NT) {
+        for (u32 bb = A.k0 + 1 + tid; bb <= A.B && A.primes[A.B] >= L; bb += NT) {
             const u64 p = A.primes[bb];
             if (p >= end) break;
             if (p >= L) {
@@ -259,16 +351,18 @@ __global__ void __launch_bounds__(NT, 4) p2_sieve_kernel(P2Args A0, P2Multi M)
         i64 acc = 0;
         u32 tl = 0;
         if (phi > plo) {
-            const u64 w0 = (plo + 1) / 240, w1 = phi / 240;
-            for (u64 w = w0 + tid; w <= w1; w += NT) {
-                u64 v = A.pit.rec[w].bits;
+            // a thread takes two bytes of the pi table (60 integers, a few primes) at a time
+            const u64 h0 = (plo + 1) / 60, h1 = phi / 60;
+            for (u64 h = h0 + tid; h <= h1; h += NT) {
+                u32 v = ((const u16*)&A.pit.rec[h >> 2].bits)[h & 3];
                 while (v) {
-                    int bi = __ffsll((long long)v) - 1;
+                    const u32 bi = __ffs(v) - 1;
                     v &= v - 1;
-                    u64 p = 240 * w + 30 * (u64)(bi >> 3) + r8(bi & 7);
+                    const u64 p = 60 * h + 30 * (u64)(bi >> 3) + r8(bi & 7);
                     if (p <= plo || p > phi) continue;
-                    u64 q = A.x / p;
-                    u32 e = seg_count_end(q, L);
+                    // x / p - L is below the segment's length
+                    const u32 rel = p2_div(A.x - L * p, (u32)p), q30 = rel / 30;
+                    const u32 e = q30 * 8 + cntle30(rel - 30 * q30);
                     u32 eb = e >> 10, ew = e >> 6;
                     u32 c = pre[eb];
                     for (u32 ww = eb << 4; ww < ew; ww++) c += __popcll(bits64[ww]);
@@ -548,7 +642,7 @@ int p2_ask(pc_ctx* ctx, u64 x, u64 y, u64* v)
     v[n++] = pc_isqrt(x);
     v[n++] = pc_isqrt(z);
     v[n++] = p2_coop_p(seg) - 1;
-    v[n++] = seg / 8;
+    v[n++] = p2_big_p(seg);
     if (ctx->params.p2_bucket) v[n++] = seg;
     return n;
 }
@@ -601,8 +695,7 @@ int run_p2(pc_ctx* ctx, u64 x, u64 y, u64 a, const u64* pv, I128Pair* out)
     A.cnt = (u32*)(A.acc + A.nseg);
     A.tally = A.cnt + A.nseg;
     A.queue = (u32*)call_queue(ctx, Q_P2);
-    const u32 nblk = A.seg_bytes >> 7;
-    size_t smem = A.seg_bytes + (2 * (size_t)nblk + 2) * sizeof(u32);
+    const size_t smem = p2_smem(A.seg_bytes, A.b_mid - A.k0 - 1);
     // the kernel's limit is shared by every host thread: set the device maximum (segments of at
     // most MAX_SEG bytes and their block counts fit in it)
     if (!ctx->p2_smem_set) {
@@ -693,6 +786,7 @@ int mq_final(pc_ctx* ctx, const MQPlan& P, u64* d_out, int* d_bad)
     return PC_OK;
 }
 
+static constexpr u32 P2_MQ_COOP = 512;
 int mq_p2(pc_ctx* ctx, const MQPlan& P)
 {
     const u32 Q = P.Q;
@@ -703,7 +797,7 @@ int mq_p2(pc_ctx* ctx, const MQPlan& P)
     T.pit = ctx->T.pi();
     T.primes = ctx->T.primes.as<u32>();
     T.primes_rcp = ctx->T.primes_rcp.as<u64>();
-    u64 v2[2] = {P2_COOP_P - 1, T.seg_bytes / 8}, pv2[2];
+    u64 v2[2] = {P2_MQ_COOP - 1, p2_big_p(T.seg_bytes)}, pv2[2];
     if (ctx->mq_mode == MQ_CAPTURE) {   // a read-back: taken in the prepare pass
         pv2[0] = ctx->mq_p2_pv[0];
         pv2[1] = ctx->mq_p2_pv[1];
@@ -762,8 +856,7 @@ int mq_p2(pc_ctx* ctx, const MQPlan& P)
         PC_CUDA(ctx, cudaMemcpyAsync(d_qa, qa.data(), Q * sizeof(P2Args), cudaMemcpyHostToDevice, st));
         PC_CUDA(ctx, cudaMemcpyAsync(d_ipref, ipref.data(), (Q + 1) * 4, cudaMemcpyHostToDevice, st));
     }
-    const u32 nblk = T.seg_bytes >> 7;
-    const size_t smem = T.seg_bytes + (2 * (size_t)nblk + 2) * sizeof(u32);
+    const size_t smem = p2_smem(T.seg_bytes, pv2[0] - T.k0);
     if (S && ctx->mq_mode != MQ_CAPTURE) {   // the shared-memory limit, set outside any capture
         cudaFuncAttributes fa;
         PC_CUDA(ctx, cudaFuncGetAttributes(&fa, p2_sieve_kernel<512, true>));

@@ -7,7 +7,8 @@ import paper_1503_01839_gb300 as pc
 
 pytestmark = pytest.mark.gpu
 
-LINES = [400_000, 40_000_000, 120_000_000, 150_000_000, 280_000_000, 700_000_000, 2_000_000_000]
+LINES = [400_000, 12_000_000, 40_000_000, 120_000_000, 280_000_000, 300_000_000, 800_000_000, 1_200_000_000,
+         2_000_000_000, 2_200_000_000]
 
 
 @pytest.mark.parametrize("z", LINES)

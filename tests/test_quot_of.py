@@ -69,3 +69,32 @@ def test_near(dbits):
         for q in [0, 1, (1 << 18) - 1, 245759] + [rng.randrange(1 << 18) for _ in range(50)]:
             for r in {0, d // 2, d - 1}:
                 assert near(q * d + r, d) == q, (q, d, r)
+
+
+def two_steps(n, d):
+    s = d.bit_length() - 1
+    top = d >> (s - 15) if s >= 15 else d << (15 - s)
+    v = 0xFFFFFFFF // (top + 1)
+    assert v < 1 << 17
+    k = max(0, s - 9)
+    assert n >> k < 1 << 32
+    q = ((n >> k) * v) >> (17 + s - k)
+    r = n - q * d
+    assert 0 <= r < d << 9, (n, d)
+    k2 = max(0, s - 21)
+    assert r >> k2 < 1 << 32
+    q2 = ((r >> k2) * v) >> (17 + s - k2)
+    r -= q2 * d
+    assert 0 <= r < 4 * d, (n, d)
+    return q + q2 + r // d
+
+
+@pytest.mark.parametrize("dbits", [1, 2, 8, 15, 16, 17, 23, 24, 31, 32])
+def test_two_steps(dbits):
+    # p2_div (pc_p2.cu): quotients below 2^22, any 32-bit divisor
+    rng = random.Random(dbits)
+    lo, hi = 1 << (dbits - 1), (1 << dbits) - 1
+    for d in {lo, hi, min(lo + 1, hi)} | {rng.randrange(lo, hi + 1) for _ in range(500)}:
+        for q in [0, 1, 2, (1 << 22) - 1] + [rng.randrange(1 << rng.randrange(1, 23)) for _ in range(50)]:
+            for r in {0, d // 2, d - 1}:
+                assert two_steps(q * d + r, d) == q, (q, d, r)
