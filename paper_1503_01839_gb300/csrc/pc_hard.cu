@@ -1039,7 +1039,7 @@ u32 pc_seg_bytes(pc_ctx* ctx, u32 dflt)
 // sub-ranges are fewer than the warps the chip holds (152 x 16), smaller ones shorten the
 // chain; once they are many, larger ones do fewer steps per integer.  The lines lie where the
 // sieve's time crosses on GB300 (8 KiB / 1 KiB against 32 KiB / 8 KiB: 0.088 / 0.223 ms at
-// z = 8e5, 0.193 / 0.324 at 6e6, 0.375 / 0.565 at 9e7; 8 KiB / 2 KiB 0.53 / 0.67 at 1.4e8;
+// z = 8e5, 0.193 / 0.324 at 6e6, 0.375 / 0.565 at 9e7; 16 KiB / 2 KiB 0.51 / 0.67 at 1.4e8;
 // 16 KiB / 4 KiB 0.825 / 1.03 at 3.3e8, 2.67 / 2.75 at 1.5e9, 4.91 / 4.65 at 3e9).
 static u32 hard_sub_for(u64 z)
 {
@@ -1048,7 +1048,7 @@ static u32 hard_sub_for(u64 z)
 
 u32 hard_seg_for(u64 z)
 {
-    return z < 400000ull ? 2048 : z < 280000000ull ? 8192 : z < 2000000000ull ? 16384 : 32768;
+    return z < 400000ull ? 2048 : z < 120000000ull ? 8192 : z < 2000000000ull ? 16384 : 32768;
 }
 
 // bytes per warp sub-range: a power of two dividing seg_bytes, at most 16 warps
@@ -1100,6 +1100,7 @@ struct PlanArgs {
     float x, z;
     u64 span, s0, s1;
     double inv_ctas4;           // 1 / (4 * resident CTAs)
+    u32 ctas;
     u64 cap;                    // slots in items
     PlanScratch* scr;
     u32* split;                 // per segment: R | bucket << 16 (R = 0: no item)
@@ -1196,18 +1197,22 @@ __global__ void plan_scatter_kernel(PlanArgs P)
 }
 
 // The planner in one launch (one CTA) for up to PLAN_ONE segments: the same decisions, with the
-// buckets in shared memory.
+// buckets in shared memory.  When the items are fewer than the launch's CTAs, every segment is
+// split further, to at least FILL_STEPS steps a replica: the steps of an item are a serial chain,
+// and the crossings a replica repeats are done by the whole CTA at once (pi(10^9) 0.125 -> 0.11 ms,
+// pi(10^11) 0.21 -> 0.155, pi(10^12) 0.256 -> 0.19; with 8, 16, 32 steps pi(10^11) 0.169, 0.167, 0.195).
 // (Four launches and their gaps cost more than the work: pi(10^12) plans 26 segments.)
 static constexpr u64 PLAN_ONE = 8192;
+static constexpr u32 FILL_STEPS = 4;
 __global__ void __launch_bounds__(1024) plan_one_kernel(PlanArgs P)
 {
     __shared__ double part[32];
     __shared__ u32 cnt[PLAN_BUCKETS], cur[PLAN_BUCKETS];
-    __shared__ u32 nheavy, ok;
+    __shared__ u32 nheavy, ok, n0;
     __shared__ unsigned long long steps;
     const u32 tid = threadIdx.x;
     if (tid < PLAN_BUCKETS) cnt[tid] = 0;
-    if (tid == 0) nheavy = 0, steps = 0;
+    if (tid == 0) nheavy = n0 = 0, steps = 0;
     double t = 0;
     unsigned long long st = 0;
     for (u64 s = P.s0 + tid; s < P.s1; s += 1024)
@@ -1225,6 +1230,19 @@ __global__ void __launch_bounds__(1024) plan_one_kernel(PlanArgs P)
     for (u64 s = P.s0 + tid; s < P.s1; s += 1024) {
         const u32 v = seg_split(P, s, target);
         P.split[s] = v;
+        if (v) atomicAdd(&n0, v & 0xFFFFu);
+    }
+    __syncthreads();
+    const u32 fill = n0 && n0 < P.ctas ? P.ctas / n0 : 1;   // items grow to at most the CTAs
+    for (u64 s = P.s0 + tid; s < P.s1; s += 1024) {
+        u32 v = P.split[s];
+        if (fill > 1 && v) {
+            const u32 R = v & 0xFFFFu, most = (P.segB[s] - P.k0) / FILL_STEPS;
+            const u32 R2 = R * fill < most ? R * fill : (most > R ? most : R);
+            // the share's bucket falls by four per halving, as in seg_split
+            const int key = (int)(v >> 16) - (int)(4.0f * log2f((float)R2 / (float)R));
+            P.split[s] = v = R2 | (u32)(key < 0 ? 0 : key) << 16;
+        }
         if (v) atomicAdd(&cnt[v >> 16], v & 0xFFFFu);
     }
     __syncthreads();
@@ -1536,7 +1554,7 @@ int run_hard_sieve(pc_ctx* ctx, const LeafProblem& P, I128Pair* out)
     A.acc = out;
     A.queue = (u32*)call_queue(ctx, Q_HARD);
     A.stat = call_hard_stat(ctx);
-    PlanArgs PA{segB, est, A.k0, (float)P.x, (float)P.z, A.span, A.s0, A.s1, 1.0 / (4.0 * ctas), cap,
+    PlanArgs PA{segB, est, A.k0, (float)P.x, (float)P.z, A.span, A.s0, A.s1, 1.0 / (4.0 * ctas), (u32)ctas, cap,
                 scr, split, ditems, heavy, A.stat};
     if (ns <= PLAN_ONE) {
         plan_one_kernel<<<1, 1024, 0, ctx->stream>>>(PA);
