@@ -86,29 +86,18 @@ __device__ __forceinline__ u64 div_rcp(u64 n, u64 d, u64 v)
 }
 PC_HD u64 pc_max(u64 a, u64 b) { return a > b ? a : b; }
 
-// floor(n / d) for d = low word of dv, v = high word = floor((2^(32+s) - 1) / d),
-// s = floor(log2 d), whenever the quotient is below 2^31.  v < 2^32 and
-// v > 2^(32+s)/d - 1, so n v / 2^(32+s) falls short of n/d by less than
-// n / 2^(32+s) < 2 (n/d) / 2^32 < 1: the estimate is the quotient or one less,
-// and one remainder test settles it.  Two 32x32 -> 64-bit products instead of
-// the 64-bit high product of div_rcp.
-__device__ __forceinline__ u32 div_dv(u64 n, u64 dv)
-{
-    const u32 d = (u32)dv, v = (u32)(dv >> 32);
-    const u64 lo = (u64)(u32)n * v;
-    const u64 hi = (u64)(u32)(n >> 32) * v + (lo >> 32);   // floor(n v / 2^32)
-    u32 q = (u32)(hi >> (31 - __clz(d)));
-    if (n - (u64)q * d >= d) q++;
-    return q;
-}
-// The same quotient for many divisors of one dividend n: with k = max(0, bits of n - 32)
+// The 32-bit reciprocal record of d: d, and v = floor((2^(32+s) - 1) / d) < 2^32, s = floor(log2 d)
+// (pc_dv).  v > 2^(32+s)/d - 1, so n v / 2^(32+s) falls short of n/d by less than n / 2^(32+s) <
+// 2 (n/d) / 2^32.
+//
+// Quotients of one dividend n by many divisors: with k = max(0, bits of n - 32)
 // and T = floor(n / 2^k) < 2^32, the estimate floor(T v / 2^(32+s-k)) falls short of n/d by
 // less than n / 2^(32+s) + 2^k / d (from v) + 0 or 2^k / d (from T, exact when k = 0).
 // With d < 2^(s+1) and n >= 2^(31+k) if k > 0, both terms are below (n/d) / 2^31: the estimate
 // is the quotient or one less whenever the quotient is below 2^30 (and s >= k there, since
 // n/d >= 2^(31+k) / 2^(s+1)).  The remainder is below 2 d, so with d < 2^31 its low 32 bits
-// decide.  One high product, one low product and a comparison, where div_dv takes two wide
-// products and a 64-bit remainder.  The easy-leaf kernel is bound by its instructions and its
+// decide.  One high product, one low product and a comparison; the whole product by v takes two
+// wide ones and a 64-bit remainder.  The easy-leaf kernel is bound by its instructions and its
 // gathers: with this, pi_odd1's masks and the runs summed by parts, 30.1 -> 21.1 ms at
 // pi(10^18), alpha 56, 1.63 -> 1.06 ms at pi(10^16).
 struct QuotOf {
@@ -201,7 +190,6 @@ __device__ __forceinline__ u32 pi_odd1(const uint2* t, u32 u1)   // u1 = u + 1
     asm("bmsk.wrap.b32 %0, 0, %1;" : "=r"(low) : "r"(h));
     return r.y + __popc(r.x & low);
 }
-__device__ __forceinline__ u32 pi_odd(const uint2* t, u32 u) { return pi_odd1(t, u + 1); }
 
 // rank structure over a plain bitset of [0, limit]: rank(v) = #set bits <= v.
 struct RankTable {

@@ -35,10 +35,11 @@
 // Load balance: hard leaves crowd near u = y (their density falls like
 // 1/u^2), so one segment can hold a large share of them.  A pre-pass counts
 // the leaves of every segment; heavy segments are handed to several CTAs
-// ("replicas"), each of which sieves the whole segment but resolves only its
-// share of every step's leaves (Section 3 mentions dynamic block scheduling;
-// here the schedule is a list of work items ordered by estimated cost,
-// planned on the device).
+// ("replicas"), each of which owns a run of consecutive steps and crosses off
+// the primes before it with no counts; so is every segment while there are
+// fewer than CTAs (Section 3 mentions dynamic block scheduling; here the
+// schedule is a list of work items ordered by estimated cost, planned on the
+// device).
 #include <algorithm>
 #include <cmath>
 #include <vector>
@@ -462,6 +463,7 @@ __global__ void __launch_bounds__(MAXT, MINB) hard_sieve_kernel(HardArgs A0, Mul
             // length.  A lane without a leaf gets a small end (no_leaf: rel <= 1).
             const u64 negL = 0 - Lw;
             const bool m31 = !(A.y >> 31);
+            const u32 gmax = A.trunc ? (u32)pc_min(A.a, 0xFFFFFFFFull) : ~0u;   // gpf(m) <= p_a
             auto leaf_end = [&](u64 xp, const uint4& r) -> u32 {
                 const u32 rel = div_near(xp + r.x * negL, r.x, r.y, m31);
                 const u32 q30 = rel / 30;
@@ -671,7 +673,7 @@ __global__ void __launch_bounds__(MAXT, MINB) hard_sieve_kernel(HardArgs A0, Mul
                             const u32 hi = __shfl_sync(0xffffffffu, hoff, i);
                             const u32 t = t0 + i, b = bb + t;
                             const u64 xp = st[t].xp;
-                            const bool valid = (r.z >> 1) > b && !(A.trunc && r.w > A.a);
+                            const bool valid = r.z > 2 * b + 1 && r.w <= gmax;
                             const u32 e = leaf_end(xp, r);
                             u32 below = 0;   // hits of the run's earlier steps below the count end
                             for (u32 k = 0; k < hi; k++) below += lg[k] < e ? 1u : 0u;
@@ -825,7 +827,7 @@ __global__ void __launch_bounds__(MAXT, MINB) hard_sieve_kernel(HardArgs A0, Mul
                     // no early exit: a lane without a leaf of b (no entry, lpf <= p_b, or
                     // gpf > p_a) runs the same code and adds 0; its block index is clamped
                     // in count_to, so its reads stay inside the sub-range
-                    const bool valid = (r.z >> 1) > b && !(A.trunc && r.w > A.a);
+                    const bool valid = r.z > 2 * b + 1 && r.w <= gmax;
                     const u32 c = count_to(leaf_end(xp, r));
                     const i32 sg = valid ? ((r.z & 1u) ? 1 : -1) : 0;
                     acc += (i64)sg * (i32)c;

@@ -58,7 +58,7 @@ struct Tables {
     u64 nprimes = 0;
     DevBuf primes;
     DevBuf primes_rcp;   // floor((2^64 - 1) / p_k), same indexing as primes
-    DevBuf primes_dv;    // p_k | floor((2^(32+s) - 1) / p_k) << 32, s = floor(log2 p_k) (div_dv)
+    DevBuf primes_dv;    // p_k | floor((2^(32+s) - 1) / p_k) << 32, s = floor(log2 p_k) (pc_dv)
     // squarefree m-list over [2, ml_limit] with lpf > p_cmin
     u64 ml_limit = 0;
     u32 ml_cmin = 99;
@@ -81,7 +81,7 @@ struct Tables {
     // patterns of the primes 7 .. 61 in the mod-30 bitset: entry (k - 4) PATTERN_P + r of p_k
     // holds the 16 bytes from byte index g = r mod p_k on, a bit clear where p_k divides
     DevBuf pat16;
-    // odd-number pi table over [0, podd_limit] (pi_odd): one uint2 per 64 integers
+    // odd-number pi table over [0, podd_limit] (pi_odd1): one uint2 per 64 integers
     DevBuf pi_odd;
     u64 podd_limit = 0;
     // phi(., c) residue tables for the primorial of c (c = 0..7)
@@ -237,8 +237,6 @@ struct LeafProblem {
 
 // phi(m, b) for every c <= b <= b_max (Section 4 starting values): out[b - c]
 int phi_starts(pc_ctx* ctx, u64 m, u32 c, u64 b_max, u64* out);
-// segments of the hard-leaf sieve for (x, z) in the context's geometry
-u64 hard_segments(pc_ctx* ctx, u64 z);
 
 // Each adds its sum to *out (device I128Pair) -- out must be zeroed first.
 int run_s1_trivial(pc_ctx* ctx, const LeafProblem& P, I128Pair* out_s1, I128Pair* out_trivial);

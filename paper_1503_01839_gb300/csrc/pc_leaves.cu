@@ -36,8 +36,8 @@ struct LeafArgs {
     u32 slK[Tables::NSUB];
     const u32* primes;
     const u64* primes_rcp;   // floor((2^64 - 1) / p_k)
-    const u64* primes_dv;    // p_k and its 32-bit reciprocal (div_dv)
-    const uint2* podd;       // odd-number pi table (pi_odd) over [0, y]
+    const u64* primes_dv;    // p_k and its 32-bit reciprocal (pc_dv)
+    const uint2* podd;       // odd-number pi table (pi_odd1) over [0, y]
     // easy-leaf gathers from the sampled table of Section 2.1 instead of the pi table
     const u32* samp;
     u32 samp_s;
@@ -695,7 +695,8 @@ __global__ void mq_s1_trivial_kernel(LeafArgs T, const MQ* qs, const u64* pref, 
             const u64 v = xm / Qc;
             const u64 f = v * phiT[Qc] + phiT[(u32)(xm - v * Qc) + 1];
             s1 += (info & 1) ? -(i128)f : (i128)f;
-            if (kb > m.c + 1) {   // trivial leaves of m: max(c, pi(T)) < b < lpf index, b <= a
+            const u64 lp = T.primes[kb];
+            if (kb > m.c + 1 && lp * lp > xm) {   // trivial leaves of m: max(c, pi(T)) < b < lpf index, b <= a
                 const u64 Tm = pc_max(div_rcp(m.y, mv, rc), pc_isqrt(xm));
                 const u64 hi = pc_min(kb - 1, m.a);
                 u64 lo = m.c;

@@ -250,14 +250,14 @@ __global__ void reciprocal_kernel(const u32* d, u64 n, u64* v)
     if (i < n) v[i] = d[i] ? ~0ull / d[i] : 0;
 }
 
-// the 32-bit reciprocal records of div_dv
+// the 32-bit reciprocal records (pc_dv)
 __global__ void dv_kernel(const u32* d, u64 n, u64* dv)
 {
     u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) dv[i] = pc_dv(d[i]);
 }
 
-// odd-number pi table (pi_odd), n records (the last may lie past the pi table: only its
+// odd-number pi table (pi_odd1), n records (the last may lie past the pi table: only its
 // count, pi of the table's limit, is read then): a thread per odd number 2t + 1,
 // a warp per record (blocks of 256 threads keep a record in one warp)
 __global__ void pi_odd_kernel(PiTable pit, u64 n, uint2* out)
