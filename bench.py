@@ -145,7 +145,7 @@ def profile_traffic():
 
 
 # Algorithmic unit costs of the roofline models (stated in the design notes).  The
-# hard-leaf sieve: per crossing one 32-bit shared-memory read-modify-write and about 4
+# hard-leaf sieve: per crossing one shared-memory read-modify-write and about 4
 # integer operations; per (segment, prime) step one 64-bit reduction (about 16 integer
 # operations); per hard leaf one 64-by-32 division (about 16) and a count of the set
 # bits below u: the block prefix plus on average half of a 1024-bit block (16 words:
@@ -155,8 +155,8 @@ HARD_INT = {"crossing": 4.0, "step": 16.0, "leaf": 48.0}
 # Easy leaves: per leaf resolved alone one division by a 32-bit reciprocal (two 32x32-bit
 # products, a shift and a remainder test: 8), the odd-number pi record's index and bit (3),
 # its popcount and sum (3) and the leaf's term (2); per run of clustered leaves, taken by its
-# pi value l, the same: one division by p_l, one lookup, and the run's term from the
-# neighbouring l's lookup (16).  P2: one shared-memory atomic per crossing.
+# pi value l, the same: one division by p_l, one lookup, and the run's term (16).
+# P2: one shared-memory atomic per crossing.
 EASY_INT = {"leaf": 16.0, "run": 16.0}
 P2_SMEM = {"crossing": 1.0}
 
@@ -184,20 +184,22 @@ def ncu_summary(name, sources):
     return rec
 
 
-def hard_roofline(st, sieve_ms, n_sm, f_mhz, traffic):
-    """Both terms of the shared-memory / INT32 model of the hard-leaf sieve:
+def hard_roofline(st, step_ms, sieve_ms, n_sm, f_mhz, traffic):
+    """Both terms of the shared-memory / INT32 model of the hard leaves, over the whole
+    S2_hard step (the sieve, and the leaves with u < p_b^2 that are read from the pi table):
     t_roof = max(bank accesses / (32 N_SM f), integer ops / (128 N_SM f))."""
     clears, leaves, steps = float(st["clears"]), float(st["hard_leaves"]), float(st["steps"])
     f = f_mhz * 1e6
-    smem = roofline_term(HARD_SMEM["crossing"] * clears + HARD_SMEM["leaf"] * leaves, sieve_ms, 32.0 * n_sm * f,
+    smem = roofline_term(HARD_SMEM["crossing"] * clears + HARD_SMEM["leaf"] * leaves, step_ms, 32.0 * n_sm * f,
                          "G smem-bank-accesses/s")
     smem["per_unit"] = "1 per crossing, 17 per hard leaf"
     ints = roofline_term(HARD_INT["crossing"] * clears + HARD_INT["step"] * steps + HARD_INT["leaf"] * leaves,
-                         sieve_ms, 128.0 * n_sm * f, "G int32-ops/s")
+                         step_ms, 128.0 * n_sm * f, "G int32-ops/s")
     ints["per_unit"] = "4 per crossing, 16 per (segment, prime) step, 48 per hard leaf"
     top = smem if smem["frac"] >= ints["frac"] else ints
     out = {"bound": "smem" if top is smem else "alu", "achieved": top["achieved"], "peak": top["peak"],
-           "unit": top["unit"], "frac": top["frac"], "traffic": traffic, "kernel": "hard_sieve_kernel",
+           "unit": top["unit"], "frac": top["frac"], "traffic": traffic,
+           "kernel": "the step: hard_sieve_kernel, and the table leaves", "step_ms": step_ms,
            "kernel_ms": sieve_ms, "terms": {"smem": smem, "int32": ints},
            "peak_basis": "32 banks / 128 INT32 lanes x %d SMs x %.0f MHz (max SM clock, MEASURED_PEAKS.json)"
                          % (n_sm, f_mhz)}
@@ -633,7 +635,7 @@ def main():
             "config": config(int(st["seg_bytes"]), "shards (Section 4 starting values)" if shard else "replicas"),
             "e2e": {"value": job_throughput(z, 1 if shard else world, e2e_s), "unit": UNIT, "h2d_bytes_per_step": 24, "d2h_bytes_per_step": 16},
             "gpu_launches": launches,
-            "roofline": hard_roofline(st, sieve_ms, n_sm, sm_max_mhz, traffic),
+            "roofline": hard_roofline(st, ms_per_step, sieve_ms, n_sm, sm_max_mhz, traffic),
             "clocks": clk.summary(),
             "s2_hard": str(sum_over_ranks(ref, world) if shard else ref),
             "hard_leaves": int(st["hard_leaves"]), "clears": int(st["clears"]),

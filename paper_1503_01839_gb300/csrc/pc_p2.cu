@@ -177,10 +177,10 @@ struct P2Multi {
     unsigned long long items;
 };
 
-// Four resident CTAs per SM (32 registers a thread, a few bytes spilled): the barriers
-// between a segment's phases then leave other CTAs to issue (P2 of pi(10^18) 7.8 ms against
-// 8.4 with three CTAs at 38 registers, 10.4 with two; earlier builds: 27.9 ms with the one
-// CTA the registers allowed when unbounded)
+// Four resident CTAs per SM (32 registers a thread): the barriers between a segment's phases then
+// leave other CTAs to issue (48 KiB segments and the crossings of an earlier build: P2 of pi(10^18)
+// 7.8 ms with four, 8.4 with three at 38 registers, 10.4 with two).  The 64 KiB segments of large z
+// leave room for three; with today's crossings the same P2 takes 5.0 ms.
 template <int NT, bool MULTI>
 __global__ void __launch_bounds__(NT, 4) p2_sieve_kernel(P2Args A0, P2Multi M)
 {
