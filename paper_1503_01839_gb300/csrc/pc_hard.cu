@@ -1453,8 +1453,10 @@ int run_hard_sieve(pc_ctx* ctx, const LeafProblem& P, I128Pair* out)
     A.kleaf = P.c > A.k0 ? P.c : A.k0;
     A.a = P.a;
     A.trunc = P.trunc;
-    A.seg_bytes = pc_seg_bytes(ctx, hard_seg_for(P.z));
-    A.sub_bytes = pc_sub_bytes(ctx, A.seg_bytes, hard_sub_for(P.z));
+    // A shard's bounds, and with them its value, are counted in segments: shards keep 32 KiB
+    // whatever z, so that parts summed from several processes do not hang on the rule by z.
+    A.seg_bytes = pc_seg_bytes(ctx, P.shard_n ? 32768 : hard_seg_for(P.z));
+    A.sub_bytes = pc_sub_bytes(ctx, A.seg_bytes, P.shard_n ? 8192 : hard_sub_for(P.z));
     A.nw = A.seg_bytes / A.sub_bytes;
     A.sub_shift = 3;
     while ((1u << A.sub_shift) < A.sub_bytes * 8) A.sub_shift++;

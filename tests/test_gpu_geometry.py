@@ -20,3 +20,12 @@ def test_default_geometry_at_its_lines(z):
             assert x // y == zz and o.iroot3(x) <= y <= o.isqrt(x)
             assert cx.s2_hard(x, y, 5) == fixed.s2_hard(x, y, 5), zz
             assert cx.p2(x, y) == fixed.p2(x, y), zz
+
+
+@pytest.mark.parametrize("x,y,n", [(1136286593, 11662, 3), (11892848023, 81551, 3), (52247375021686, 1075462, 5)])
+def test_shard_bounds_do_not_follow_the_rule(x, y, n):
+    """Shards are runs of 32 KiB segments at every z."""
+    with pc.Context(0) as cx, pc.Context(0, seg_bytes=32768) as fixed:
+        got = [cx.s2_hard_shard(x, y, 5, k, n) for k in range(n)]
+        assert got == [fixed.s2_hard_shard(x, y, 5, k, n) for k in range(n)]
+        assert sum(got) == cx.s2_hard(x, y, 5)
