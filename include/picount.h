@@ -57,7 +57,8 @@ typedef struct pc_params {
     uint32_t seg_bytes;   /* bytes of shared-memory bitset per sieve segment:
                              1024, 2048, or a multiple of 4096 up to 131072;
                              one byte holds 30 consecutive integers (mod-30
-                             wheel) */
+                             wheel).  Above 65536 the hard-leaf sieve rounds it
+                             down to a multiple of 8192 */
     uint32_t ctas_per_sm; /* resident sieve CTAs per SM (1..4) */
     uint32_t threads;     /* reserved (the sieve uses one warp per warp_bytes) */
     uint32_t alpha;       /* default alpha of pc_pi_count (y = alpha*iroot3(x)) */

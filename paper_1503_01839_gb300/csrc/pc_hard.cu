@@ -1064,6 +1064,26 @@ static u32 pc_sub_bytes(pc_ctx* ctx, u32 seg_bytes, u32 dflt)
     return wb;
 }
 
+// The sieve's geometry from the two defaults.  Above 16 x 4096 bytes only 8192-byte sub-ranges
+// are few enough, so a segment of an odd multiple of 4096 there is rounded down to a multiple
+// of 8192: the sub-ranges have to tile it, or its last bytes belong to no warp.
+static int set_geometry(pc_ctx* ctx, HardArgs& A, u32 seg_dflt, u32 sub_dflt)
+{
+    A.seg_bytes = pc_seg_bytes(ctx, seg_dflt);
+    if (A.seg_bytes > MAX_NW * (MAX_SUB / 2)) A.seg_bytes = A.seg_bytes / MAX_SUB * MAX_SUB;
+    A.sub_bytes = pc_sub_bytes(ctx, A.seg_bytes, sub_dflt);
+    A.nw = A.seg_bytes / A.sub_bytes;
+    if (A.nw * A.sub_bytes != A.seg_bytes) {
+        pc_set_error(ctx, "hard-leaf sieve: sub-ranges of %u bytes do not tile a segment of %u", A.sub_bytes, A.seg_bytes);
+        return PC_EINVAL;
+    }
+    A.sub_shift = 3;
+    while ((1u << A.sub_shift) < A.sub_bytes * 8) A.sub_shift++;
+    A.span = 30ull * A.seg_bytes;
+    A.dspan = 30ull * A.sub_bytes;
+    return PC_OK;
+}
+
 // Work items: segments, heavy ones split into replicas; sorted by estimated
 // cost, heaviest first.  Costs in units of one leaf: one (segment, prime)
 // step of all warps costs about STEP_COST leaves, one crossing-off about
@@ -1455,13 +1475,7 @@ int run_hard_sieve(pc_ctx* ctx, const LeafProblem& P, I128Pair* out)
     A.trunc = P.trunc;
     // A shard's bounds, and with them its value, are counted in segments: shards keep 32 KiB
     // whatever z, so that parts summed from several processes do not hang on the rule by z.
-    A.seg_bytes = pc_seg_bytes(ctx, P.shard_n ? 32768 : hard_seg_for(P.z));
-    A.sub_bytes = pc_sub_bytes(ctx, A.seg_bytes, P.shard_n ? 8192 : hard_sub_for(P.z));
-    A.nw = A.seg_bytes / A.sub_bytes;
-    A.sub_shift = 3;
-    while ((1u << A.sub_shift) < A.sub_bytes * 8) A.sub_shift++;
-    A.span = 30ull * A.seg_bytes;
-    A.dspan = 30ull * A.sub_bytes;
+    PC_TRY(set_geometry(ctx, A, P.shard_n ? 32768 : hard_seg_for(P.z), P.shard_n ? 8192 : hard_sub_for(P.z)));
     A.nseg = P.z / A.span + 1;
     A.s0 = 0;
     A.s1 = A.nseg;
@@ -1661,13 +1675,7 @@ int mq_hard(pc_ctx* ctx, const MQPlan& P)
     HardArgs T{};   // what every query of the batch shares: tables, geometry, queue, counters
     T.k0 = 5;
     T.kleaf = 5;
-    T.seg_bytes = pc_seg_bytes(ctx, ctx->batch_seg ? ctx->batch_seg : 16384);
-    T.sub_bytes = pc_sub_bytes(ctx, T.seg_bytes, 8192);
-    T.nw = T.seg_bytes / T.sub_bytes;
-    T.sub_shift = 3;
-    while ((1u << T.sub_shift) < T.sub_bytes * 8) T.sub_shift++;
-    T.span = 30ull * T.seg_bytes;
-    T.dspan = 30ull * T.sub_bytes;
+    PC_TRY(set_geometry(ctx, T, ctx->batch_seg ? ctx->batch_seg : 16384, 8192));
     T.pit = ctx->T.pi();
     T.rk = ctx->T.rank();
     T.ml = ctx->T.mlist();
