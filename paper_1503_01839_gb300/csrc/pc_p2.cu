@@ -355,10 +355,11 @@ __global__ void __launch_bounds__(NT, 4) p2_sieve_kernel(P2Args A0, P2Multi M)
             const u64 h0 = (plo + 1) / 60, h1 = phi / 60;
             for (u64 h = h0 + tid; h <= h1; h += NT) {
                 u32 v = ((const u16*)&A.pit.rec[h >> 2].bits)[h & 3];
+                if (h == 0) v |= 7u << 16;   // bits 16, 17, 18: the primes 2, 3 and 5 (y < 5)
                 while (v) {
                     const u32 bi = __ffs(v) - 1;
                     v &= v - 1;
-                    const u64 p = 60 * h + 30 * (u64)(bi >> 3) + r8(bi & 7);
+                    const u64 p = bi < 16 ? 60 * h + 30 * (u64)(bi >> 3) + r8(bi & 7) : bi == 18 ? 5 : bi - 14;
                     if (p <= plo || p > phi) continue;
                     // x / p - L is below the segment's length
                     const u32 rel = p2_div(A.x - L * p, (u32)p), q30 = rel / 30;
