@@ -635,6 +635,8 @@ static int run_p2_buckets(pc_ctx* ctx, const P2Args& A, int ctas, size_t smem)
 
 static u32 p2_seg(pc_ctx* ctx, u64 z) { return pc_seg_bytes(ctx, ctx->params.p2_bucket ? 4096 : p2_seg_for(z)); }
 
+// The arguments stay inside the pi table, which reaches the first four (it covers at least 65536):
+// a bucket prime's line beyond it is refused by run_p2, once it is known that P2 has terms.
 int p2_ask(pc_ctx* ctx, u64 x, u64 y, u64* v)
 {
     const u64 z = x / y;
@@ -644,7 +646,7 @@ int p2_ask(pc_ctx* ctx, u64 x, u64 y, u64* v)
     v[n++] = pc_isqrt(z);
     v[n++] = p2_coop_p(seg) - 1;
     v[n++] = p2_big_p(seg);
-    if (ctx->params.p2_bucket) v[n++] = seg;
+    if (ctx->params.p2_bucket) v[n++] = pc_min(seg, ctx->T.pi_limit);
     return n;
 }
 
@@ -677,6 +679,10 @@ int run_p2(pc_ctx* ctx, u64 x, u64 y, u64 a, const u64* pv, I128Pair* out)
     }
     const bool bucket = ctx->params.p2_bucket != 0;
     A.seg_bytes = p2_seg(ctx, z);
+    if (bucket && A.seg_bytes > ctx->T.pi_limit) {
+        pc_set_error(ctx, "pi lookup %u beyond table %llu", A.seg_bytes, (unsigned long long)ctx->T.pi_limit);
+        return PC_EINVAL;
+    }
     A.span = 30ull * A.seg_bytes;
     A.b_mid = (u32)pc_min(pc_max(pv[2] + 1, (u64)A.k0 + 1), B + 1);
     A.b_big = (u32)pc_min(pc_max(pv[3] + 1, (u64)A.b_mid), B + 1);
