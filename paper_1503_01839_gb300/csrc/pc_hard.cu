@@ -574,7 +574,7 @@ __global__ void __launch_bounds__(MAXT, MINB) hard_sieve_kernel(HardArgs A0, Mul
                     const u16* fs = first + 8 * ((lane < avail ? ts : t0) * nw + w);
                     const StepInfo& ss = st[lane < avail ? ts : t0];
                     const u32 p = ss.p;
-                    u32 hm = 0, self = ~0u;
+                    u32 hm = 0, self = ~0u, nx = 0;   // nx: the step's crossings
                     if (lane < avail && bb + ts < Bs) {
                         const uint4 f4 = *(const uint4*)fs;
                         const uint2 c8 = *(const uint2*)ss.cbit;
@@ -587,7 +587,7 @@ __global__ void __launch_bounds__(MAXT, MINB) hard_sieve_kernel(HardArgs A0, Mul
                             for (u32 m = 0; m < (1u << RUN_SHIFT); m++, by += p) {
                                 if (by < sub_bytes) {
                                     hm |= ((myb[by] >> bj) & 1u) << (8 * m + j);
-                                    nclears++;
+                                    nx++;
                                 }
                             }
                         }
@@ -620,6 +620,7 @@ __global__ void __launch_bounds__(MAXT, MINB) hard_sieve_kernel(HardArgs A0, Mul
                     if (!__any_sync(0xffffffffu, n)) {
                         __syncwarp();
                         each_hit(clear_hit);
+                        nclears += nx;
                         if (lane < avail) cw[ts * nw + w] = cnt - hin;
                         cnt -= __shfl_sync(0xffffffffu, hin, 31);
                         __syncwarp();
@@ -637,6 +638,7 @@ __global__ void __launch_bounds__(MAXT, MINB) hard_sieve_kernel(HardArgs A0, Mul
                     const u32 len = enough ? (u32)__ffs(enough) : fits;   // steps t0 .. t0 + len - 1
                     const u32 TL = __shfl_sync(0xffffffffu, incl, len - 1);
                     const u32 loff = incl - n;                             // first leaf of step t0 + lane
+                    if (lane < len) nclears += nx;   // the steps past the run are crossed again in the next one
                     // leaf g of the run: its step i (the last i < len with loff_i <= g) and its
                     // m-list data (nothing for g >= TL)
                     auto run_leaf = [&](u32 g, u32& i, uint4& r) {
