@@ -226,6 +226,17 @@ static int read_slots(pc_ctx* ctx, int n, i128* out)
     return PC_OK;
 }
 
+// The end of a call's enqueued part: after a failure nothing of the call may still run, as the
+// caller may switch streams and the next call takes the same scratch.
+static int drained(pc_ctx* ctx, int rc)
+{
+    if (rc == PC_OK) return rc;
+    for (cudaStream_t s : ctx->side)
+        if (s) cudaStreamSynchronize(s);
+    cudaStreamSynchronize(ctx->stream);
+    return rc;
+}
+
 // p_a by binary search on the pi table (smallest v with pi(v) >= a)
 __global__ void nth_prime_kernel(PiTable pit, u64 a, u64 hi, u64* out)
 {
@@ -357,13 +368,7 @@ static int leaf_parts(pc_ctx* ctx, u64 x, u64 y, u32 c, u64 a, bool want_p2, boo
     ctx->stats.c = c;
     int rc = phases(ctx, P, want_p2 ? pv + 4 : nullptr);
     if (rc == PC_OK) rc = read_slots(ctx, 5, parts);
-    if (rc != PC_OK) {
-        // nothing of this call may still run when the next one takes its scratch
-        for (cudaStream_t s : ctx->side)
-            if (s) cudaStreamSynchronize(s);
-        cudaStreamSynchronize(ctx->stream);
-        return rc;
-    }
+    PC_TRY(drained(ctx, rc));
     float ms = 0;
     double* phase[] = {&ctx->stats.ms_s1, &ctx->stats.ms_easy, &ctx->stats.ms_hard, &ctx->stats.ms_p2};
     for (int i = 0; i < (want_p2 ? 4 : 3); i++)
@@ -435,11 +440,13 @@ static int s2_hard_impl(pc_ctx* ctx, uint64_t x, uint64_t y, uint32_t c, u32 sha
     ctx->stats.c = c;
     I128Pair* d;
     PC_TRY(result_slots(ctx, &d));
+    int rc = PC_OK;
     if (shard_n == 0 || shard_k == 0)
-        PC_TRY(run_hard_smallb(ctx, P, d));   // closed-form leaves (b <= 3): counted once, in shard 0
-    PC_TRY(run_hard_sieve(ctx, P, d));
+        rc = run_hard_smallb(ctx, P, d);   // closed-form leaves (b <= 3): counted once, in shard 0
+    if (rc == PC_OK) rc = run_hard_sieve(ctx, P, d);
     i128 v;
-    PC_TRY(read_slots(ctx, 1, &v));
+    if (rc == PC_OK) rc = read_slots(ctx, 1, &v);
+    PC_TRY(drained(ctx, rc));
     ctx->stats.ms_hard = ph.ms();
     *out = to_pc(v);
     ctx->stats.ms_total = t.ms();
@@ -464,9 +471,10 @@ extern "C" int pc_p2(pc_ctx* ctx, uint64_t x, uint64_t y, uint64_t* out)
     PC_TRY(tables_pi_values(ctx, vals, pv, 1 + p2_ask(ctx, x, y, vals + 1)));
     I128Pair* d;
     PC_TRY(result_slots(ctx, &d));
-    PC_TRY(run_p2(ctx, x, y, pv[0], pv + 1, d));
+    int rc = run_p2(ctx, x, y, pv[0], pv + 1, d);
     i128 v;
-    PC_TRY(read_slots(ctx, 1, &v));
+    if (rc == PC_OK) rc = read_slots(ctx, 1, &v);
+    PC_TRY(drained(ctx, rc));
     if (v < 0 || (v >> 64) != 0) return PC_EOVERFLOW;
     *out = (uint64_t)v;
     ctx->stats.ms_p2 = t.ms();
