@@ -310,10 +310,18 @@ static int timed_phase(pc_ctx* ctx, int e, int k, F&& enqueue)
 // one after the other: pi(1e17) with P2 beside 16.8 ms against 15.4, and the easy leaves beside
 // the sieve, which leaves them no L1, gain nothing either, 67.6 and 62.5 against 61.4 ms at
 // pi(1e18) with a full grid and with two or three CTAs per SM).
+// A whole pass of easy leaves without the odd-number table (the sampled table, or y >= 2^29)
+// takes longer than the sieve beside it, and its CTAs, which stay to the end, then run at half
+// their speed: from EASY_AFTER_Z on it follows the sieve.  With the sampled table, beside and
+// after: pi(1e16) 19.2 (at times 9.5) and 9.6 ms, pi(4e15) 10.8 and 5.7, pi(1e14) 1.04 and 1.07,
+// pi(1e13) 0.53 and 0.78; leaf sums at 1e18, y = 1e9: 1473 and 1298 ms.  A tree cut at p_a <=
+// iroot3(x) has few easy leaves and keeps them beside (phi(1e16, 3000) 2.9 and 3.1 ms).
 static constexpr u64 SIDES_Z = 2000000000ull;
+static constexpr u64 EASY_AFTER_Z = 100000000ull;
 static int phases(pc_ctx* ctx, const LeafProblem& P, const u64* p2_pv)
 {
     const bool sides = P.z < SIDES_Z;
+    const bool easy_beside = sides && (P.z < EASY_AFTER_Z || P.a <= P.E || easy_odd_table(ctx, P));
     I128Pair* d;
     if (sides) PC_TRY(sides_ensure(ctx));
     PC_TRY(result_slots(ctx, &d));
@@ -325,7 +333,7 @@ static int phases(pc_ctx* ctx, const LeafProblem& P, const u64* p2_pv)
     if (p2_pv)
         PC_TRY(timed_phase(ctx, 12, sides ? 1 : -1, [&] { return run_p2(ctx, P.x, P.y, P.a, p2_pv, d + 4); }));
     PC_TRY(timed_phase(ctx, 6, sides ? 0 : -1, [&] { return run_s1_trivial(ctx, P, d + 0, d + 1); }));
-    PC_TRY(timed_phase(ctx, 8, sides ? 0 : -1, [&] { return run_easy(ctx, P, d + 2); }));
+    PC_TRY(timed_phase(ctx, 8, easy_beside ? 0 : -1, [&] { return run_easy(ctx, P, d + 2); }));
     for (int k = 0; sides && k < (p2_pv ? 2 : 1); k++) {
         SideScope side(ctx, k);
         PC_TRY(side.join());

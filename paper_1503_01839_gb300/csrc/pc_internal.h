@@ -240,6 +240,8 @@ int phi_starts(pc_ctx* ctx, u64 m, u32 c, u64 b_max, u64* out);
 
 // Each adds its sum to *out (device I128Pair) -- out must be zeroed first.
 int run_s1_trivial(pc_ctx* ctx, const LeafProblem& P, I128Pair* out_s1, I128Pair* out_trivial);
+// whether the easy leaves read pi(u) from the odd-number table (the fastest way; y < 2^29)
+bool easy_odd_table(const pc_ctx* ctx, const LeafProblem& P);
 int run_easy(pc_ctx* ctx, const LeafProblem& P, I128Pair* out);
 int run_hard_smallb(pc_ctx* ctx, const LeafProblem& P, I128Pair* out);
 int run_hard_sieve(pc_ctx* ctx, const LeafProblem& P, I128Pair* out);

@@ -518,6 +518,11 @@ __global__ void __launch_bounds__(256, 8) easy_kernel(LeafArgs A, u64 b_lo, u64 
     if (threadIdx.x == 0 && v != 0) mq_atomic_add_i128(out, v);
 }
 
+bool easy_odd_table(const pc_ctx* ctx, const LeafProblem& P)
+{
+    return ctx->params.pi_gather != 1 && P.y < PI_ODD_Y && ctx->T.podd_limit >= P.y;
+}
+
 // The leaves of the primes b_lo <= b < b_lo + nb (see easy_range for what, u_lo, u_hi)
 static int leaf_pass(pc_ctx* ctx, const LeafProblem& P, u64 b_lo, u64 nb, u32 what, u64 u_lo, u64 u_hi,
                      I128Pair* out)
@@ -530,7 +535,7 @@ static int leaf_pass(pc_ctx* ctx, const LeafProblem& P, u64 b_lo, u64 nb, u32 wh
     u64* choff = off_buf.as<u64>();
     u32* nch = (u32*)(choff + nb + 1);
     LeafArgs A = make_args(ctx, P);
-    const bool odd = !A.sampled && P.y < PI_ODD_Y && ctx->T.podd_limit >= P.y;
+    const bool odd = easy_odd_table(ctx, P);
     if (odd) A.clust_chunk = 0;   // clustered chunks by pi value
     easy_ranges_kernel<<<(unsigned)((nb + 255) / 256), 256, 0, ctx->stream>>>(A, b_lo, nb, what, u_lo, u_hi, rng, nch);
     PC_LAUNCHED(ctx);
