@@ -1028,8 +1028,7 @@ __global__ void __launch_bounds__(NT) hard_combine_kernel(HardArgs A, I128Pair* 
 // ---------------------------------------------------------------- host
 u32 pc_seg_bytes(pc_ctx* ctx, u32 dflt)
 {
-    u32 sb = ctx->params.seg_bytes ? ctx->params.seg_bytes : ctx->seg_call;
-    if (sb == 0) sb = dflt;
+    u32 sb = ctx->params.seg_bytes ? ctx->params.seg_bytes : dflt;
     if (sb < 1024) sb = 1024;
     if (sb > MAX_SEG) sb = MAX_SEG;
     if (sb > 4096) sb = sb / 4096 * 4096;
@@ -1477,7 +1476,8 @@ int run_hard_sieve(pc_ctx* ctx, const LeafProblem& P, I128Pair* out)
     A.trunc = P.trunc;
     // A shard's bounds, and with them its value, are counted in segments: shards keep 32 KiB
     // whatever z, so that parts summed from several processes do not hang on the rule by z.
-    PC_TRY(set_geometry(ctx, A, P.shard_n ? 32768 : hard_seg_for(P.z), P.shard_n ? 8192 : hard_sub_for(P.z)));
+    const u32 seg = ctx->seg_call ? ctx->seg_call : hard_seg_for(P.z);
+    PC_TRY(set_geometry(ctx, A, P.shard_n ? 32768 : seg, P.shard_n ? 8192 : hard_sub_for(P.z)));
     A.nseg = P.z / A.span + 1;
     A.s0 = 0;
     A.s1 = A.nseg;

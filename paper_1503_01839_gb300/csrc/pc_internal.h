@@ -139,7 +139,7 @@ struct pc_ctx {
     // autotuned alpha and segment bytes per decimal digit count of x (0 = not tuned)
     u32 tuned_alpha[21] = {0};
     u32 tuned_seg[21] = {0};
-    u32 seg_call = 0;   // segment bytes chosen for the running pi(x) call (0 = default)
+    u32 seg_call = 0;   // hard-leaf segment bytes chosen for the running pi(x) call (0 = default)
     u32 tuned_ctas[21] = {0};   // autotuned resident CTAs per SM of the hard-leaf sieve (0 = most)
     u32 ctas_call = 0;          // the value for the running call
     // device counters of the running call (easy leaves, runs, their leaves, P2 crossings, table
@@ -341,7 +341,7 @@ struct SegGeom {
     size_t smem;
 };
 
-// segment bytes: the context's fixed size, else the tuned one of the call, else dflt
+// segment bytes: the context's fixed size, else dflt
 u32 pc_seg_bytes(pc_ctx* ctx, u32 dflt);
 // default segment bytes of the hard-leaf sieve over [0, z]
 u32 hard_seg_for(u64 z);
