@@ -213,11 +213,15 @@ int pc_pi_count_batch(pc_ctx* ctx, const uint64_t* xs, size_t n, uint64_t* out, 
  * built-in one (alpha/2 .. 2 alpha) and hard-leaf segments of 16, 32 and
  * 64 KiB, `reps` timed runs each (0 = 2), and keeps the fastest pair for that
  * decade in ctx; pc_pi_count(x, 0), the batch and the server then use it.
+ * 16 and 32 KiB are limits: the built-in segments, smaller at small z, stay
+ * below them (32 KiB is the built-in choice itself).  P2's segments follow a
+ * rule of their own.
  * A fixed pc_params alpha or seg_bytes is kept fixed.  No result depends on
  * the choice (every candidate's pi is compared; a mismatch is PC_EOVERFLOW).
  * The paper tunes alpha by hand (Section 5, y_max = alpha x^(1/3)). */
 int pc_autotune(pc_ctx* ctx, uint64_t x_lo, uint64_t x_hi, uint32_t reps);
-/* The alpha and segment bytes pc_pi_count(x, 0) uses now. */
+/* The alpha and the hard-leaf segment bytes pc_pi_count(x, 0) uses now (on a tuned
+ * context the tuned size, see above). */
 int pc_tuned(pc_ctx* ctx, uint64_t x, uint32_t* alpha, uint32_t* seg_bytes);
 
 /* Autotuner of the batched schedule (pc_pi_count_batch): its one hard-leaf sieve

@@ -46,6 +46,7 @@ int workers_ensure(pc_ctx* ctx, int n)
         memcpy(w->tuned_alpha, ctx->tuned_alpha, sizeof(ctx->tuned_alpha));
         memcpy(w->tuned_seg, ctx->tuned_seg, sizeof(ctx->tuned_seg));
         memcpy(w->tuned_ctas, ctx->tuned_ctas, sizeof(ctx->tuned_ctas));
+        memcpy(w->tuned_ctas_seg, ctx->tuned_ctas_seg, sizeof(ctx->tuned_ctas_seg));
     }
     return PC_OK;
 }
@@ -640,7 +641,8 @@ extern "C" void pc_server_destroy(pc_server* s)
 // ---------------------------------------------------------------- autotune
 // For every decade of x in [x_lo, x_hi] (x >= 2^20), time pi(x) at a
 // representative x for a few alphas around the built-in choice and a few
-// hard-leaf segment sizes, and keep the fastest pair for that decade.  Every
+// hard-leaf segment sizes, and keep the fastest pair for that decade.  (Sizes up
+// to 32 KiB are limits on those of the rule by z, see run_hard_sieve.)  Every
 // candidate must return the same pi(x); a mismatch is reported as an error.
 extern "C" int pc_autotune(pc_ctx* ctx, uint64_t x_lo, uint64_t x_hi, uint32_t reps)
 {
@@ -698,7 +700,7 @@ extern "C" int pc_autotune(pc_ctx* ctx, uint64_t x_lo, uint64_t x_hi, uint32_t r
         ctx->tuned_alpha[d] = fixed_alpha ? 0 : best_a;
         ctx->tuned_seg[d] = best_s;
         // then the resident CTAs per SM of the hard-leaf sieve at that alpha and segment size
-        ctx->tuned_ctas[d] = 0;
+        ctx->tuned_ctas[d] = ctx->tuned_ctas_seg[d] = 0;
         if (!ctx->params.ctas_per_sm) {
             const u32 ctas[4] = {0, 2, 4, 6};
             double best_c = 1e300;
@@ -730,6 +732,7 @@ extern "C" int pc_autotune(pc_ctx* ctx, uint64_t x_lo, uint64_t x_hi, uint32_t r
                 }
             }
             ctx->tuned_ctas[d] = best_k;
+            ctx->tuned_ctas_seg[d] = ctx->stats.seg_bytes;
         }
     }
     return PC_OK;

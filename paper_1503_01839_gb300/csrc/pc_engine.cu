@@ -505,6 +505,7 @@ int pi_count_impl(pc_ctx* ctx, u64 x, u32 alpha, u64* out)
     if (alpha == 0) alpha = choose_alpha(ctx, x);
     ctx->seg_call = choose_seg(ctx, x);
     ctx->ctas_call = ctx->params.ctas_per_sm ? 0 : ctx->tuned_ctas[decimal_digits(x)];
+    ctx->ctas_seg_call = ctx->tuned_ctas_seg[decimal_digits(x)];
     const u64 r = pc_isqrt(x);
     u64 y = (u64)alpha * pc_iroot3(x);
     if (y > r) y = r;
@@ -521,7 +522,7 @@ int pi_count_impl(pc_ctx* ctx, u64 x, u32 alpha, u64* out)
     u64 a = 0;
     const int rc = leaf_parts(ctx, x, y, c, 0, true, true, parts, &a);
     ctx->seg_call = 0;
-    ctx->ctas_call = 0;
+    ctx->ctas_call = ctx->ctas_seg_call = 0;
     if (rc != PC_OK) return rc;
     i128 pi = parts[0] + parts[1] + parts[2] + parts[3] + (i128)a - 1 - parts[4];
     if (pi < 0 || (pi >> 64) != 0) {

@@ -1049,9 +1049,10 @@ static u32 hard_sub_for(u64 z)
     return z < 120000000ull ? 1024 : z < 280000000ull ? 2048 : z < 2000000000ull ? 4096 : 8192;
 }
 
+static constexpr u32 HARD_SEG_TOP = 32768;
 u32 hard_seg_for(u64 z)
 {
-    return z < 400000ull ? 2048 : z < 120000000ull ? 8192 : z < 2000000000ull ? 16384 : 32768;
+    return z < 400000ull ? 2048 : z < 120000000ull ? 8192 : z < 2000000000ull ? 16384 : HARD_SEG_TOP;
 }
 
 // bytes per warp sub-range: a power of two dividing seg_bytes, at most 16 warps
@@ -1393,7 +1394,8 @@ static int choose_hard_kernel(pc_ctx* ctx, const HardArgs& A, size_t smem, void 
                                        {hard_sieve_kernel<512, 2, MULTI>, 512, 2},
                                        {hard_sieve_kernel<256, 4, MULTI>, 256, 4}};
     const int nt = 32 * (int)A.nw;
-    const int want = (int)(ctx->params.ctas_per_sm ? ctx->params.ctas_per_sm : ctx->ctas_call);
+    const bool other_seg = ctx->ctas_seg_call && ctx->ctas_seg_call != A.seg_bytes;   // tuned at another size
+    const int want = (int)(ctx->params.ctas_per_sm ? ctx->params.ctas_per_sm : other_seg ? 0 : ctx->ctas_call);
     if (!MULTI && ctx->hk.fn && ctx->hk.nt == nt && ctx->hk.smem == smem && ctx->hk.want == want) {
         *out = (void (*)(HardArgs, MultiArgs))ctx->hk.fn;
         *out_per_sm = ctx->hk.per_sm;
@@ -1476,7 +1478,12 @@ int run_hard_sieve(pc_ctx* ctx, const LeafProblem& P, I128Pair* out)
     A.trunc = P.trunc;
     // A shard's bounds, and with them its value, are counted in segments: shards keep 32 KiB
     // whatever z, so that parts summed from several processes do not hang on the rule by z.
-    const u32 seg = ctx->seg_call ? ctx->seg_call : hard_seg_for(P.z);
+    // One tuned size serves a whole decade of x, over which z grows more than fourfold: sizes up to
+    // the rule's largest are limits on the rule's, so that the tuner can keep the rule (32 KiB)
+    // and small z keep their segments (tuned 16 KiB as a limit and as the size itself: pi(7e12)
+    // 0.31 and 0.38 ms, pi(3e11) 0.156 and 0.182).
+    const u32 rule = hard_seg_for(P.z), tuned = ctx->seg_call;
+    const u32 seg = tuned > HARD_SEG_TOP || (tuned && tuned < rule) ? tuned : rule;
     PC_TRY(set_geometry(ctx, A, P.shard_n ? 32768 : seg, P.shard_n ? 8192 : hard_sub_for(P.z)));
     A.nseg = P.z / A.span + 1;
     A.s0 = 0;

@@ -141,7 +141,9 @@ struct pc_ctx {
     u32 tuned_seg[21] = {0};
     u32 seg_call = 0;   // hard-leaf segment bytes chosen for the running pi(x) call (0 = default)
     u32 tuned_ctas[21] = {0};   // autotuned resident CTAs per SM of the hard-leaf sieve (0 = most)
+    u32 tuned_ctas_seg[21] = {0};   // segment bytes they were timed at: for another size they say nothing
     u32 ctas_call = 0;          // the value for the running call
+    u32 ctas_seg_call = 0;      // and its segment bytes (0: any)
     // device counters of the running call (easy leaves, runs, their leaves, P2 crossings, table
     // leaves), beside the result slots; null outside a leaf-sum call
     unsigned long long* dstat = nullptr;

@@ -1,5 +1,5 @@
-"""GPU test of a tuned context: the tuned segment size is the hard-leaf sieve's, and P2 keeps its
-own segments."""
+"""GPU test of a tuned context: the tuned segment size is the hard-leaf sieve's, a limit on the size
+the rule by z takes, and P2 keeps its own segments."""
 import pytest
 
 import paper_1503_01839_gb300 as pc
@@ -25,3 +25,13 @@ def test_p2_keeps_its_segments(tuned, x):
     assert got["y"] == want["y"]
     # P2's sieve starts at a bound of its own segments: the same crossings, the same segments
     assert got["p2_clears"] == want["p2_clears"]
+
+
+@pytest.mark.parametrize("x", XS)
+def test_small_z_keep_the_rule(tuned, x):
+    """A tuned size of 16 or 32 KiB is a limit on the size the rule by z takes."""
+    alpha, seg = tuned.tuned(x)
+    with pc.Context(0) as plain:
+        assert tuned.pi_count(x) == plain.pi_count(x, alpha)
+        rule = plain.stats()["seg_bytes"]
+    assert tuned.stats()["seg_bytes"] == (seg if seg > 32768 else min(seg, rule))
