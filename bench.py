@@ -147,11 +147,13 @@ def profile_traffic():
 # Algorithmic unit costs of the roofline models (stated in the design notes).  The
 # hard-leaf sieve: per crossing one shared-memory read-modify-write and about 4
 # integer operations; per (segment, prime) step one 64-bit reduction (about 16 integer
-# operations); per hard leaf one 64-by-32 division (about 16) and a count of the set
-# bits below u: the block prefix plus on average half of a 1024-bit block (16 words:
-# 16 bank accesses and about 32 integer operations) -> 17 accesses and 48 operations.
-HARD_SMEM = {"crossing": 1.0, "leaf": 17.0}
-HARD_INT = {"crossing": 4.0, "step": 16.0, "leaf": 48.0}
+# operations); per hard leaf that the sieve resolves one 64-by-32 division (about 16) and
+# a count of the set bits below u: the block prefix plus on average half of a 256-bit
+# block (4 words: 4 bank accesses and about 8 integer operations) -> 5 accesses and 24
+# operations; per hard leaf read from the pi table what an easy leaf costs, one quotient
+# and one lookup in global memory: 16 operations, no shared memory.
+HARD_SMEM = {"crossing": 1.0, "leaf": 5.0}
+HARD_INT = {"crossing": 4.0, "step": 16.0, "leaf": 24.0, "table_leaf": 16.0}
 # Easy leaves: per leaf resolved alone one division by a 32-bit reciprocal (two 32x32-bit
 # products, a shift and a remainder test: 8), the odd-number pi record's index and bit (3),
 # its popcount and sum (3) and the leaf's term (2); per run of clustered leaves, taken by its
@@ -188,14 +190,16 @@ def hard_roofline(st, step_ms, sieve_ms, n_sm, f_mhz, traffic):
     """Both terms of the shared-memory / INT32 model of the hard leaves, over the whole
     S2_hard step (the sieve, and the leaves with u < p_b^2 that are read from the pi table):
     t_roof = max(bank accesses / (32 N_SM f), integer ops / (128 N_SM f))."""
-    clears, leaves, steps = float(st["clears"]), float(st["hard_leaves"]), float(st["steps"])
+    clears, steps, table = float(st["clears"]), float(st["steps"]), float(st["table_leaves"])
+    leaves = float(st["hard_leaves"]) - table   # those the sieve resolves
     f = f_mhz * 1e6
     smem = roofline_term(HARD_SMEM["crossing"] * clears + HARD_SMEM["leaf"] * leaves, step_ms, 32.0 * n_sm * f,
                          "G smem-bank-accesses/s")
-    smem["per_unit"] = "1 per crossing, 17 per hard leaf"
-    ints = roofline_term(HARD_INT["crossing"] * clears + HARD_INT["step"] * steps + HARD_INT["leaf"] * leaves,
-                         step_ms, 128.0 * n_sm * f, "G int32-ops/s")
-    ints["per_unit"] = "4 per crossing, 16 per (segment, prime) step, 48 per hard leaf"
+    smem["per_unit"] = "1 per crossing, 5 per hard leaf of the sieve"
+    ints = roofline_term(HARD_INT["crossing"] * clears + HARD_INT["step"] * steps + HARD_INT["leaf"] * leaves +
+                         HARD_INT["table_leaf"] * table, step_ms, 128.0 * n_sm * f, "G int32-ops/s")
+    ints["per_unit"] = ("4 per crossing, 16 per (segment, prime) step, 24 per hard leaf of the sieve, "
+                        "16 per hard leaf read from the pi table")
     top = smem if smem["frac"] >= ints["frac"] else ints
     out = {"bound": "smem" if top is smem else "alu", "achieved": top["achieved"], "peak": top["peak"],
            "unit": top["unit"], "frac": top["frac"], "traffic": traffic,
@@ -600,7 +604,7 @@ def main():
             e1.record(stream)
             assert v == ref
             evs.append((e0, e1))
-            stats.append(ctx.stats())
+            stats.append(dict(ctx.stats(), table_leaves=ctx.table_leaves()))
         torch.cuda.synchronize()
         t_wall = time.perf_counter() - t_wall0
     step_ms = [a.elapsed_time(b) for a, b in evs]
@@ -638,7 +642,8 @@ def main():
             "roofline": hard_roofline(st, ms_per_step, sieve_ms, n_sm, sm_max_mhz, traffic),
             "clocks": clk.summary(),
             "s2_hard": str(sum_over_ranks(ref, world) if shard else ref),
-            "hard_leaves": int(st["hard_leaves"]), "clears": int(st["clears"]),
+            "hard_leaves": int(st["hard_leaves"]), "table_leaves": int(st["table_leaves"]),
+            "clears": int(st["clears"]),
             "hard_leaves_per_s": float(st["hard_leaves"]) / (ms_per_step / 1000.0),
             "segments": int(st["segments"]), "steps_seg_prime": int(st["steps"]),
             "work_items": int(st["work_items"]), "item_steps": int(st["item_steps"]),

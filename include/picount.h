@@ -349,6 +349,10 @@ int pc_tuned_ctas(pc_ctx* ctx, uint64_t x, uint32_t* ctas_per_sm);
 /* Counters of the last successful call. */
 int pc_last_stats(pc_ctx* ctx, pc_stats* out);
 
+/* Those of the last call's hard_leaves that were read from the pi table (u < p_b^2); the sieve
+ * resolved the others.  (Not a field of pc_stats, whose size callers have compiled in.) */
+int pc_table_leaves(pc_ctx* ctx, uint64_t* out);
+
 /* Static description of an error code. */
 const char* pc_strerror(int code);
 

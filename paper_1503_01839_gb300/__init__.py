@@ -21,7 +21,7 @@ SYMBOLS = ["pc_create", "pc_destroy", "pc_set_stream", "pc_pi_count", "pc_phi", 
            "pc_leaf_sums", "pc_pi_count_batch", "pc_last_stats", "pc_strerror", "pc_last_error", "pc_version",
            "pc_p2_noalloc", "pc_server_create", "pc_server_submit", "pc_server_poll", "pc_server_get_stats",
            "pc_server_footprint", "pc_server_destroy", "pc_autotune", "pc_tuned", "pc_s2_hard_shard",
-           "pc_phi_starts", "pc_tuned_ctas", "pc_autotune_batch", "pc_tuned_batch"]
+           "pc_phi_starts", "pc_tuned_ctas", "pc_autotune_batch", "pc_tuned_batch", "pc_table_leaves"]
 
 PC_QUERY_PI = 0
 PC_QUERY_PHI = 1
@@ -105,6 +105,7 @@ def lib():
             L.pc_leaf_sums.argtypes = [p, u64, u64, u32, u64, ctypes.POINTER(PcI128)]
             L.pc_pi_count_batch.argtypes = [p, p, ctypes.c_size_t, p, p]
             L.pc_last_stats.argtypes = [p, ctypes.POINTER(PcStats)]
+            L.pc_table_leaves.argtypes = [p, ctypes.POINTER(u64)]
             L.pc_strerror.argtypes = [ctypes.c_int]
             L.pc_strerror.restype = ctypes.c_char_p
             L.pc_last_error.argtypes = [p]
@@ -132,7 +133,7 @@ def lib():
                          "pc_leaf_sums", "pc_pi_count_batch", "pc_last_stats", "pc_server_create",
                          "pc_server_submit", "pc_server_poll", "pc_server_get_stats", "pc_autotune", "pc_tuned",
                          "pc_s2_hard_shard", "pc_phi_starts", "pc_tuned_ctas", "pc_autotune_batch",
-                         "pc_tuned_batch"):
+                         "pc_tuned_batch", "pc_table_leaves"):
                 getattr(L, name).restype = ctypes.c_int
             _lib = L
     return _lib
@@ -261,6 +262,12 @@ class Context:
         s = PcStats()
         self._check(self._L.pc_last_stats(self._h, ctypes.byref(s)))
         return s.as_dict()
+
+    def table_leaves(self) -> int:
+        """How many of stats()["hard_leaves"] were read from the pi table (u < p_b^2)."""
+        v = ctypes.c_uint64()
+        self._check(self._L.pc_table_leaves(self._h, ctypes.byref(v)))
+        return v.value
 
 
 class Server:

@@ -177,14 +177,14 @@ static int run_queries(pc_ctx* ctx, const std::vector<Query>& q, std::vector<u64
     std::atomic<size_t> next{0};
     std::atomic<int> first_rc{PC_OK};
     std::mutex mu;
-    std::vector<pc_stats> st(W);
+    std::vector<pc_ctx::Stats> st(W);
     auto body = [&](int k) {
         pc_ctx* w = ctx->workers[k];
         if (cudaSetDevice(ctx->device) != cudaSuccess) {
             first_rc = PC_ECUDA;
             return;
         }
-        pc_stats acc{};
+        pc_ctx::Stats acc{};
         for (;;) {
             const size_t i = next.fetch_add(1);
             if (i >= n || first_rc.load() != PC_OK) break;
@@ -202,6 +202,7 @@ static int run_queries(pc_ctx* ctx, const std::vector<Query>& q, std::vector<u64
             out[j] = v;
             acc.kernel_launches += w->stats.kernel_launches;
             acc.hard_leaves += w->stats.hard_leaves;
+            acc.table_leaves += w->stats.table_leaves;
             acc.clears += w->stats.clears;
             acc.steps += w->stats.steps;
             acc.segments += w->stats.segments;
@@ -212,10 +213,11 @@ static int run_queries(pc_ctx* ctx, const std::vector<Query>& q, std::vector<u64
     for (int k = 1; k < W; k++) th.emplace_back(body, k);
     body(0);
     for (auto& t : th) t.join();
-    pc_stats agg{};
-    for (const pc_stats& s : st) {
+    pc_ctx::Stats agg{};
+    for (const pc_ctx::Stats& s : st) {
         agg.kernel_launches += s.kernel_launches;
         agg.hard_leaves += s.hard_leaves;
+        agg.table_leaves += s.table_leaves;
         agg.clears += s.clears;
         agg.steps += s.steps;
         agg.segments += s.segments;
@@ -928,7 +930,7 @@ int phi_starts(pc_ctx* ctx, u64 m, u32 c, u64 b_max, u64* out)
     }
     PC_TRY(build_needs(ctx, N));
     std::vector<u64> qv(q.size(), 0);
-    const pc_stats keep = ctx->stats;   // the queries run on the worker slots; keep the caller's counters
+    const pc_ctx::Stats keep = ctx->stats;   // the queries run on the worker slots; keep the caller's counters
     const int rq = run_queries(ctx, q, qv);
     ctx->stats = keep;
     PC_TRY(rq);

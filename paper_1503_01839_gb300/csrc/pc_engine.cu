@@ -140,6 +140,13 @@ extern "C" int pc_last_stats(pc_ctx* ctx, pc_stats* out)
 }
 
 // ------------------------------------------------------------ helpers
+extern "C" int pc_table_leaves(pc_ctx* ctx, uint64_t* out)
+{
+    if (!ctx || !out) return PC_EINVAL;
+    *out = ctx->stats.table_leaves;
+    return PC_OK;
+}
+
 static void stats_begin(pc_ctx* ctx, u64 x)
 {
     memset(&ctx->stats, 0, sizeof(ctx->stats));
@@ -217,6 +224,7 @@ static int read_slots(pc_ctx* ctx, int n, i128* out)
     ctx->stats.easy_run_leaves += c[2];
     ctx->stats.p2_clears += c[3];
     ctx->stats.hard_leaves += c[4];   // those read from the pi table
+    ctx->stats.table_leaves += c[4];
     float ms = 0;
     if (ctx->hard_timed && cudaEventElapsedTime(&ms, ctx->ev[0], ctx->ev[1]) == cudaSuccess) ctx->stats.ms_hard_sieve += ms;
     if (ctx->easy_timed && cudaEventElapsedTime(&ms, ctx->ev[2], ctx->ev[3]) == cudaSuccess) ctx->stats.ms_easy_kernel += ms;

@@ -126,7 +126,11 @@ struct pc_ctx {
     DevBuf p2_bkt;   // P2 bucket sieve: the buckets of one wave of segments and their fill counts
     // pinned host staging for small results
     void* host_stage = nullptr;
-    pc_stats stats{};
+    // the counters of pc_last_stats, and those with an entry point of their own
+    struct Stats : pc_stats {
+        u64 table_leaves;   // hard leaves read from the pi table (pc_table_leaves)
+    };
+    Stats stats{};
     char errmsg[512] = {0};
     cudaEvent_t ev[16];
     bool ev_ok = false;
