@@ -216,9 +216,13 @@ def hard_roofline(st, step_ms, sieve_ms, n_sm, f_mhz, traffic):
 
 def other_rooflines(sp, n_sm, f_mhz):
     """Rooflines of the easy-leaf kernel (INT32) and the P2 sieve (shared-memory
-    atomics) from one pi(x) call's counters and CUDA-event kernel times."""
+    atomics) from one pi(x) call's counters and CUDA-event kernel times.  Where phases ran
+    beside one another (their times add up to more than the call's), a kernel's time is that
+    of a shared chip and says nothing about its rate: then only the times are given."""
     f = f_mhz * 1e6
     out = {}
+    if sum(sp[k] for k in ("ms_s1", "ms_easy", "ms_hard", "ms_p2")) > sp["ms_total"]:
+        return {"overlapped": True, "easy_kernel_ms": sp["ms_easy_kernel"], "p2_sieve_kernel_ms": sp["ms_p2_kernel"]}
     if sp.get("ms_easy_kernel", 0) > 0:
         work = EASY_INT["leaf"] * sp["easy_leaves"] + EASY_INT["run"] * sp["easy_runs"]
         t = roofline_term(work, sp["ms_easy_kernel"], 128.0 * n_sm * f, "G int32-ops/s")

@@ -116,11 +116,12 @@ typedef struct pc_stats {
                                trivial leaves (one kernel; ms_trivial stays 0).  The phases of a leaf-sum
                                call are timed by CUDA events and may overlap; ms_tables and ms_total
                                on the host. */
-    double ms_hard_sieve;   /* the segmented sieve kernel alone (CUDA events) */
+    double ms_hard_sieve;   /* the segmented sieve kernel's launch (CUDA events); like the phases it may
+                               overlap others, and its time is then that of a shared chip */
     uint64_t warp_steps;      /* (warp sub-range, prime) steps with work in the hard-leaf sieve */
     uint64_t leaf_warp_steps; /* of which resolved leaves */
-    double ms_easy_kernel;    /* the easy-leaf kernel alone (CUDA events) */
-    double ms_p2_kernel;      /* the P2 sieve kernel alone (CUDA events) */
+    double ms_easy_kernel;    /* the easy-leaf kernel's launch (CUDA events), likewise */
+    double ms_p2_kernel;      /* the P2 sieve kernel's launch (CUDA events), likewise */
     uint64_t easy_leaves;     /* easy leaves resolved one at a time */
     uint64_t easy_runs;       /* runs of clustered easy leaves: with the odd-number pi table, the
                                  (b, pi value) pairs taken (one division and one pi lookup each,
