@@ -453,9 +453,14 @@ struct pc_server {
 // to size scratch estimates, never in a count.
 static double pi_upper(double n) { return n < 17 ? 7.0 : 1.26 * n / std::log(n); }
 
-// Device scratch of one query: the hard-leaf count and tally rows (at most
-// segments x pi(isqrt z) u32 pairs), per-segment and per-work-item arrays,
-// the easy-leaf ranges (one per b <= pi(y)) and the P2 segment results.
+// Device scratch of one query, an upper bound: the hard-leaf count and tally rows,
+// per-segment and per-work-item arrays, the easy-leaf ranges and the P2 segment results.
+// Segments are counted at the tuned or largest size of the rule by z, which takes smaller ones
+// at small z, and the rows at pi(isqrt z) a segment; but a segment's rows end at pi(x^(1/4)),
+// half of them or fewer, the easy ranges (60 bytes each) at pi(iroot3 x), far below pi(y), and
+// z below 2e9 has arrays of kilobytes beside the fixed 4 MiB.  What a query reserves, summed up
+// from the sizes that its phases ask for, is at most 0.22 of this for x from 2^20 to 2^63 at
+// every fixed and tuned segment size, alpha from half to twice the built-in one.
 static u64 footprint(const pc_server* s, int kind, u64 x, u64 a)
 {
     const pc_ctx* ctx = s->ctx;

@@ -258,8 +258,8 @@ __device__ __forceinline__ i128 block_sum_i128(i128 v, i128* scratch)
 }
 
 // --------------------------------------------------------------- results
-// Partial sums are written as i128 into per-block slots and summed by
-// reduce_i128_kernel (pc_engine.cu).
+// A part of a result: most kernels add to it by exact 128-bit atomics (mq_atomic_add_i128); the
+// closed-form leaves write per-block slots that reduce_i128_kernel (pc_util.cu) sums.
 struct I128Pair { i64 lo; i64 hi; };
 
 __device__ __forceinline__ void store_i128(I128Pair* p, i128 v)

@@ -218,7 +218,6 @@ static int read_slots(pc_ctx* ctx, int n, i128* out)
     ctx->stats.work_items = hs[4];
     ctx->stats.item_steps += hs[5];
     ctx->stats.presieve_steps += hs[7];
-    if (hs[8]) ctx->stats.steps = hs[8];
     ctx->stats.easy_leaves += c[0];
     ctx->stats.easy_runs += c[1];
     ctx->stats.easy_run_leaves += c[2];

@@ -1086,16 +1086,11 @@ static int set_geometry(pc_ctx* ctx, HardArgs& A, u32 seg_dflt, u32 sub_dflt)
     return PC_OK;
 }
 
-// Work items: segments, heavy ones split into replicas; sorted by estimated
-// cost, heaviest first.  Costs in units of one leaf: one (segment, prime)
-// step of all warps costs about STEP_COST leaves, one crossing-off about
-// CLEAR_COST.  A segment's crossings are estimated by Mertens' theorem,
-// span * 8/30 * sum_{13 <= p <= P} 1/p ~ span * 8/30 * (ln ln P - 1.0056),
-// P = isqrt(x / L), the largest prime the segment sieves with.
-// Work items, planned on the device.  Cost of a segment (arbitrary units): its
-// (segment, prime) steps, its crossings (span * 8/30 * the sum of 1/p over its
-// primes, about ln ln P - ln ln 11 for primes up to P) and its estimated hard
-// leaves.  A segment whose leaves outweigh both its sieve and a fair share of
+// Work items, planned on the device: segments, heavy ones split into replicas.  Cost of a
+// segment (seg_cost, in units of one leaf): 128 for each of its (segment, prime) steps, 0.08
+// for each crossing (by Mertens' theorem span * 8/30 * sum_{13 <= p <= P} 1/p ~
+// span * 8/30 * (ln ln P - 1.0056), P the largest prime the segment sieves with) and its
+// estimated hard leaves.  A segment whose leaves outweigh both its sieve and a fair share of
 // the launch (total / (4 * resident CTAs)) becomes R replicas that share its
 // leaves.  Items are handed out largest first from an atomic counter, ordered
 // by cost in buckets of a quarter octave (the order only balances the load).
@@ -1296,7 +1291,7 @@ __global__ void __launch_bounds__(1024) plan_one_kernel(PlanArgs P)
 
 // Estimated cost of step b of the segment [L, L + span), in the units of seg_cost (one
 // leaf = 1): 128 for the step, 0.08 per crossing, plus its hard leaves (upper bound, as in
-// hard_estimate_kernel).  Integer, so that prefix sums are exact.
+// hard_prep_kernel).  Integer, so that prefix sums are exact.
 __device__ __forceinline__ unsigned long long step_cost(const HardArgs& A, u32 b, u64 L, u64 vL, u64 vLs)
 {
     const u64 p = A.primes[b], vp = A.primes_rcp[b];

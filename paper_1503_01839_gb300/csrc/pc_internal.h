@@ -214,8 +214,8 @@ int tables_pi_values(pc_ctx* ctx, const u64* v, u64* out, int n);
 int tables_pi_many(pc_ctx* ctx, const u64* v, u64* out, size_t n);
 
 // The running call's result buffer, zeroed once per call and read back once at its end: eight
-// I128Pair parts, then (as u64) the call's counters (dstat), the hard-leaf sieve's (HardArgs::stat;
-// [8] = its count rows) and the work queues, each on a line of its own.
+// I128Pair parts, then (as u64) the call's counters (dstat), the hard-leaf sieve's (HardArgs::stat)
+// and the work queues, each on a line of its own.
 static constexpr size_t RES_DSTAT = 128, RES_HARD = 256, RES_QUEUE = 384, RES_BYTES = 768;
 enum { Q_EASY = 0, Q_HARD = 1, Q_P2 = 2, Q_TABLE = 3 };
 inline unsigned long long* call_dstat(pc_ctx* c) { return (unsigned long long*)(c->result.as<unsigned char>() + RES_DSTAT); }
@@ -331,21 +331,11 @@ __device__ __forceinline__ u64 mq_find(const u64* pref, u64 n, u64 v)
     return lo;
 }
 
-int mq_info(pc_ctx* ctx, MQPlan& P);          // fills a, B, K, nlim, E (one read-back for the batch)
+int mq_info(pc_ctx* ctx, MQPlan& P);          // fills a, B, K, nlim, E, R4 (one read-back for the batch)
 int mq_s1_trivial(pc_ctx* ctx, const MQPlan& P);
 int mq_easy(pc_ctx* ctx, const MQPlan& P);
 int mq_hard(pc_ctx* ctx, const MQPlan& P);
 int mq_p2(pc_ctx* ctx, const MQPlan& P);
-
-// segment geometry shared by the sieve kernels
-struct SegGeom {
-    u32 seg_bytes;   // bytes per segment (multiple of 128)
-    u64 span;        // numbers per segment = 30 * seg_bytes
-    u64 nseg;
-    int threads;
-    int ctas;
-    size_t smem;
-};
 
 // segment bytes: the context's fixed size, else dflt
 u32 pc_seg_bytes(pc_ctx* ctx, u32 dflt);

@@ -642,8 +642,8 @@ static LeafArgs table_args(pc_ctx* ctx)
     return make_args(ctx, P);
 }
 
-// per query: pi(y), pi(isqrt z), pi(isqrt x), the m-list entries up to y, pi(iroot3 x);
-// and the ordinary leaf n = 1, phi(x, c), into S1
+// per query: pi(y), pi(isqrt z), pi(isqrt x), the m-list entries up to y, pi(iroot3 x),
+// pi(x^(1/4)); and the ordinary leaf n = 1, phi(x, c), into S1
 __global__ void mq_info_kernel(PiTable pit, RankTable rk, MQ* qs, u32 Q, const u32* phiT, u32 Qc, I128Pair* parts)
 {
     const u32 q = blockIdx.x * blockDim.x + threadIdx.x;
