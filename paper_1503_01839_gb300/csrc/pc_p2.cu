@@ -181,7 +181,9 @@ struct P2Multi {
 // leave other CTAs to issue (48 KiB segments and the crossings of an earlier build: P2 of pi(10^18)
 // 7.8 ms with four, 8.4 with three at 38 registers, 10.4 with two).  The 64 KiB segments of large z
 // leave room for three; with today's crossings the same P2 takes 5.0 ms.
-template <int NT, bool MULTI>
+// TINY: y < 5, the primes 2, 3 and 5 may be terms of the sum too (an instantiation of its own: the
+// test for them in every query costs P2(1e17) 0.3 %).
+template <int NT, bool MULTI, bool TINY>
 __global__ void __launch_bounds__(NT, 4) p2_sieve_kernel(P2Args A0, P2Multi M)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -355,11 +357,12 @@ __global__ void __launch_bounds__(NT, 4) p2_sieve_kernel(P2Args A0, P2Multi M)
             const u64 h0 = (plo + 1) / 60, h1 = phi / 60;
             for (u64 h = h0 + tid; h <= h1; h += NT) {
                 u32 v = ((const u16*)&A.pit.rec[h >> 2].bits)[h & 3];
-                if (h == 0) v |= 7u << 16;   // bits 16, 17, 18: the primes 2, 3 and 5 (y < 5)
+                if (TINY && h == 0) v |= 7u << 16;   // bits 16, 17, 18: the primes 2, 3 and 5
                 while (v) {
                     const u32 bi = __ffs(v) - 1;
                     v &= v - 1;
-                    const u64 p = bi < 16 ? 60 * h + 30 * (u64)(bi >> 3) + r8(bi & 7) : bi == 18 ? 5 : bi - 14;
+                    u64 p = 60 * h + 30 * (u64)(bi >> 3) + r8(bi & 7);
+                    if (TINY && bi >= 16) p = bi == 18 ? 5 : bi - 14;
                     if (p <= plo || p > phi) continue;
                     // x / p - L is below the segment's length
                     const u32 rel = p2_div(A.x - L * p, (u32)p), q30 = rel / 30;
@@ -561,7 +564,7 @@ __global__ void __launch_bounds__(256) p2_bucket_fill_kernel(P2Args A, u64 w0, u
 // The sieve of P2 with bucket primes: waves of W segments, each with its buckets filed
 // first; W from the bound on a bucket's entries and a budget of 2^26 entries (256 MiB), so
 // the buckets' memory does not grow with the number of segments.
-static int run_p2_buckets(pc_ctx* ctx, const P2Args& A, int ctas, size_t smem)
+static int run_p2_buckets(pc_ctx* ctx, const P2Args& A, void (*kern)(P2Args, P2Multi), int ctas, size_t smem)
 {
     PC_TRY(buf_reserve(ctx, ctx->p2_bkt, 256));
     p2_bucket_bound_kernel<<<1, 1024, 0, ctx->stream>>>(A, ctx->p2_bkt.as<unsigned long long>());
@@ -617,8 +620,7 @@ static int run_p2_buckets(pc_ctx* ctx, const P2Args& A, int ctas, size_t smem)
         Aw.bkt = d_bkt;
         Aw.bkt_n = d_n;
         Aw.bkt_cap = (u32)cap;
-        p2_sieve_kernel<512, false><<<(unsigned)pc_min((u64)ctas, (u64)Wc), 512, smem, ctx->stream>>>(Aw,
-                                                                                                     P2Multi{});
+        kern<<<(unsigned)pc_min((u64)ctas, (u64)Wc), 512, smem, ctx->stream>>>(Aw, P2Multi{});
         PC_LAUNCHED(ctx);
         ctx->stats.kernel_launches += 2;
     }
@@ -705,18 +707,21 @@ int run_p2(pc_ctx* ctx, u64 x, u64 y, u64 a, const u64* pv, I128Pair* out)
     const size_t smem = p2_smem(A.seg_bytes, A.b_mid - A.k0 - 1);
     // the kernel's limit is shared by every host thread: set the device maximum (segments of at
     // most MAX_SEG bytes and their block counts fit in it)
+    void (*const kerns[2])(P2Args, P2Multi) = {p2_sieve_kernel<512, false, false>, p2_sieve_kernel<512, false, true>};
     if (!ctx->p2_smem_set) {
-        cudaFuncAttributes fa;
-        PC_CUDA(ctx, cudaFuncGetAttributes(&fa, p2_sieve_kernel<512, false>));
-        const size_t dyn_max = ctx->smem_optin - fa.sharedSizeBytes;
-        cudaError_t e = cudaFuncSetAttribute(p2_sieve_kernel<512, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)dyn_max);
-        if (e != cudaSuccess) {
-            pc_set_error(ctx, "p2 smem attribute: %s", cudaGetErrorString(e));
-            return PC_ECUDA;
+        for (auto k : kerns) {
+            cudaFuncAttributes fa;
+            PC_CUDA(ctx, cudaFuncGetAttributes(&fa, k));
+            const size_t dyn_max = ctx->smem_optin - fa.sharedSizeBytes;
+            cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn_max);
+            if (e != cudaSuccess) {
+                pc_set_error(ctx, "p2 smem attribute: %s", cudaGetErrorString(e));
+                return PC_ECUDA;
+            }
         }
         ctx->p2_smem_set = true;
     }
+    const auto kern = kerns[y < 5];
     int per_sm = (int)(ctx->smem_optin / (smem + 4096));
     if (per_sm < 1) per_sm = 1;
     if (per_sm > 4) per_sm = 4;
@@ -724,10 +729,10 @@ int run_p2(pc_ctx* ctx, u64 x, u64 y, u64 a, const u64* pv, I128Pair* out)
     if ((u64)ctas > A.nseg) ctas = (int)A.nseg;
     A.stat = ctx->dstat;
     if (A.b_bkt <= B) {
-        PC_TRY(run_p2_buckets(ctx, A, ctas, smem));
+        PC_TRY(run_p2_buckets(ctx, A, kern, ctas, smem));
     } else {
         PC_CUDA(ctx, cudaEventRecord(ctx->ev[4], ctx->stream));
-        p2_sieve_kernel<512, false><<<ctas, 512, smem, ctx->stream>>>(A, P2Multi{});
+        kern<<<ctas, 512, smem, ctx->stream>>>(A, P2Multi{});
         PC_LAUNCHED(ctx);
         PC_CUDA(ctx, cudaEventRecord(ctx->ev[5], ctx->stream));
     }
@@ -866,10 +871,10 @@ int mq_p2(pc_ctx* ctx, const MQPlan& P)
     const size_t smem = p2_smem(T.seg_bytes, pv2[0] - T.k0);
     if (S && ctx->mq_mode != MQ_CAPTURE) {   // the shared-memory limit, set outside any capture
         cudaFuncAttributes fa;
-        PC_CUDA(ctx, cudaFuncGetAttributes(&fa, p2_sieve_kernel<512, true>));
+        PC_CUDA(ctx, cudaFuncGetAttributes(&fa, p2_sieve_kernel<512, true, false>));
         const size_t dyn_max = ctx->smem_optin - fa.sharedSizeBytes;
         if (smem > dyn_max) return PC_EINVAL;
-        PC_CUDA(ctx, cudaFuncSetAttribute(p2_sieve_kernel<512, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        PC_CUDA(ctx, cudaFuncSetAttribute(p2_sieve_kernel<512, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           (int)dyn_max));
     }
     if (!mq_device_work(ctx)) return PC_OK;
@@ -881,7 +886,7 @@ int mq_p2(pc_ctx* ctx, const MQPlan& P)
         const u64 ctas = pc_min((u64)ctx->sm_count * per_sm, S);
         T.queue = d_queue;
         T.nseg = 0;
-        p2_sieve_kernel<512, true><<<(unsigned)ctas, 512, smem, st>>>(T, P2Multi{d_qa, d_ipref, Q, S});
+        p2_sieve_kernel<512, true, false><<<(unsigned)ctas, 512, smem, st>>>(T, P2Multi{d_qa, d_ipref, Q, S});
         PC_LAUNCHED(ctx);
     }
     mq_p2_combine_kernel<<<(unsigned)((Q * 32 + 255) / 256), 256, 0, st>>>(d_qa, P.dq, Q, P.parts);
